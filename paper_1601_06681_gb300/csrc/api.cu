@@ -213,7 +213,10 @@ ehdg_status download(Ctx& c, double* dst, const double* src_soa, int64_t outer, 
 
 // Kernels of one step right-hand side: the tensor-core G = P w, if used,
 // before the step kernel.
-int step_launches(const Ctx& c) { return (c.use_ozaki && c.oz_step.img) ? 2 : 1; }
+int step_launches(const Ctx& c) {
+  if (md_active(c)) return c.n_bface > 0 ? 2 : 1;   // the step and its inflow boundary faces
+  return (c.use_ozaki && c.oz_step.img) ? 2 : 1;
+}
 
 // A tensor-core sweep whose bounded mbarrier wait gave up leaves a flag.
 ehdg_status check_tc_err(Ctx& c) {
@@ -227,8 +230,7 @@ ehdg_status check_tc_err(Ctx& c) {
 ehdg_status run_step(Ctx& c, int fixed_iters, int* iters, double* res) {
   CK(counted(c, EHDG_KERNEL_AUX, 1, [&] { return launch_reset_iter(c); }));
   CK(counted(c, EHDG_KERNEL_STEP, step_launches(c), [&] { return launch_step(c); }));
-  CK(counted(c, EHDG_KERNEL_FACE, face_launches(c, kFaceInitial),
-             [&] { return launch_face(c, kFaceInitial); }));
+  CK(counted(c, EHDG_KERNEL_FACE, trace0_launches(c), [&] { return launch_trace0(c); }));
   const int n_it = fixed_iters > 0 ? fixed_iters : c.max_iter;
   bool persist = fixed_iters <= 0 && persistent_sweep_ok(c);
   if (persist) {   // every iteration of the step in one cooperative launch
@@ -327,7 +329,7 @@ ehdg_status capture_step(Ctx& c, cudaStream_t s, cudaStream_t body_stream, bool 
   cudaError_t err = cudaSuccess;
   if ((err = launch_reset_iter(c)) != cudaSuccess) return cuda_fail(err, "capture reset");
   if ((err = launch_step(c)) != cudaSuccess) return cuda_fail(err, "capture step");
-  if ((err = launch_face(c, kFaceInitial)) != cudaSuccess) return cuda_fail(err, "capture face");
+  if ((err = launch_trace0(c)) != cudaSuccess) return cuda_fail(err, "capture face");
   if (allow_persist && persistent_sweep_ok(c)) {
     // every iteration in one cooperative launch: no conditional node needed
     if ((err = launch_sweep_persistent(c)) != cudaSuccess)
@@ -463,7 +465,7 @@ ehdg_status run_graph(Ctx& c, int n_steps, int* iters_per_step, double* res) {
     if (first == EHDG_OK && c.step_status_h[s] != EHDG_OK) first = (ehdg_status)c.step_status_h[s];
   }
   c.launches[EHDG_KERNEL_ELEM] += c.graph_persist ? n_steps : sweeps;
-  c.launches[EHDG_KERNEL_FACE] += (int64_t)n_steps * face_launches(c, kFaceInitial) +
+  c.launches[EHDG_KERNEL_FACE] += (int64_t)n_steps * trace0_launches(c) +
                                    ((c.pde == EHDG_TRANSPORT) ? (c.n_tan > 0 ? sweeps : 0) : sweeps);
   if (c.mixed) {
     c.launches[EHDG_KERNEL_CORR] += (sweeps - n_steps) * c.inner_sweeps * lp_sweep_launches(c);
@@ -1040,6 +1042,7 @@ ehdg_status ehdg_create(const ehdg_mesh_desc* mesh, const ehdg_problem_desc* pro
     // 2D contexts keep the cold start, so that the batched loop's once-per-step
     // kernels (2D only) and solo runs stay equal bit for bit
     c.warm_ok = c.dim == 3 && c.scheme != EHDG_CN && c.n_tan == 0;
+    md_prepare(c);   // hexahedra: the FP64 step in Schur coefficients, where it applies
     if (c.n_tan > 0) {
       TRYC(dalloc(c, &c.tan_g, tg.size()));
       TRYC(dalloc(c, &c.tan_face, tf.size()));

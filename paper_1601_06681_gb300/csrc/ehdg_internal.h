@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <memory>
 #include <string>
 #include <utility>
 #include <vector>
@@ -61,6 +62,10 @@ struct IterState {
   unsigned int bar;              // grid-barrier arrivals of a persistent sweep
   int abort;                     // a persistent sweep's bounded wait gave up
   double r_last;
+};
+
+struct MdTables {   // kernel arguments of sweep_modal.cu
+  virtual ~MdTables() = default;
 };
 
 struct Ctx {
@@ -167,6 +172,9 @@ struct Ctx {
   double* sf_Dy = nullptr;       // [NQFS][NB]
   double sf_s[6] = {0, 0, 0, 0, 0, 0};   // J_f |beta.n| of each local face
   std::vector<int> sf_map;       // [NB][3] faces of each boundary node: f | a_t1 << 4 | a_t2 << 8
+  // the FP64 step of such a problem in Schur coefficients (sweep_modal.cu)
+  std::shared_ptr<const MdTables> md;
+  double* md_trace = nullptr;    // [2][Nqf][nface] trace coefficients, ping-pong pair
   int inner_sweeps = 0;
   int sweep_ft = 4;              // row groups per 32-element tile of k_sweep_fused (2, 4 or 8)
   float* Hy32 = nullptr;         // FP32 copy of Hy in the sweep's slot layout
@@ -229,6 +237,8 @@ cudaError_t launch_face_signs(Ctx& c);
 cudaError_t launch_step(Ctx& c);
 cudaError_t launch_elem(Ctx& c);
 cudaError_t launch_face(Ctx& c, int mode, int graph_mode = 0);   // 0 initial trace, 1 iteration
+cudaError_t launch_trace0(Ctx& c);   // a step's initial trace, where launch_step has not formed it
+int trace0_launches(const Ctx& c);
 cudaError_t launch_final(Ctx& c);
 cudaError_t launch_aos_to_soa(const double* src, double* dst, int64_t outer, int inner,
                               cudaStream_t s);   // src [outer][inner] -> dst [inner][outer]
@@ -247,6 +257,13 @@ bool sf_supported(const Ctx& c);
 ehdg_status sf_prepare(Ctx& c);                           // host tables, before assembly
 cudaError_t launch_sweep_sf(Ctx& c, int graph_mode, int* grid_out);
 cudaError_t launch_final_sf(Ctx& c);
+// its FP64 step in Schur coefficients (sweep_modal.cu): the right-hand side with
+// the initial trace, the sweep, the reconstruction with the end-of-step trace
+bool md_prepare(Ctx& c);
+bool md_active(const Ctx& c);
+cudaError_t launch_step_md(Ctx& c);
+cudaError_t launch_sweep_md(Ctx& c, int graph_mode);
+cudaError_t launch_final_md(Ctx& c);
 // one-thread-per-element 2D transport sweep (sweep_pe.cu)
 bool pe_supported(const Ctx& c);
 cudaError_t launch_sweep_pe(Ctx& c, int graph_mode, int* grid_out);

@@ -483,6 +483,7 @@ static bool step_sf_plan(const Ctx& c, StepParams& s) {
 }
 
 cudaError_t launch_step(Ctx& c) {
+  if (md_active(c)) return launch_step_md(c);
   StepParams s;
   s.nel = c.nel;
   s.n = c.n;
@@ -892,6 +893,12 @@ cudaError_t launch_face(Ctx& c, int mode, int graph_mode) {
   return cudaGetLastError();
 }
 
+int trace0_launches(const Ctx& c) { return md_active(c) ? 0 : face_launches(c, kFaceInitial); }
+
+cudaError_t launch_trace0(Ctx& c) {
+  return md_active(c) ? cudaSuccess : launch_face(c, kFaceInitial);
+}
+
 // ===========================================================================
 // End of step: u^{n+1} = G + H uhat (Crank-Nicolson: 2 v - u^n), trace update
 // ===========================================================================
@@ -933,6 +940,7 @@ __global__ void k_trace_end(int64_t total, int cn, const IterState* it, double* 
 }
 
 cudaError_t launch_final(Ctx& c) {
+  if (md_active(c)) return launch_final_md(c);
   FinalParams p;
   p.nel = c.nel;
   p.nface = c.nface;

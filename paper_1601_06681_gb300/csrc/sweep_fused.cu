@@ -410,6 +410,7 @@ int fused_sweep_grid(const Ctx& c) {
 }
 
 cudaError_t launch_sweep_fused(Ctx& c, int graph_mode) {
+  if (md_active(c)) return launch_sweep_md(c, graph_mode);
   FusedParams p;
   p.nel = c.nel;
   p.nface = c.nface;
