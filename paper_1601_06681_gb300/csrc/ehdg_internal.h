@@ -174,7 +174,8 @@ struct Ctx {
   std::vector<int> sf_map;       // [NB][3] faces of each boundary node: f | a_t1 << 4 | a_t2 << 8
   // the FP64 step of such a problem in Schur coefficients (sweep_modal.cu)
   std::shared_ptr<const MdTables> md;
-  double* md_trace = nullptr;    // [2][Nqf][nface] trace coefficients, ping-pong pair
+  int64_t* md_trace = nullptr;   // [2][Nqf][nface] trace coefficients, ping-pong pair
+  unsigned long long* md_exp = nullptr;   // exponents of the traces' and Gy's rows
   int inner_sweeps = 0;
   int sweep_ft = 4;              // row groups per 32-element tile of k_sweep_fused (2, 4 or 8)
   float* Hy32 = nullptr;         // FP32 copy of Hy in the sweep's slot layout

@@ -19,18 +19,23 @@
 // two columns of Q are rotated so that r vanishes on the last one.
 //
 // Products per element and sweep at p = 3: lifts 336, off-block elimination
-// 240, block inverses 216, outputs 144, residual 96: 1,032 FP64 operations,
-// against 3,552 for the sum-factorised product with the dense
-// Ey A^{-1}[:, bnd] (sweep_sf.cu). Q is orthonormal, so the rounding error
-// stays that of the dense product.
+// 240, block inverses 216, outputs 144: 936, against 3,552 for the
+// sum-factorised product with the dense Ey A^{-1}[:, bnd] (sweep_sf.cu).
 //
-// What bounds it: the FP64 pipe. At 64^3, p = 3 a sweep takes 567 us (1,721 with
-// the sum-factorised product, sweep_sf.cu), 0.94 of the rate that independent
-// FMA chains reach on this part (1.61 per clock and SM). One thread per
-// element keeps all (p+1)^3 unknowns in registers; every coefficient is a
-// kernel parameter with a compile-time index, so an FMA reads it from the
-// constant bank and nothing else competes for the pipe. Memory traffic is the
-// traces and Gy, about 1.2 KB per element at p = 3.
+// The sweep forms them in fixed point on the integer pipe. The FP64 pipe
+// issues 1.6 operations per clock and SM, the integer pipe 57 multiply-adds
+// 32 x 32 + 64 (both measured); three of these make one product of 56-bit
+// numbers held as two limbs. Per element all traces and Gy are aligned to one
+// power of two, chosen from their largest magnitude, with IB = 55 or 56 bits
+// (one or two more than a double's rounding leaves of the largest value), and
+// the coefficients are rounded to 2^-56. Rounding errors of the element's
+// values are then at most a few 2^-56 of its largest trace, where a double
+// accumulation leaves 2^-53 of the partial sums. Traces live in HBM between
+// sweeps as 62-bit integers with one exponent per block of 2 x 2 coefficients.
+// The sums of squares of the residual are exact integers.
+//
+// Measured: see k_sweep_fx. Memory traffic is the traces and Gy, about 1.2 KB
+// per element at p = 3.
 //
 // The API's traces stay values at the face Gauss points and its states nodal
 // values: the step kernel transforms u^n, the end-of-step kernels transform
@@ -64,6 +69,21 @@ struct MdBlocks {
   }
 };
 
+// Trace coefficients and Gy in HBM: 62-bit integers m with one exponent per
+// block of (tangential group) x (tangential group) coefficients, value m 2^e;
+// the exponents of a face's blocks are 16-bit fields of one word. kExpZero: the
+// block is zero; kExpNan: it holds a value that is not finite.
+constexpr int kExpZero = -32768, kExpNan = 32767;
+constexpr int kExpLow = -1200, kExpHigh = 1100;   // outside: zero, not finite
+
+struct FxTraces {
+  int64_t nel, nface;
+  long long* m;                  // [2][P1^2][nface] ping-pong pair
+  unsigned long long* e;         // [2][nface]
+  long long* Gm;                 // [3 P1^2][nel] outflow coefficients of G
+  unsigned long long* Ge;        // [3][nel]
+};
+
 template <int P1>
 struct MdParams {
   int64_t nel, nface;
@@ -73,9 +93,44 @@ struct MdParams {
   double r[P1];
   double T[3][P1][P1];           // c_a T (entries right of the diagonal blocks)
   double inv[MdBlocks<P1>::NINV];
+  FxTraces tr;
+  IterState* it;
+};
+
+// The same tables in fixed point for the sweep, the equation divided by
+// sigma: coefficient c as the limbs of round(c 2^56)
+struct Cfx {
+  int h, l;
+};
+
+// The fixed-point sweep splits an element over warps: along the second and
+// third axes the coefficients go in pairs (groups; at P1 = 3 the first group
+// is a padded single one), one warp per pair of groups. Group 1 of an axis
+// holds the complex pair.
+template <int P1>
+struct FxShape {
+  static constexpr int NG = (P1 + 1) / 2;          // groups per axis
+  static constexpr int OFF = 2 * NG - P1;          // padding before coefficient 0
+  static constexpr int NW = NG * NG;               // warps per element
+  static constexpr int NINV = 16 * MdBlocks<P1>::S2;   // inverse entries per warp
+  // offset of x block I's inverse ((4 s) x (4 s)) in a warp's table
+  __host__ __device__ static constexpr int off(int I) { return 16 * MdBlocks<P1>::pre(I); }
+  __host__ __device__ static constexpr int group(int t) { return (t + OFF) >> 1; }
+};
+
+template <int P1>
+struct FxParams {
+  int64_t nel;
+  const int32_t* elem_face;
+  int fin[3], fout[3];
+  int ib;                        // bits of the element's largest input
   double fw[3];                  // J_f of each axis's faces
-  double* mt;                    // [2][P1^2][nface] trace coefficients, ping-pong pair
-  double* Gy;                    // [3 P1^2][nel] outflow coefficients of G
+  Cfx clx[P1], crx[P1], rx[P1];  // first axis
+  Cfx cl[2][4], cr[2][4], r[4];  // second and third axes, padded index
+  Cfx Tx[P1][P1];                // -c_x T / sigma
+  Cfx T[2][2][2];                // couplings group 1 -> group 0, second and third axes
+  Cfx inv[FxShape<P1>::NW][FxShape<P1>::NINV];
+  FxTraces tr;
   IterState* it;
 };
 
@@ -106,18 +161,157 @@ __device__ __forceinline__ constexpr int md_idx(int a, int i, int t1, int t2) {
                 : (a == 1 ? t1 + P1 * (i + P1 * t2) : t1 + P1 * (t2 + P1 * i));
 }
 
+// --- fixed point ------------------------------------------------------------
+constexpr int kW = 28;                                  // bits of a low limb
+constexpr long long kHalf = 1LL << (kW - 1);
+
+// t = h 2^28 + l with l in [-2^27, 2^27)
+struct Limb {
+  int h, l;
+};
+__device__ __forceinline__ Limb fx_split(long long t) {
+  Limb x;
+  x.h = (int)((t + kHalf) >> kW);
+  x.l = (int)((unsigned)t - ((unsigned)x.h << kW));
+  return x;
+}
+
+__device__ __forceinline__ long long fx_pack(const Limb& x) {
+  return (long long)((unsigned long long)(unsigned)x.h << 32 | (unsigned)x.l);
+}
+__device__ __forceinline__ Limb fx_limb(long long v) {
+  return Limb{(int)(v >> 32), (int)v};
+}
+
+// a += c x. As mad.wide: from the C++ product and sum the compiler made 10
+// instructions of an Acc::mac, from three of these 6.
+__device__ __forceinline__ void fx_mad(long long& a, int c, int x) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(c), "r"(x), "l"(a));
+  a = r;
+}
+
+// a sum of products c x 2^56 as hi 2^56 + mid 2^28 (the products of two low
+// limbs, below a quarter of the last place each, are left out)
+struct Acc {
+  long long hi, mid;
+  __device__ __forceinline__ explicit Acc(long long y) : hi(y), mid(kHalf) {}
+  __device__ __forceinline__ void mac(const Cfx& c, const Limb& x) {
+    fx_mad(hi, c.h, x.h);
+    fx_mad(mid, c.h, x.l);
+    fx_mad(mid, c.l, x.h);
+  }
+  __device__ __forceinline__ long long get() const { return hi + (mid >> kW); }
+};
+
+// the value at byte offset off (below 2^32) of a uniform base
+template <class T>
+__device__ __forceinline__ T& fx_at(T* base, unsigned off) {
+  return *reinterpret_cast<T*>(reinterpret_cast<char*>(base) + off);
+}
+template <class T>
+__device__ __forceinline__ const T& fx_at(const T* base, unsigned off) {
+  return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
+}
+
+// named barriers 1 and 2 of a 128-thread block
+template <int ID>
+__device__ __forceinline__ void bar_sync() {
+  asm volatile("bar.sync %0, 128;" ::"n"(ID) : "memory");
+}
+template <int ID>
+__device__ __forceinline__ void bar_arrive() {
+  asm volatile("bar.arrive %0, 128;" ::"n"(ID) : "memory");
+}
+
+__device__ __forceinline__ int fx_field(unsigned long long e, int b) {
+  return (int)(short)(e >> (16 * b));
+}
+template <int P1>
+__host__ __device__ constexpr int fx_block(int g) {
+  return FxShape<P1>::group(g % P1) + 2 * FxShape<P1>::group(g / P1);
+}
+
+constexpr unsigned long long kExpAllZero = 0x8000800080008000ULL;
+__device__ __forceinline__ unsigned long long fx_set_field(unsigned long long e, int b, int v) {
+  return (e & ~(0xffffULL << (16 * b))) | ((unsigned long long)(unsigned short)v << (16 * b));
+}
+
+// value of a block with exponent e in units of 2^L, rounded
+struct Align {
+  int s;
+  long long half;
+  __device__ __forceinline__ Align(int L, int e) {
+    s = min(63, L - e);
+    half = 1LL << (s - 1);
+  }
+  __device__ __forceinline__ long long operator()(long long m) const { return (m + half) >> s; }
+};
+
+// 2^e as a double, e in [-1022, 1023]
+__device__ __forceinline__ double fx_pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
+
+__device__ __forceinline__ double fx_to_double(long long m, int e) {
+  if (e == kExpNan) return __hiloint2double(0x7ff80000, 0);
+  if (e == kExpZero) return 0.0;
+  if (e > -1000 && e < 900) return (double)m * fx_pow2(e);
+  const int h = e / 2;
+  return (double)m * fx_pow2(h) * fx_pow2(e - h);
+}
+
+// a face's coefficients to 62-bit integers; returns the blocks' exponents
+template <int P1>
+__device__ __forceinline__ unsigned long long fx_face(const double (&x)[P1 * P1],
+                                                      long long (&m)[P1 * P1]) {
+  constexpr int N2 = P1 * P1;
+  unsigned long long ex = kExpAllZero;
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    int emax = 0;
+    bool used = false;
+#pragma unroll
+    for (int g = 0; g < N2; ++g)
+      if (fx_block<P1>(g) == b) {
+        emax = max(emax, (__double2hiint(x[g]) >> 20) & 0x7ff);
+        used = true;
+      }
+    if (!used) continue;
+    const bool fin = emax != 0x7ff;
+    emax = max(emax, 1);
+    long long any = 0;
+#pragma unroll
+    for (int g = 0; g < N2; ++g)
+      if (fx_block<P1>(g) == b) {
+        const long long d = __double_as_longlong(x[g]);
+        const int e = (int)(d >> 52) & 0x7ff;
+        long long v = (d & 0xfffffffffffffLL) | (e ? 1LL << 52 : 0LL);
+        const int s = min(63, emax - max(e, 1));
+        v = ((v << 9) + (s ? 1LL << (s - 1) : 0LL)) >> s;
+        any |= v;
+        const long long sg = d >> 63;
+        m[g] = fin ? (v ^ sg) - sg : 0;
+      }
+    ex = fx_set_field(ex, b, !fin ? kExpNan : (any == 0 ? kExpZero : emax - 1075 - 9));
+  }
+  return ex;
+}
+
 // v = sum_a c_a (l X_in + r X_out)
 template <int P1>
 __device__ __forceinline__ void md_lift(double (&v)[P1 * P1 * P1], const MdParams<P1>& p,
-                                        const double* src, const int (&fi)[3],
-                                        const int (&fo)[3]) {
-  constexpr int RC = MdBlocks<P1>::RC;
+                                        int slot, int64_t e) {
+  constexpr int RC = MdBlocks<P1>::RC, N2 = P1 * P1;
+  const int64_t nface = p.nface;
+  const long long* src = p.tr.m + (int64_t)slot * N2 * nface;
+  const unsigned long long* ee = p.tr.e + (int64_t)slot * nface;
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
+  for (int a = 0; a < 3; ++a) {
+    const int fi = p.elem_face[p.fin[a] * p.nel + e], fo = p.elem_face[p.fout[a] * p.nel + e];
+    const unsigned long long ei = ee[fi], eo = ee[fo];
 #pragma unroll
-    for (int g = 0; g < P1 * P1; ++g) {
-      const double xi = src[g * p.nface + fi[a]];
-      const double xo = src[g * p.nface + fo[a]];
+    for (int g = 0; g < N2; ++g) {
+      const double xi = fx_to_double(src[g * nface + fi], fx_field(ei, fx_block<P1>(g)));
+      const double xo = fx_to_double(src[g * nface + fo], fx_field(eo, fx_block<P1>(g)));
 #pragma unroll
       for (int i = 0; i < P1; ++i) {
         double& t = v[md_idx<P1>(a, i, g % P1, g / P1)];
@@ -125,6 +319,7 @@ __device__ __forceinline__ void md_lift(double (&v)[P1 * P1 * P1], const MdParam
         if (i < RC) t = fma(p.cr[a][i], xo, t);
       }
     }
+  }
 }
 
 // v <- (tau + sum_a c_a T_a)^{-1} v, last block first
@@ -179,6 +374,21 @@ __device__ __forceinline__ double md_out(const double (&v)[P1 * P1 * P1], const 
   return t;
 }
 
+// the outflow coefficients of axis a to dst[g * stride]; returns the blocks' exponents
+template <int P1>
+__device__ __forceinline__ unsigned long long md_store_out(const double (&v)[P1 * P1 * P1],
+                                                           const MdParams<P1>& p, int a,
+                                                           long long* dst, int64_t stride) {
+  double x[P1 * P1];
+  long long m[P1 * P1];
+#pragma unroll
+  for (int g = 0; g < P1 * P1; ++g) x[g] = md_out<P1>(v, p, a, g, 0.0);
+  const unsigned long long ex = fx_face<P1>(x, m);
+#pragma unroll
+  for (int g = 0; g < P1 * P1; ++g) dst[g * stride] = m[g];
+  return ex;
+}
+
 // x <- (m_0 x m_1 x m_2) x, m_a applied along axis a
 template <int P1>
 __device__ __forceinline__ void md_transform(double (&x)[P1 * P1 * P1],
@@ -199,40 +409,291 @@ __device__ __forceinline__ void md_transform(double (&x)[P1 * P1 * P1],
     }
 }
 
-template <int P1>
-// Four blocks per SM at p = 3 (128 registers, a few spilled coefficients): the
-// FP64 pipe then always has another warp's product; two blocks (255 registers)
-// took 624 us per sweep at 64^3, three 577, four 567.
-__global__ void __launch_bounds__(128, P1 == 4 ? 4 : 1) k_sweep_md(const __grid_constant__ MdParams<P1> p,
-                                                  const __grid_constant__ MdResid q) {
-  constexpr int N2 = P1 * P1;
-  const int64_t ne = p.nel, nface = p.nface;
+// The sweep in fixed point: 32 elements per tile. Role (J, K) holds the unknowns
+// of group J of the second and K of the third axis and solves them as dense
+// blocks (4 x the first axis's block) after it has taken the couplings from the
+// higher groups, so (1, 1) goes first, then (0, 1) and (1, 0), then (0, 0); the
+// right-hand sides and the solved values lie in shared memory, which the
+// outflow sums along these axes read too. SOLO: one warp does a tile's roles
+// in turn; otherwise a team of NW warps, one role each.
+//
+// Why roles and rolled loops: one thread per element, straight-line, is 936
+// products instead of 1,140 but 17,200 instructions, more than the instruction
+// caches hold; it took 768 us per sweep at 64^3, p = 3, its warps waiting for
+// instructions. This form runs 15,500 instructions per tile from about 1,000
+// distinct ones: 243 us (1,721 with the sum-factorised FP64 sweep, 567 with
+// this algorithm on the FP64 pipe). 224 MB are read and 79 MB written to DRAM,
+// 1.2 TB/s: the ALU (a mad.wide is a multiply and a 64-bit add) and the latency
+// of the sums at 12 warps per SM bound it.
+template <int P1, bool SOLO>
+__global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 : 4)
+    k_sweep_fx(const __grid_constant__ FxParams<P1> p, const __grid_constant__ MdResid q) {
+  using B = MdBlocks<P1>;
+  using S = FxShape<P1>;
+  constexpr int N2 = P1 * P1, NG = S::NG, OFF = S::OFF, RC = B::RC;
+  // each warp's right-hand sides, then its solved limbs, at [i * 4 + jj + 2 kz];
+  // two buffers (alternate tiles), since other warps read the solved values
+  constexpr bool TEAM = NG > 1 && !SOLO;       // warps of a block share an element
+  __shared__ long long Msh[TEAM ? 2 : 1][S::NW][P1 * 4][32];
+  const int64_t ne = p.nel, nface = p.tr.nface;
+  const int lane = threadIdx.x;
+  // (the reduction makes it a uniform value: coefficients by role come from the
+  // constant bank through uniform registers)
+  const int role0 = (int)__reduce_max_sync(0xffffffffu, (threadIdx.y + blockIdx.x) % S::NW);
   const int kk = p.it->k;                       // read before the last block advances it
-  const double* src = p.mt + (int64_t)(kk & 1) * N2 * nface;
-  double* dst = p.mt + (int64_t)((kk + 1) & 1) * N2 * nface;
+  const long long* src = p.tr.m + (int64_t)(kk & 1) * N2 * nface;
+  long long* dst = p.tr.m + (int64_t)((kk + 1) & 1) * N2 * nface;
+  const unsigned long long* esrc = p.tr.e + (int64_t)(kk & 1) * nface;
+  unsigned long long* edst = p.tr.e + (int64_t)((kk + 1) & 1) * nface;
+  const int64_t ntiles = (ne + 31) / 32;
   double res = 0.0;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    int fi[3], fo[3];
+  int buf = 0;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= TEAM ? 1 : 0) {
+    const bool live = tile * 32 + lane < ne;
+    const int64_t e = live ? tile * 32 + lane : ne - 1;
+    const unsigned e8 = 8u * (unsigned)e;
+    unsigned fi[3], fo[3];                     // byte offsets of the faces' first coefficients
+    unsigned long long ei[3], eo[3], eg[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      fi[a] = p.elem_face[p.fin[a] * ne + e];
-      fo[a] = p.elem_face[p.fout[a] * ne + e];
+      fi[a] = 8u * (unsigned)p.elem_face[p.fin[a] * ne + e];
+      fo[a] = 8u * (unsigned)p.elem_face[p.fout[a] * ne + e];
     }
-    double v[P1 * N2];
-    md_lift<P1>(v, p, src, fi, fo);
-    md_solve<P1>(v, p);
+    unsigned m0 = 0x80008000u, m1 = 0x80008000u;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      double s = 0.0;
+      ei[a] = fx_at(esrc, fi[a]);
+      eo[a] = fx_at(esrc, fo[a]);
+      eg[a] = fx_at(p.tr.Ge + a * ne, e8);
+      m0 = __vmaxs2(__vmaxs2(m0, (unsigned)ei[a]), __vmaxs2((unsigned)eo[a], (unsigned)eg[a]));
+      m1 = __vmaxs2(__vmaxs2(m1, (unsigned)(ei[a] >> 32)),
+                    __vmaxs2((unsigned)(eo[a] >> 32), (unsigned)(eg[a] >> 32)));
+    }
+    m0 = __vmaxs2(m0, m1);
+    const int top = max((int)(short)m0, (int)(short)(m0 >> 16));
+    // values in units of 2^L: the largest has p.ib bits
+    const int L = top + 62 - p.ib;
+
+    double r = 0.0;
+#pragma unroll 1
+    for (int step = 0; step < (SOLO ? S::NW : 1); ++step) {
+    // (one tile's role; the body keeps the outer indentation)
+    const int role = SOLO ? S::NW - 1 - step : role0;
+    const int J = role % NG, K = role / NG;
+    long long(*M)[32] = Msh[buf][role];
+    // lifts
+    {
+      Limb xi[4], xo[4];
+      const int b0 = J + 2 * K;
+      const Align ai(L, fx_field(ei[0], b0)), ao(L, fx_field(eo[0], b0));
 #pragma unroll
-      for (int g = 0; g < N2; ++g) {
-        const double x = md_out<P1>(v, p, a, g, p.Gy[(int64_t)(a * N2 + g) * ne + e]);
-        const double d = x - src[g * nface + fo[a]];
-        dst[g * nface + fo[a]] = x;
-        s = fma(d, d, s);
+      for (int u = 0; u < 4; ++u) {
+        const int j = 2 * J + (u & 1) - OFF, k = 2 * K + (u >> 1) - OFF;
+        const bool ok = OFF == 0 || (j >= 0 && k >= 0);
+        const int64_t g = ok ? j + P1 * k : 0;
+        xi[u] = fx_split(ok ? ai(fx_at(src + g * nface, fi[0])) : 0);
+        xo[u] = fx_split(ok ? ao(fx_at(src + g * nface, fo[0])) : 0);
       }
-      res = fma(p.fw[a], s, res);
+#pragma unroll 1
+      for (int i = 0; i < P1; ++i) {
+        const int by = S::group(i) + 2 * K, bz = S::group(i) + 2 * J;
+        const Align yi(L, fx_field(ei[1], by)), yo(L, fx_field(eo[1], by));
+        const Align zi(L, fx_field(ei[2], bz)), zo(L, fx_field(eo[2], bz));
+        Limb ty[2][2], tz[2][2];                  // [in, out][index in the group]
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int k = 2 * K + u - OFF, j = 2 * J + u - OFF;
+          const bool oky = OFF == 0 || k >= 0, okz = OFF == 0 || j >= 0;
+          const int64_t gy = oky ? i + P1 * k : 0, gz = okz ? i + P1 * j : 0;
+          ty[0][u] = fx_split(oky ? yi(fx_at(src + gy * nface, fi[1])) : 0);
+          ty[1][u] = fx_split(oky ? yo(fx_at(src + gy * nface, fo[1])) : 0);
+          tz[0][u] = fx_split(okz ? zi(fx_at(src + gz * nface, fi[2])) : 0);
+          tz[1][u] = fx_split(okz ? zo(fx_at(src + gz * nface, fo[2])) : 0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int jj = u & 1, kz = u >> 1;
+          Acc t(0);
+          t.mac(p.clx[i], xi[u]);
+          t.mac(p.crx[i], xo[u]);
+          t.mac(p.cl[0][2 * J + jj], ty[0][kz]);
+          t.mac(p.cr[0][2 * J + jj], ty[1][kz]);
+          t.mac(p.cl[1][2 * K + kz], tz[0][jj]);
+          t.mac(p.cr[1][2 * K + kz], tz[1][jj]);
+          M[i * 4 + u][lane] = t.get();
+        }
+      }
+    }
+    // couplings from the warps of higher groups
+    // barrier 1: (1, 1) has published; barrier 2: (0, 1) and (1, 0) have.
+    // Every warp meets both once per tile and waits only for what it reads,
+    // and (1, 1) at the end of its tile for barrier 2, so that no warp comes to
+    // a barrier a second time before its first phase has ended: (1, 1) and, by
+    // barrier 1, the next two need barrier 2 of the tile before, (0, 0) waits
+    // for it itself. The same order lets a buffer be written again two tiles on.
+    if (NG > 1 && !(J && K)) {
+      if (TEAM) {
+        if (J || K) {
+          bar_sync<1>();
+        } else {
+          bar_arrive<1>();
+          bar_sync<2>();
+        }
+      }
+      const long long(*VJ)[32] = Msh[buf][(1 + NG * K) % S::NW];   // (1, K)
+      const long long(*VK)[32] = Msh[buf][(J + NG) % S::NW];       // (J, 1)
+#pragma unroll 1
+      for (int i = 0; i < P1; ++i) {
+        Acc t[4] = {Acc(M[i * 4][lane]), Acc(M[i * 4 + 1][lane]), Acc(M[i * 4 + 2][lane]),
+                    Acc(M[i * 4 + 3][lane])};
+        if (J == 0) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {           // (c, kz)
+            const Limb x = fx_limb(VJ[i * 4 + u][lane]);
+            t[u & 2].mac(p.T[0][0][u & 1], x);
+            t[(u & 2) + 1].mac(p.T[0][1][u & 1], x);
+          }
+        }
+        if (K == 0) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {           // (jj, c)
+            const Limb x = fx_limb(VK[i * 4 + u][lane]);
+            t[u & 1].mac(p.T[1][0][u >> 1], x);
+            t[(u & 1) + 2].mac(p.T[1][1][u >> 1], x);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) M[i * 4 + u][lane] = t[u].get();
+      }
+    }
+    // the blocks along the first axis, last first
+    const Cfx* inv = p.inv[role];
+#pragma unroll
+    for (int I = B::NB - 1; I >= 0; --I) {
+      const int si = B::size(I), m = 4 * si;
+      Limb b[8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        if (x >= m) continue;
+        const int i = I + x / 4;
+        long long y = M[i * 4 + (x & 3)][lane];
+        if (I + si < P1) {
+          Acc t(y);
+#pragma unroll
+          for (int c = 0; c < P1; ++c)
+            if (c >= I + si) t.mac(p.Tx[i][c], fx_limb(M[c * 4 + (x & 3)][lane]));
+          y = t.get();
+        }
+        b[x] = fx_split(y);
+      }
+#pragma unroll 4
+      for (int x = 0; x < m; ++x) {
+        Acc t(0);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          if (c < m) t.mac(inv[S::off(I) + x * m + c], b[c]);
+        M[I * 4 + x][lane] = fx_pack(fx_split(t.get()));
+      }
+    }
+    if (TEAM && (J || K)) {
+      if (J && K) bar_arrive<1>();
+      else bar_arrive<2>();
+    }
+    // outflow coefficients: residual, normalisation, store
+    // sums of squares D = d1 2^30 + d0 per axis
+    long long s11, s10, s00;
+    auto emit = [&](int blk, const long long (&y)[4], const int (&g)[4], const bool (&ok)[4],
+                    unsigned face, unsigned long long ea) {
+      const Align ao(L, fx_field(ea, blk));
+      unsigned long long any = 0;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        if (!ok[t]) continue;
+        const long long d = y[t] - ao(fx_at(src + g[t] * nface, face));
+        const int d1 = (int)((d + (1 << 29)) >> 30);
+        const int d0 = (int)((unsigned)d - ((unsigned)d1 << 30));
+        fx_mad(s11, d1, d1);
+        fx_mad(s10, d1, d0);
+        fx_mad(s00, d0, d0);
+        any |= (unsigned long long)(y[t] ^ (y[t] >> 63));
+      }
+      const int sh = __clzll((long long)any) - 2;
+      int ex = L - sh;
+      if (any == 0 || ex < kExpLow) ex = kExpZero;
+      if (ex > kExpHigh || top == kExpNan) ex = kExpNan;
+      if (live) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+          if (ok[t]) fx_at(dst + g[t] * nface, face) = ex == kExpZero ? 0 : y[t] << (sh & 63);
+        if (NG > 1)
+          reinterpret_cast<short*>(&fx_at(edst, face))[blk] = (short)ex;
+        else
+          fx_at(edst, face) = fx_set_field(kExpAllZero, 0, ex);
+      }
+    };
+    auto fold = [&](int a) {
+      const double s = fma(1073741824.0, fma(1073741824.0, (double)s11, 2.0 * (double)s10),
+                           (double)s00);
+      r = fma(p.fw[a], s, r);
+    };
+    {
+      s11 = s10 = s00 = 0;
+      long long y[4];
+      int g[4];
+      bool ok[4];
+      const int b0 = J + 2 * K;
+      const Align ag(L, fx_field(eg[0], b0));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = 2 * J + (u & 1) - OFF, k = 2 * K + (u >> 1) - OFF;
+        ok[u] = OFF == 0 || (j >= 0 && k >= 0);
+        g[u] = ok[u] ? j + P1 * k : 0;
+        Acc t(ok[u] ? ag(fx_at(p.tr.Gm + g[u] * ne, e8)) : 0);
+#pragma unroll
+        for (int i = 0; i < RC; ++i) t.mac(p.rx[i], fx_limb(M[i * 4 + u][lane]));
+        y[u] = t.get();
+      }
+      emit(b0, y, g, ok, fo[0], eo[0]);
+      fold(0);
+    }
+#pragma unroll 1
+    for (int a = 1; a < 3; ++a) {
+      // axis 2: sums over jj (this warp and (1, K)); axis 3: over kz and (J, 1)
+      if (a == 1 ? J != 0 : K != 0) continue;
+      const int own = a == 1 ? 1 : 2, other = 3 - own;       // strides of summed and kept index
+      const int blk = a == 1 ? K : J;
+      const long long(*V2)[32] = Msh[buf][(a == 1 ? 1 + NG * K : J + NG) % S::NW];
+      const unsigned face = a == 1 ? fo[1] : fo[2];
+      const unsigned long long ea = a == 1 ? eo[1] : eo[2], ga = a == 1 ? eg[1] : eg[2];
+      s11 = s10 = s00 = 0;
+#pragma unroll 1
+      for (int ig = 0; ig < NG; ++ig) {
+        long long y[4];
+        int g[4];
+        bool ok[4];
+        const int b = ig + 2 * blk;
+        const Align ag(L, fx_field(ga, b));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = 2 * ig + (u & 1) - OFF, w = u >> 1, t2 = 2 * blk + w - OFF;
+          ok[u] = OFF == 0 || (i >= 0 && t2 >= 0);
+          g[u] = ok[u] ? i + P1 * t2 : 0;
+          const int at = max(i, 0) * 4 + w * other;
+          Acc t(ok[u] ? ag(fx_at(p.tr.Gm + (a * N2 + g[u]) * ne, e8)) : 0);
+          t.mac(p.r[0], fx_limb(M[at][lane]));
+          t.mac(p.r[1], fx_limb(M[at + own][lane]));
+          if (NG > 1) t.mac(p.r[2], fx_limb(V2[at][lane]));
+          y[u] = t.get();
+        }
+        emit(b, y, g, ok, face, ea);
+      }
+      fold(a);
+    }
+    if (TEAM && J && K) bar_sync<2>();
+    }
+    if (live) {
+      const double sc = fx_pow2(max(-1022, min(1023, L)));
+      res = top == kExpNan ? __hiloint2double(0x7ff80000, 0) : fma(r * sc, sc, res);
     }
   }
   finish_residual(res, q.partials, blockIdx.x, gridDim.x, p.it, q.hist, q.max_iter, q.tol,
@@ -256,8 +717,7 @@ __global__ void __launch_bounds__(128) k_step_md(const __grid_constant__ MdParam
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const int64_t face = p.elem_face[p.fout[a] * ne + e];
-#pragma unroll
-      for (int g = 0; g < N2; ++g) p.mt[g * p.nface + face] = md_out<P1>(v, p, a, g, 0.0);
+      p.tr.e[face] = md_store_out<P1>(v, p, a, p.tr.m + face, p.nface);
     }
     if (!s.have_force) {
 #pragma unroll
@@ -276,9 +736,7 @@ __global__ void __launch_bounds__(128) k_step_md(const __grid_constant__ MdParam
     for (int c = 0; c < N3; ++c) s.G[c * ne + e] = v[c];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int g = 0; g < N2; ++g)
-        p.Gy[(int64_t)(a * N2 + g) * ne + e] = md_out<P1>(v, p, a, g, 0.0);
+      p.tr.Ge[a * ne + e] = md_store_out<P1>(v, p, a, p.tr.Gm + (int64_t)a * N2 * ne + e, ne);
   }
 }
 
@@ -289,17 +747,11 @@ __global__ void __launch_bounds__(128) k_final_md(const __grid_constant__ MdPara
                                                   const __grid_constant__ MdVolume<P1> s) {
   constexpr int N2 = P1 * P1, N3 = P1 * N2;
   const int64_t ne = p.nel;
-  const double* src = p.mt + (int64_t)((p.it->k + 1) & 1) * N2 * p.nface;
+  const int slot = (p.it->k + 1) & 1;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne;
        e += (int64_t)gridDim.x * blockDim.x) {
-    int fi[3], fo[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      fi[a] = p.elem_face[p.fin[a] * ne + e];
-      fo[a] = p.elem_face[p.fout[a] * ne + e];
-    }
     double v[N3];
-    md_lift<P1>(v, p, src, fi, fo);
+    md_lift<P1>(v, p, slot, e);
     md_solve<P1>(v, p);
 #pragma unroll
     for (int c = 0; c < N3; ++c) v[c] += s.G[c * ne + e];
@@ -324,7 +776,7 @@ struct MdFace {
   const int8_t* sgn;
   const double* gb;
   double* gb_old;
-  double* mt;
+  FxTraces tr;
   double* uhat;
   double* uhat_n;
   const IterState* it;
@@ -378,11 +830,15 @@ __global__ void __launch_bounds__(128) k_bnd_md(const __grid_constant__ MdFace<P
     if (ax == 0) md_face_transform<P1>(x, p.C[1], p.C[2]);
     else if (ax == 1) md_face_transform<P1>(x, p.C[0], p.C[2]);
     else md_face_transform<P1>(x, p.C[0], p.C[1]);
+    long long m[N2];
+    const unsigned long long ex = fx_face<P1>(x, m);
 #pragma unroll
     for (int g = 0; g < N2; ++g) {
-      p.mt[g * nface + f] = x[g];
-      p.mt[(int64_t)N2 * nface + g * nface + f] = x[g];
+      p.tr.m[g * nface + f] = m[g];
+      p.tr.m[(N2 + g) * nface + f] = m[g];
     }
+    p.tr.e[f] = ex;
+    p.tr.e[nface + f] = ex;
   }
 }
 
@@ -392,13 +848,15 @@ template <int P1>
 __global__ void __launch_bounds__(128) k_trace_end_md(const __grid_constant__ MdFace<P1> p) {
   constexpr int N2 = P1 * P1;
   const int64_t nface = p.nface;
-  const double* fin = p.mt + (int64_t)(p.it->k & 1) * N2 * nface;
+  const int slot = p.it->k & 1;
+  const long long* fin = p.tr.m + (int64_t)slot * N2 * nface;
   if (p.warm && blockIdx.x == 0 && threadIdx.x == 0) *p.warm = p.it->k >= 1 ? 1 : 0;
   for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < nface;
        f += (int64_t)gridDim.x * blockDim.x) {
     double x[N2];
+    const unsigned long long ex = p.tr.e[slot * nface + f];
 #pragma unroll
-    for (int g = 0; g < N2; ++g) x[g] = fin[g * nface + f];
+    for (int g = 0; g < N2; ++g) x[g] = fx_to_double(fin[g * nface + f], fx_field(ex, fx_block<P1>(g)));
     const int ax = p.face_local[f] >> 1;
     if (ax == 0) md_face_transform<P1>(x, p.V[1], p.V[2]);
     else if (ax == 1) md_face_transform<P1>(x, p.V[0], p.V[2]);
@@ -602,10 +1060,124 @@ bool md_1d(const Ref1D& R, Md1D* o) {
 // reversed where beta_a < 0
 inline int md_node(bool rev, int i, int n) { return rev ? n - 1 - i : i; }
 
+// X = (tau + sum c_a T_a)^{-1} on the index box of sizes s3 at o3 (axis 0 fastest)
+bool md_block_inverse(int n, const Md1D& t, const ld (&ca)[3], ld tau, const int (&s3)[3],
+                      const int (&o3)[3], std::vector<ld>* X) {
+  const int m = s3[0] * s3[1] * s3[2];
+  std::vector<ld> A(m * m, 0.0L);
+  for (int u = 0; u < m; ++u)
+    for (int v = 0; v < m; ++v) {
+      const int iu[3] = {u % s3[0], (u / s3[0]) % s3[1], u / (s3[0] * s3[1])};
+      const int iv[3] = {v % s3[0], (v / s3[0]) % s3[1], v / (s3[0] * s3[1])};
+      ld x = u == v ? tau : 0.0L;
+      for (int a = 0; a < 3; ++a)
+        if (iu[(a + 1) % 3] == iv[(a + 1) % 3] && iu[(a + 2) % 3] == iv[(a + 2) % 3])
+          x += ca[a] * t.T[(o3[a] + iu[a]) * n + o3[a] + iv[a]];
+      A[u * m + v] = x;
+    }
+  return invert(m, A, X);
+}
+
+// Bounds, for traces and Gy of magnitude at most one in every coefficient, of
+// what the fixed-point sweep forms: the right-hand side of each diagonal block
+// (A_bb v_b, split into limbs), the outflow coefficients without Gy, and the
+// largest sum of magnitudes in an accumulator of the lifts and couplings.
+// H = A^{-1} L exactly bounds v; A is upper block triangular.
+void md_bounds(int n, const Md1D& t, const ld (&ca)[3], ld tau, ld sigma, std::vector<double>* rhs,
+               double* out, double* sum) {
+  const int n2 = n * n, N = n * n2, M = 6 * n2;
+  std::vector<double> A((size_t)N * N, 0.0), H((size_t)N * M, 0.0), labs(N, 0.0);
+  auto at = [&](int a, int i, int t1, int t2) {
+    return a == 0 ? i + n * (t1 + n * t2) : (a == 1 ? t1 + n * (i + n * t2) : t1 + n * (t2 + n * i));
+  };
+  for (int a = 0; a < 3; ++a)
+    for (int g = 0; g < n2; ++g)
+      for (int i = 0; i < n; ++i) {
+        const int row = at(a, i, g % n, g / n);
+        H[(size_t)row * M + 2 * a * n2 + g] = (double)(ca[a] * t.l[i] / sigma);
+        H[(size_t)row * M + (2 * a + 1) * n2 + g] = (double)(ca[a] * t.r[i] / sigma);
+        labs[row] += std::fabs((double)(ca[a] * t.l[i] / sigma)) +
+                     std::fabs((double)(ca[a] * t.r[i] / sigma));
+        for (int c = 0; c < n; ++c)
+          A[(size_t)row * N + at(a, c, g % n, g / n)] += (double)(ca[a] * t.T[i * n + c] / sigma);
+      }
+  for (int i = 0; i < N; ++i) A[(size_t)i * N + i] += (double)(tau / sigma);
+  // H <- A^{-1} H: elimination without pivoting is enough here (A's symmetric
+  // part is positive), row by row from the block triangle's structure
+  std::vector<double> U = A;
+  for (int c = 0; c < N; ++c)
+    for (int i = c + 1; i < N; ++i) {
+      const double f = U[(size_t)i * N + c] / U[(size_t)c * N + c];
+      if (f == 0.0) continue;
+      for (int j = c; j < N; ++j) U[(size_t)i * N + j] -= f * U[(size_t)c * N + j];
+      for (int j = 0; j < M; ++j) H[(size_t)i * M + j] -= f * H[(size_t)c * M + j];
+    }
+  for (int i = N - 1; i >= 0; --i) {
+    for (int c = i + 1; c < N; ++c) {
+      const double f = U[(size_t)i * N + c];
+      if (f == 0.0) continue;
+      for (int j = 0; j < M; ++j) H[(size_t)i * M + j] -= f * H[(size_t)c * M + j];
+    }
+    for (int j = 0; j < M; ++j) H[(size_t)i * M + j] /= U[(size_t)i * N + i];
+  }
+  std::vector<double> v(N, 0.0);
+  for (int i = 0; i < N; ++i)
+    for (int j = 0; j < M; ++j) v[i] += std::fabs(H[(size_t)i * M + j]);
+  const int nr = n == 2 ? 2 : (n == 3 ? 1 : 2);
+  auto blk = [&](int i) { return i < nr ? i : nr; };       // first axis
+  auto grp = [&](int i) { return (i + (n & 1)) >> 1; };    // second and third axes
+  auto same = [&](int x, int y) {
+    return blk(x % n) == blk(y % n) && grp((x / n) % n) == grp((y / n) % n) &&
+           grp(x / n2) == grp(y / n2);
+  };
+  *sum = 0.0;
+  for (int i = 0; i < N; ++i) {
+    double s = labs[i];
+    std::vector<double> r(M, 0.0);
+    for (int c = 0; c < N; ++c) {
+      const double f = A[(size_t)i * N + c];
+      if (f == 0.0) continue;
+      if (same(i, c))
+        for (int j = 0; j < M; ++j) r[j] += f * H[(size_t)c * M + j];
+      else
+        s += std::fabs(f) * v[c];
+    }
+    (*rhs)[i] = 0.0;
+    for (int j = 0; j < M; ++j) (*rhs)[i] += std::fabs(r[j]);
+    (*rhs)[i] = std::max((*rhs)[i], v[i]);
+    *sum = std::max(*sum, s);
+  }
+  *out = 0.0;
+  for (int a = 0; a < 3; ++a)
+    for (int g = 0; g < n2; ++g) {
+      double s = 0.0, m = 0.0;
+      for (int j = 0; j < M; ++j) {
+        double x = 0.0;
+        for (int i = 0; i < n; ++i) x += (double)t.r[i] * H[(size_t)at(a, i, g % n, g / n) * M + j];
+        s += std::fabs(x);
+      }
+      for (int i = 0; i < n; ++i) m += std::fabs((double)t.r[i]) * v[at(a, i, g % n, g / n)];
+      *out = std::max(*out, s);
+      *sum = std::max(*sum, m + 1.0);
+    }
+}
+
+FxTraces md_traces(const Ctx& c) {
+  FxTraces t;
+  t.nel = c.nel;
+  t.nface = c.nface;
+  t.m = reinterpret_cast<long long*>(c.md_trace);
+  t.e = c.md_exp;
+  t.Gm = reinterpret_cast<long long*>(c.Gy);
+  t.Ge = c.md_exp + 2 * c.nface;
+  return t;
+}
+
 // a context's kernel arguments, formed once (have_force is set per launch)
 template <int P1>
 struct MdKernelArgs : MdTables {
   MdParams<P1> p;
+  FxParams<P1> x;
   MdVolume<P1> s;
   MdFace<P1> f;
 };
@@ -619,6 +1191,7 @@ template <int P1>
 bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
   using B = MdBlocks<P1>;
   MdParams<P1>* p = &args->p;
+  FxParams<P1>* x = &args->x;
   MdVolume<P1>* s = &args->s;
   MdFace<P1>* f = &args->f;
   const ld tau = c.scheme == EHDG_STEADY ? 0.0L : 1.0L / (ld)c.dt_eff;
@@ -631,7 +1204,9 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
     ld jf = 1.0L;
     for (int d = 0; d < 3; ++d)
       if (d != a) jf *= 0.5L * (ld)c.elem_h[d];
-    p->fw[a] = (double)jf;
+    x->fin[a] = p->fin[a];
+    x->fout[a] = p->fout[a];
+    x->fw[a] = (double)jf;
     for (int i = 0; i < P1; ++i) {
       p->cl[a][i] = (double)(ca[a] * t.l[i]);
       p->cr[a][i] = (double)(ca[a] * t.r[i]);
@@ -639,44 +1214,108 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
       for (int j = 0; j < P1; ++j) {
         p->T[a][i][j] = (double)(ca[a] * t.T[i * P1 + j]);
         // W = Q^T M1 [i][node j], C [i][point j], V [point i][j]
-        ld w = 0.0L, x = 0.0L, y = 0.0L;
+        ld w = 0.0L, cs = 0.0L, y = 0.0L;
         for (int k = 0; k < P1; ++k) {
           w += t.Q[k * P1 + i] * t.M[k * P1 + md_node(rev, j, P1)];
-          x += t.Q[md_node(rev, k, P1) * P1 + i] * (ld)c.r1d.L[j * P1 + k];
+          cs += t.Q[md_node(rev, k, P1) * P1 + i] * (ld)c.r1d.L[j * P1 + k];
           y += (ld)c.r1d.L[i * P1 + k] * t.Q[md_node(rev, k, P1) * P1 + j];
         }
         s->W[a][i][j] = (double)w;
         s->Q[a][i][j] = (double)t.Q[md_node(rev, i, P1) * P1 + j];
-        f->C[a][i][j] = (double)(x * (ld)c.r1d.om[j]);
+        f->C[a][i][j] = (double)(cs * (ld)c.r1d.om[j]);
         f->V[a][i][j] = (double)y;
       }
     }
   }
+  // sigma makes the fixed-point coefficients and values of order one
+  const ld sigma = tau + ca[0] + ca[1] + ca[2];
+  bool fits = sigma > 0.0L;
+  auto fix = [&](ld v) {
+    if (!(std::fabs(v) < 7.9L)) {
+      fits = false;
+      return Cfx{0, 0};
+    }
+    const long long q = (long long)std::floor(std::ldexp(v, 56) + 0.5L);
+    const long long h = (q + kHalf) >> kW;
+    return Cfx{(int)h, (int)(q - (h << kW))};
+  };
+  using S = FxShape<P1>;
+  for (int i = 0; i < 4; ++i) {
+    const int j = i - S::OFF;                         // padded index
+    const bool ok = j >= 0 && j < P1;
+    x->r[i] = ok ? fix(t.r[j]) : Cfx{0, 0};
+    for (int a = 0; a < 2; ++a) {
+      x->cl[a][i] = ok ? fix(ca[1 + a] * t.l[j] / sigma) : Cfx{0, 0};
+      x->cr[a][i] = ok ? fix(ca[1 + a] * t.r[j] / sigma) : Cfx{0, 0};
+      for (int c = 0; c < 2; ++c)
+        if (i < 2)
+          x->T[a][i][c] = ok && S::NG > 1 ? fix(-ca[1 + a] * t.T[j * P1 + 2 + c - S::OFF] / sigma)
+                                          : Cfx{0, 0};
+    }
+  }
+  for (int i = 0; i < P1; ++i) {
+    x->rx[i] = fix(t.r[i]);
+    x->clx[i] = fix(ca[0] * t.l[i] / sigma);
+    x->crx[i] = fix(ca[0] * t.r[i] / sigma);
+    for (int j = 0; j < P1; ++j)
+      x->Tx[i][j] = i < j ? fix(-ca[0] * t.T[i * P1 + j] / sigma) : Cfx{0, 0};
+  }
+  // bounds of the sweep's values for inputs of magnitude one (see md_bounds)
+  const int N3 = P1 * P1 * P1;
+  std::vector<double> rhs_bound(N3, 0.0);
+  double out_bound = 0.0, sum_bound = 0.0;
+  md_bounds(P1, t, ca, tau, sigma, &rhs_bound, &out_bound, &sum_bound);
+  double split_bound = out_bound + 1.0;             // what must fit two limbs
   for (int I = 0; I < B::NB; ++I)
     for (int J = 0; J < B::NB; ++J)
       for (int K = 0; K < B::NB; ++K) {
-        const int si = B::size(I), sj = B::size(J), sk = B::size(K), m = si * sj * sk;
-        std::vector<ld> A(m * m, 0.0L), X;
-        for (int x = 0; x < m; ++x)
-          for (int y = 0; y < m; ++y) {
-            const int xi = x % si, xj = (x / si) % sj, xk = x / (si * sj);
-            const int yi = y % si, yj = (y / si) % sj, yk = y / (si * sj);
-            ld v = 0.0L;
-            if (x == y) v += tau;
-            if (xj == yj && xk == yk) v += ca[0] * t.T[(I + xi) * P1 + I + yi];
-            if (xi == yi && xk == yk) v += ca[1] * t.T[(J + xj) * P1 + J + yj];
-            if (xi == yi && xj == yj) v += ca[2] * t.T[(K + xk) * P1 + K + yk];
-            A[x * m + y] = v;
-          }
-        if (!invert(m, A, &X)) return false;
-        for (int x = 0; x < m * m; ++x) p->inv[B::off(I, J, K) + x] = (double)X[x];
+        // the blocks of the FP64 kernels (the step and the reconstruction)
+        const int s3[3] = {B::size(I), B::size(J), B::size(K)}, o3[3] = {I, J, K};
+        std::vector<ld> X;
+        if (!md_block_inverse(P1, t, ca, tau, s3, o3, &X)) return false;
+        for (size_t u = 0; u < X.size(); ++u) p->inv[B::off(I, J, K) + u] = (double)X[u];
       }
-  p->nel = c.nel;
+  for (int w = 0; w < S::NW; ++w)
+    for (int I = 0; I < B::NB; ++I) {
+      // the fixed-point blocks: x block I times the groups' pairs, padded
+      // entries zero; local order (pair of axis 2, pair of axis 3, x)
+      const int J = w % S::NG, K = w / S::NG;
+      const int j0 = std::max(0, 2 * J - S::OFF), k0 = std::max(0, 2 * K - S::OFF);
+      const int j1 = 2 * J + 2 - S::OFF, k1 = 2 * K + 2 - S::OFF;
+      const int s3[3] = {B::size(I), j1 - j0, k1 - k0}, o3[3] = {I, j0, k0};
+      std::vector<ld> X;
+      if (!md_block_inverse(P1, t, ca, tau, s3, o3, &X)) return false;
+      const int m = 4 * s3[0], mm = s3[0] * s3[1] * s3[2];
+      auto local = [&](int u) {                       // padded (jj, kz, i) -> packed, or -1
+        const int jj = 2 * J + (u & 1) - S::OFF - j0, kz = 2 * K + ((u >> 1) & 1) - S::OFF - k0;
+        return jj < 0 || kz < 0 ? -1 : (u >> 2) + s3[0] * (jj + s3[1] * kz);
+      };
+      for (int u = 0; u < m; ++u) {
+        const int lu = local(u);
+        double asum = 0.0;
+        for (int v = 0; v < m; ++v) {
+          const int lv = local(v);
+          const ld c = lu < 0 || lv < 0 ? 0.0L : X[lu * mm + lv] * sigma;
+          x->inv[w][S::off(I) + u * m + v] = fix(c);
+          if (lv >= 0 && lu >= 0) {
+            const int iv = lv % s3[0], jv = (lv / s3[0]) % s3[1], kv = lv / (s3[0] * s3[1]);
+            asum += std::fabs((double)c) * rhs_bound[(I + iv) + P1 * (j0 + jv + P1 * (k0 + kv))];
+          }
+        }
+        sum_bound = std::max(sum_bound, asum);
+      }
+    }
+  for (double v : rhs_bound) split_bound = std::max(split_bound, v);
+  // a value to be split keeps its high limb in 31 bits, an accumulator (56-bit
+  // coefficients of magnitude below 8, at most 16 terms) below 2^63
+  x->ib = 59 - (int)std::ceil(std::log2(split_bound * 1.001));
+  x->ib = std::min(x->ib, 56);
+  if (!fits || !std::isfinite(split_bound) || x->ib < 54 || !(sum_bound < 64.0)) return false;
+  p->nel = x->nel = c.nel;
   p->nface = c.nface;
-  p->elem_face = c.geo.elem_face;
-  p->mt = c.md_trace;
-  p->Gy = c.Gy;
-  p->it = c.it;
+  p->elem_face = x->elem_face = c.geo.elem_face;
+  p->tr = x->tr = f->tr = md_traces(c);
+  p->it = x->it = c.it;
   s->ucoef = c.scheme == EHDG_STEADY ? 0.0 : 1.0 / c.dt_eff;
   s->have_force = 0;
   s->force_avg = s->cn = f->cn = c.scheme == EHDG_CN ? 1 : 0;
@@ -691,7 +1330,6 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
   f->sgn = c.sgn;
   f->gb = c.gb;
   f->gb_old = c.gb_old;
-  f->mt = c.md_trace;
   f->uhat = c.uhat;
   f->uhat_n = c.uhat_n;
   f->it = c.it;
@@ -730,7 +1368,7 @@ cudaError_t step_t(Ctx& c) {
 
 template <int P1>
 cudaError_t sweep_t(Ctx& c, int graph_mode) {
-  const MdParams<P1>& p = md_args<P1>(c).p;
+  const FxParams<P1>& p = md_args<P1>(c).x;
   MdResid q;
   q.partials = c.partials;
   q.hist = c.hist;
@@ -739,9 +1377,23 @@ cudaError_t sweep_t(Ctx& c, int graph_mode) {
   q.max_iter = c.max_iter;
   q.graph_mode = graph_mode;
   q.handle = c.handle;
-  const int th = md_threads(c.nel);
-  const int grid = std::min(md_grid(k_sweep_md<P1>, th, c.nel), c.n_partials);
-  k_sweep_md<P1><<<grid, th, 0, c.stream>>>(p, q);
+  constexpr int NW = FxShape<P1>::NW;
+  const int64_t ntiles = (c.nel + 31) / 32;
+  // One warp does all groups of its elements where there are tiles enough to
+  // keep 12 warps per SM on full runs: 243 against 265 us at 8,192 tiles (64^3,
+  // p = 3). With fewer the team's shorter tile wins: 93 against 109 us per
+  // iteration at 2,000 tiles, 31 against 45 at 16.
+  if (NW == 1 || ntiles >= 32 * device_sms()) {
+    const int bpsm = fn_blocks_per_sm((const void*)k_sweep_fx<P1, true>, 32, 0);
+    const int grid = (int)std::min<int64_t>(
+        c.n_partials, std::min<int64_t>((int64_t)bpsm * device_sms(), ntiles));
+    k_sweep_fx<P1, true><<<grid, 32, 0, c.stream>>>(p, q);
+  } else {
+    const int bpsm = fn_blocks_per_sm((const void*)k_sweep_fx<P1, false>, 32 * NW, 0);
+    const int grid = (int)std::min<int64_t>(
+        c.n_partials, std::min<int64_t>((int64_t)bpsm * device_sms(), ntiles));
+    k_sweep_fx<P1, false><<<grid, dim3(32, NW), 0, c.stream>>>(p, q);
+  }
   return cudaGetLastError();
 }
 
@@ -771,13 +1423,15 @@ std::shared_ptr<const MdTables> md_make(const Ctx& c, const Md1D& t) {
 
 bool md_prepare(Ctx& c) {
   if (!c.use_sf || c.mixed) return false;
+  // the sweep addresses a face's or an element's coefficient by a 32-bit byte offset
+  if (c.nface >= (1LL << 29) || c.nel >= (1LL << 29)) return false;
   for (int a = 0; a < 3; ++a)
     if (c.beta_const[a] == 0.0) return false;
   Md1D t;
   if (!md_1d(c.r1d, &t)) return false;
-  if (dalloc_raw(c, (void**)&c.md_trace, sizeof(double) * 2 * c.Nqf * c.nface) != cudaSuccess) {
+  if (dalloc_raw(c, (void**)&c.md_trace, sizeof(int64_t) * 2 * c.Nqf * c.nface) != cudaSuccess ||
+      dalloc_raw(c, (void**)&c.md_exp, sizeof(int64_t) * (2 * c.nface + 3 * c.nel)) != cudaSuccess) {
     cudaGetLastError();
-    c.md_trace = nullptr;
     return false;
   }
   c.md = c.p == 1 ? md_make<2>(c, t) : (c.p == 2 ? md_make<3>(c, t) : md_make<4>(c, t));

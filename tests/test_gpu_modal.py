@@ -62,3 +62,72 @@ def test_modal_step_matches_oracle(n, p, signs, scheme, force):
     assert got == iters
     assert rel(u, u_ref) < 1e-12
     assert rel(uh, uh_ref) < 1e-12
+
+
+def _run(n, p, precision, u0, g, **kw):
+    mesh = E.ehdg_mesh_structured(n)
+    with E.Solver(mesh, p, dt=5e-3, tol=1e-11, beta_const=(0.7, -0.4, 0.6), precision=precision,
+                  **kw) as s:
+        s.set_boundary(g(s))
+        s.set_state(u0(s))
+        it = s.run(1)
+        return it, *s.get_state()
+
+
+@pytest.mark.parametrize("n,p", [((55, 54, 53), 2), ((55, 54, 53), 3)])
+def test_one_warp_form_matches_tensor_core_path(n, p):
+    """Meshes large enough for one warp per tile (over 4,864 tiles, the last one
+    ragged), against the tensor-core FP64-accurate path, which shares no kernel
+    with it: 1e-12, the parity bound of both against the oracle."""
+    u0 = lambda s: np.random.default_rng(1).standard_normal(s.state_shape)   # noqa: E731
+    g = lambda s: np.random.default_rng(2).standard_normal(s.trace_shape)    # noqa: E731
+    it_a, u_a, uh_a = _run(n, p, "fp64", u0, g)
+    it_b, u_b, uh_b = _run(n, p, "fp64_emulated", u0, g)
+    assert it_a == it_b
+    assert rel(u_a, u_b) < 1e-12 and rel(uh_a, uh_b) < 1e-12
+
+
+@pytest.mark.parametrize("p", [1, 2, 3])
+def test_fixed_point_scales_exactly(p):
+    """The sweep aligns each element to a power of two, so inputs scaled by a
+    power of two (with the tolerance) give iterates scaled by it, far below and
+    far above one. The step's and the reconstruction's FP64 sums scale exactly
+    too, so equality is bit for bit."""
+    n = (3, 4, 5)
+    mesh = E.ehdg_mesh_structured(n)
+    out = []
+    for k in (0, -140, 90):
+        with E.Solver(mesh, p, dt=1e-2, tol=np.ldexp(1e-11, k), beta_const=(0.7, -0.4, 0.6)) as s:
+            rng = np.random.default_rng(3)
+            s.set_boundary(np.ldexp(rng.standard_normal(s.trace_shape), k))
+            s.set_state(np.ldexp(rng.standard_normal(s.state_shape), k))
+            it = s.run(2)
+            u, uh = s.get_state()
+            out.append((it, np.ldexp(u, -k), np.ldexp(uh, -k)))
+    for it, u, uh in out[1:]:
+        assert it == out[0][0]
+        assert np.array_equal(u, out[0][1]) and np.array_equal(uh, out[0][2])
+
+
+@pytest.mark.parametrize("p", [1, 2, 3])
+def test_zero_and_non_finite_states(p):
+    """A zero state stays exactly zero; a state with a NaN ends as diverged and
+    the context then still solves (a constant state stays constant)."""
+    mesh = E.ehdg_mesh_structured((3, 3, 4))
+    with E.Solver(mesh, p, dt=1e-2, tol=1e-11, beta_const=(0.7, -0.4, 0.6)) as s:
+        s.set_boundary(np.zeros(s.trace_shape))
+        s.set_state(np.zeros(s.state_shape))
+        s.run(1)
+        u, uh = s.get_state()
+        assert not u.any() and not uh.any()
+        bad = np.ones(s.state_shape)
+        bad[5, 0, 0] = np.nan
+        s.set_state(bad)
+        with pytest.raises(E.EhdgError) as err:
+            s.run(1)
+        assert err.value.status == 5
+        s.set_state(np.ones(s.state_shape))
+        s.set_boundary(np.ones(s.trace_shape))
+        s.run(1)
+        u, uh = s.get_state()
+        assert np.abs(u - 1).max() < 1e-12 and np.abs(uh - 1).max() < 1e-12
