@@ -1066,6 +1066,8 @@ ehdg_status ehdg_create(const ehdg_mesh_desc* mesh, const ehdg_problem_desc* pro
       TRYC(dalloc(c, &c.partials, (size_t)((c.nel + 127) / 128)));
       c.n_partials = (int)((c.nel + 127) / 128);
     }
+    CKC(build_pe_operator(c));
+    CKC(cudaStreamSynchronize(c.stream));
     c.use_pe = true;
   }
   if (c.shared_op) {

@@ -54,7 +54,9 @@ struct BInst {
   const double* Gy;
   double* Y;
   float* R_out;
-  const double* Hy;
+  const int2* Hx;               // the sweep rows of Hy in row order, fixed-point limbs
+  const int* hs;
+  int own[2];                   // their local faces
   double* uhat;
   IterState* it;
   double* partials;
@@ -72,10 +74,8 @@ struct BInst {
   float* Y32;
   int* err;
   const uint4* Bimg;            // the rounded operator rows, K-major image (Np x Kp)
-  // the sweep rows of the operator in row order, for the persistent form
-  // (read through L1 instead of staged per item): [n_rows][NQFS] FP64 and,
-  // with FP32 corrections, [n_up][NQFS] FP32
-  const double* Hyc;
+  // the FP32 sweep rows of the operator in row order, [n_up][NQFS], for the
+  // persistent form (read through L1, like Hx, instead of staged per item)
   const float* Hy32c;
   const int* rowfg;             // [Np] face | point << 8 of each row
   // fixed-shape tile body (quadrilaterals, whole faces as rows): row faces,
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kPeTile) k_batch_sweep(const BInst* inst, cons
   const int* pre = lv.pre_sw(lists);
   const int n_items = n_act > 0 ? pre[n_act] : 0;
   int cur = -1;
-  double* Hsh = sm;                                   // the instance's sweep rows [n_rows][NQ]
+  int2* Hsh = reinterpret_cast<int2*>(sm);            // the instance's sweep rows [n_rows][NQ]
   for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
     // every listed instance iterates; its state cannot change before all its
     // work items are done
@@ -243,10 +243,7 @@ __global__ void __launch_bounds__(kPeTile) k_batch_sweep(const BInst* inst, cons
     const BInst& I = inst[idx];
     const int nq = I.NQFS;
     if (idx != cur) {   // the previous item's threads are past its last barrier
-      for (int i = tid; i < I.n_rows * nq; i += kPeTile) {
-        const int j = i / nq, c = i - j * nq;
-        Hsh[i] = I.Hy[I.rows[j] * nq + c];
-      }
+      for (int i = tid; i < I.n_rows * nq; i += kPeTile) Hsh[i] = I.Hx[i];
       __syncthreads();
       cur = idx;
     }
@@ -255,14 +252,13 @@ __global__ void __launch_bounds__(kPeTile) k_batch_sweep(const BInst* inst, cons
     PeView v = {};
     v.nel = I.nel;
     v.nface = I.nface;
-    v.n_rows = I.n_rows;
-    v.n_up = I.n_up;
-    v.rows = I.rows;
+    v.own[0] = I.own[0];
+    v.own[1] = I.own[1];
+    v.hs = I.hs;
     v.elem_face = I.elem_face;
     v.face_jf = I.face_jf;
     v.fw = I.fw;
     v.Gy = I.Gy;
-    v.Y = I.Y;
     v.R_out = I.R_out;
     v.partials = I.partials;
     v.it = I.it;
@@ -594,14 +590,11 @@ __global__ void __launch_bounds__(kBTcThreads) k_batch_tc(const BInst* inst, con
                  "r"(ncols));
 }
 
-// Setup of the persistent form: instance i's sweep rows in row order
-__global__ void k_batch_rows(const double* Hy, const float* Hy32, const int* rows, int n_rows,
-                             int n_up, int NQFS, double* Hyc, float* Hy32c) {
-  for (int t = threadIdx.x; t < n_rows * NQFS; t += blockDim.x) {
-    const int j = t / NQFS, c = t - j * NQFS;
-    Hyc[t] = Hy[rows[j] * NQFS + c];
-    if (Hy32c && j < n_up) Hy32c[t] = Hy32[rows[j] * NQFS + c];
-  }
+// Setup of the persistent form: instance i's FP32 sweep rows in row order
+__global__ void k_batch_rows(const float* Hy32, const int* rows, int n_up, int NQFS,
+                             float* Hy32c) {
+  for (int t = threadIdx.x; t < n_up * NQFS; t += blockDim.x)
+    Hy32c[t] = Hy32[rows[t / NQFS] * NQFS + t % NQFS];
 }
 
 // Setup: instance i's operator rows rounded to TF32 / BF16 in the K-major
@@ -654,8 +647,8 @@ __global__ void __launch_bounds__(kPeTile) k_batch_lp(const BInst* inst, const i
     LpPeView v;
     v.nel = I.nel;
     v.nface = I.nface;
-    v.n_up = I.n_up;
-    v.rows = I.rows;
+    v.own[0] = I.own[0];
+    v.own[1] = I.own[1];
     v.elem_face = I.elem_face;
     v.R = I.R32;
     v.in = j == 0 ? I.R32 : I.d32 + (int64_t)((j - 1) & 1) * trace;
@@ -792,18 +785,17 @@ __global__ void k_batch_qinit(const BInst* inst, int n_inst, BQueue* q, long lon
 }
 
 template <int NQ>
-__device__ __forceinline__ bool q_sweep_item(const BInst& I, const double* Hsh, int64_t tile) {
+__device__ __forceinline__ bool q_sweep_item(const BInst& I, const int2* Hsh, int64_t tile) {
   PeView v = {};
   v.nel = I.nel;
   v.nface = I.nface;
-  v.n_rows = I.n_rows;
-  v.n_up = I.n_up;
-  v.rows = I.rows;
+  v.own[0] = I.own[0];
+  v.own[1] = I.own[1];
+  v.hs = I.hs;
   v.elem_face = I.elem_face;
   v.face_jf = I.face_jf;
   v.fw = I.fw;
   v.Gy = I.Gy;
-  v.Y = I.Y;
   v.R_out = I.R_out;
   v.partials = I.partials;
   v.it = I.it;
@@ -826,8 +818,8 @@ __device__ __forceinline__ void q_corr_item(const BInst& I, const float* Hsh32, 
   LpPeView v;
   v.nel = I.nel;
   v.nface = I.nface;
-  v.n_up = I.n_up;
-  v.rows = I.rows;
+  v.own[0] = I.own[0];
+  v.own[1] = I.own[1];
   v.elem_face = I.elem_face;
   v.R = I.R32;
   v.in = j == 0 ? I.R32 : I.d32 + (int64_t)((j - 1) & 1) * trace;
@@ -883,7 +875,7 @@ __global__ void __launch_bounds__(kPeTile, 5) k_batch_persist(const BInst* inst,
     // instances
     bool done;
     if (kind == 0) {
-      const double* hr = I.Hyc;
+      const int2* hr = I.Hx;
       switch (nq) {
         case 8: done = q_sweep_item<8>(I, hr, idx); break;
         case 12: done = q_sweep_item<12>(I, hr, idx); break;
@@ -1257,7 +1249,10 @@ cudaError_t BatchLoop::build(const std::vector<Ctx*>& ctxs, unsigned long long* 
     I.Gy = c.Gy;
     I.Y = c.Y;
     I.R_out = c.mixed ? c.R32 : nullptr;
-    I.Hy = c.Hy;
+    I.Hx = reinterpret_cast<const int2*>(c.pe_hx);
+    I.hs = c.pe_hs;
+    I.own[0] = c.rows_host[0] / c.Nqf;
+    I.own[1] = c.rows_host[c.Nqf] / c.Nqf;
     I.uhat = c.uhat;
     I.it = c.it;
     I.partials = c.partials;
@@ -1372,24 +1367,20 @@ cudaError_t BatchLoop::build(const std::vector<Ctx*>& ctxs, unsigned long long* 
   const bool persist_fits =
       batch_persist_fits(std::vector<const Ctx*>(ctxs.begin(), ctxs.end()));
   if (!L.any_mma && persist_fits) {
-    // the persistent form reads every instance's sweep rows in row order
-    std::vector<size_t> off(L.n_inst, 0), off32(L.n_inst, 0);
+    // the persistent form reads every instance's FP32 sweep rows in row order
+    std::vector<size_t> off32(L.n_inst, 0);
     size_t bytes = 0;
     for (int i = 0; i < L.n_inst; ++i) {
-      off[i] = bytes;
-      bytes += (sizeof(double) * h[i].n_rows * h[i].NQFS + 255) / 256 * 256;
       off32[i] = bytes;
-      if (h[i].tc) bytes += (sizeof(float) * h[i].n_rows * h[i].NQFS + 255) / 256 * 256;
+      if (h[i].tc) bytes += (sizeof(float) * h[i].n_up * h[i].NQFS + 255) / 256 * 256;
     }
     if ((e = cudaMalloc(&L.d_rows, std::max<size_t>(bytes, 256))) != cudaSuccess) return e;
     for (int i = 0; i < L.n_inst; ++i) {
+      if (!h[i].tc) continue;
       const Ctx& c = *ctxs[i];
-      double* hyc = reinterpret_cast<double*>(L.d_rows + off[i]);
-      float* hy32c = h[i].tc ? reinterpret_cast<float*>(L.d_rows + off32[i]) : nullptr;
-      k_batch_rows<<<1, 256>>>(c.Hy, h[i].tc ? c.Hy32 : nullptr, c.rows, c.n_rows, h[i].n_up,
-                               c.NQFS, hyc, hy32c);
+      float* hy32c = reinterpret_cast<float*>(L.d_rows + off32[i]);
+      k_batch_rows<<<1, 256>>>(c.Hy32, c.rows, h[i].n_up, c.NQFS, hy32c);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      h[i].Hyc = hyc;
       h[i].Hy32c = hy32c;
     }
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;

@@ -165,6 +165,8 @@ struct Ctx {
   // face-point rows and Ab = A^{-1}[:, bnd] the volume values
   bool use_pe = false;           // 2D shared-operator FP64 sweep, one thread per element
   double* pe_fw = nullptr;       // its face Gauss weights [Nqf]
+  void* pe_hx = nullptr;         // [n_rows][NQFS] its rows of Hy as fixed-point limbs (int2)
+  int* pe_hs = nullptr;          // [1] their scale
   bool use_sf = false;
   int sf_NB = 0;                 // boundary nodes per element
   int* sf_bnd = nullptr;         // [NB] their node indices
@@ -267,6 +269,7 @@ cudaError_t launch_sweep_md(Ctx& c, int graph_mode);
 cudaError_t launch_final_md(Ctx& c);
 // one-thread-per-element 2D transport sweep (sweep_pe.cu)
 bool pe_supported(const Ctx& c);
+cudaError_t build_pe_operator(Ctx& c);
 cudaError_t launch_sweep_pe(Ctx& c, int graph_mode, int* grid_out);
 cudaError_t launch_lp_sweep_pe(Ctx& c, const float* in, float* out);   // FP32 corrections
 // fused transport sweep (sweep_fused.cu)

@@ -1,10 +1,17 @@
 // One 128-element tile of the FP64 transport sweep on quadrilaterals with one
 // local operator shared by every element (Sec. 3, eqs. transportLocalk1 and
 // transportLocale), one thread per element: the thread gathers its element's
-// traces at its NQ face points into registers, forms every sweep row
-// Y = Gy + Hy uhat (even and odd columns in two FMA chains), and as the
-// upwind element writes the new trace at the points it owns, adding
-// w (uhat^{k+1} - uhat^k)^2 to the residual.
+// traces at its NQ face points into registers, forms the rows Y = Gy + Hy uhat
+// of the two faces it is upwind of (NQ / 2 rows; no point has beta.n = 0),
+// writes the new trace there and adds w (uhat^{k+1} - uhat^k)^2 to the residual.
+//
+// The products run in fixed point on the integer pipe (fixed_point.cuh), the
+// element's traces and Gy aligned to the largest of them with 56 bits: the FP64
+// pipe, 1.6 operations per clock and SM, bounded the double form (NQ^2 / 2
+// products per element, 200 at p = 4). What is left there is four operations
+// per row: the conversion of the result, the increment, its square, the sum.
+// Every load of a tile is issued before the first product, so that a small
+// problem waits for memory twice (face ids, then all values).
 //
 // The residual is reduced per tile (warp sums, then the warps in order) into
 // partials[tile]; the tile that takes the last ticket of the sweep adds the
@@ -18,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include "ehdg_internal.h"
+#include "fixed_point.cuh"
 #include "sweep_common.cuh"
 
 namespace ehdg {
@@ -35,13 +43,12 @@ __device__ __forceinline__ T pe_ld(const T* p) {
 
 struct PeView {
   int64_t nel, nface;
-  int n_rows, n_up;
-  const int* rows;              // sweep rows (face-point slots), upwind first
+  int own[2];                   // the local faces of the sweep rows: 0 or 1, 2 or 3
+  const int* hs;                // [1] scale: Hy = 2^(hs - 56) x the limbs below
   const int32_t* elem_face;     // [4][nel]
   const double* face_jf;        // [nface]
   const double* fw;             // face Gauss weight of each face point
   const double* Gy;             // [slot][nel]
-  double* Y;                    // rows of tangential points
   float* R_out;                 // mixed precision: F(uhat) - uhat at owned points (or null)
   double* partials;             // [tiles]
   IterState* it;
@@ -52,13 +59,13 @@ struct PeView {
   __host__ __device__ const double* uhat_slot(int s, int64_t tlen) const { return uhat + s * tlen; }
 };
 
-// Hsh: the sweep rows of the operator in row order, [n_rows][NQ]. Returns true
-// in the block that did the final reduction.
+// Hsh: the sweep rows of the operator in row order, limbs, [NQ / 2][NQ] (16-byte
+// aligned). Returns true in the block that did the final reduction.
 template <int NQ, bool CG = false>
-__device__ __forceinline__ bool pe_tile(const PeView& v, const double* Hsh, const double* src,
+__device__ __forceinline__ bool pe_tile(const PeView& v, const int2* Hsh, const double* src,
                                         double* dst, int64_t tile, int64_t ntiles, int graph_mode,
                                         cudaGraphConditionalHandle handle) {
-  constexpr int NQF = NQ / 4;
+  constexpr int NQF = NQ / 4, RN = NQ / 2;
   __shared__ double red[kPeTile / 32];
   __shared__ bool last;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -66,37 +73,52 @@ __device__ __forceinline__ bool pe_tile(const PeView& v, const double* Hsh, cons
   const int64_t e = tile * kPeTile + tid;
   double res = 0.0;
   if (e < ne) {
-    double u[NQ];
+    double u[NQ], gy[RN], w[NQF];
+    int64_t face[4];
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      const int64_t face = v.elem_face[f * ne + e];
+    for (int f = 0; f < 4; ++f) face[f] = v.elem_face[f * ne + e];
 #pragma unroll
-      for (int g = 0; g < NQF; ++g) u[f * NQF + g] = pe_ld<CG>(src + g * nface + face);
-    }
+    for (int j = 0; j < RN; ++j) gy[j] = v.Gy[j * ne + e];
+    const int hs = *v.hs;
 #pragma unroll
-    for (int j = 0; j < NQ; ++j) {
-      if (j >= v.n_rows) break;
-      const double* Hr = Hsh + j * NQ;
-      double a0 = v.Gy[j * ne + e], a1 = 0.0;
+    for (int g = 0; g < NQF; ++g) w[g] = v.fw[g];
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+#pragma unroll
+      for (int g = 0; g < NQF; ++g) u[f * NQF + g] = pe_ld<CG>(src + g * nface + face[f]);
+    const int64_t fo[2] = {v.own[0] ? face[1] : face[0], v.own[1] == 3 ? face[3] : face[2]};
+    const double jf[2] = {v.face_jf[fo[0]], v.face_jf[fo[1]]};
+    int emax = 1;
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) emax = max(emax, fx_exponent(u[c]));
+#pragma unroll
+    for (int j = 0; j < RN; ++j) emax = max(emax, fx_exponent(gy[j]));
+    double sq[2] = {0.0, 0.0};
+    Limb x[NQ];
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) x[c] = fx_split(fx_from_double(u[c], emax));
+#pragma unroll
+    for (int j = 0; j < RN; ++j) {
+      const int4* Hr = reinterpret_cast<const int4*>(Hsh + j * NQ);
+      // the sum in units of 2^(emax - 1078 + hs), Gy aligned to it
+      Acc t(fx_from_double(gy[j], emax + hs));
 #pragma unroll
       for (int c = 0; c < NQ; c += 2) {
-        a0 = fma(Hr[c], u[c], a0);
-        a1 = fma(Hr[c + 1], u[c + 1], a1);
+        const int4 h = Hr[c / 2];
+        t.mac(Cfx{h.x, h.y}, x[c]);
+        t.mac(Cfx{h.z, h.w}, x[c + 1]);
       }
-      const double acc = a0 + a1;
-      const int r = v.rows[j];
-      if (j < v.n_up) {
-        const int f = r / NQF, g = r - f * NQF;
-        const int64_t face = v.elem_face[f * ne + e];
-        const int64_t pt = g * nface + face;
-        dst[pt] = acc;
-        const double d = acc - pe_ld<CG>(src + pt);
-        res += v.face_jf[face] * v.fw[g] * d * d;
-        if (v.R_out) v.R_out[pt] = (float)d;
-      } else {
-        v.Y[(int64_t)r * ne + e] = acc;
-      }
+      double acc = fx_value(t.get(), emax - 1078 + hs);
+      if (emax == 0x7ff) acc = __hiloint2double(0x7ff80000, 0);   // an input is not finite
+      const int b = j / NQF, g = j - b * NQF;
+      const int64_t pt = g * nface + fo[b];
+      const double old = v.own[b] & 1 ? u[(2 * b + 1) * NQF + g] : u[2 * b * NQF + g];
+      const double d = acc - old;
+      dst[pt] = acc;
+      if (v.R_out) v.R_out[pt] = (float)d;
+      sq[b] = fma(w[g], d * d, sq[b]);
     }
+    res = fma(jf[0], sq[0], jf[1] * sq[1]);
   }
   // the tile's partial sum, then a ticket
   res = fsum_warp(res);
@@ -145,8 +167,7 @@ __device__ __forceinline__ bool pe_tile(const PeView& v, const double* Hsh, cons
 // [n_rows][NQ], one FMA chain per row.
 struct LpPeView {
   int64_t nel, nface;
-  int n_up;
-  const int* rows;
+  int own[2];                   // the local faces of the sweep rows
   const int32_t* elem_face;     // [4][nel]
   const float* R;               // [Nqf][nface]
   const float* in;
@@ -155,28 +176,28 @@ struct LpPeView {
 
 template <int NQ, bool CG = false>
 __device__ __forceinline__ void lp_pe_tile(const LpPeView& v, const float* Hsh32, int64_t tile) {
-  constexpr int NQF = NQ / 4;
+  constexpr int NQF = NQ / 4, RN = NQ / 2;
   const int64_t ne = v.nel, nface = v.nface;
   const int64_t e = tile * kPeTile + threadIdx.x;
   if (e >= ne) return;
-  float d[NQ];
+  int64_t face[4];
 #pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    const int64_t face = v.elem_face[f * ne + e];
+  for (int f = 0; f < 4; ++f) face[f] = v.elem_face[f * ne + e];
+  const int64_t fo[2] = {v.own[0] ? face[1] : face[0], v.own[1] == 3 ? face[3] : face[2]};
+  float d[NQ], r[RN];
 #pragma unroll
-    for (int g = 0; g < NQF; ++g) d[f * NQF + g] = pe_ld<CG>(v.in + g * nface + face);
-  }
+  for (int f = 0; f < 4; ++f)
 #pragma unroll
-  for (int j = 0; j < NQ; ++j) {
-    if (j >= v.n_up) break;
+    for (int g = 0; g < NQF; ++g) d[f * NQF + g] = pe_ld<CG>(v.in + g * nface + face[f]);
+#pragma unroll
+  for (int j = 0; j < RN; ++j) r[j] = pe_ld<CG>(v.R + (j % NQF) * nface + fo[j / NQF]);
+#pragma unroll
+  for (int j = 0; j < RN; ++j) {
     const float* Hr = Hsh32 + j * NQ;
     float a = 0.f;
 #pragma unroll
     for (int c = 0; c < NQ; ++c) a = fmaf(Hr[c], d[c], a);
-    const int r = v.rows[j];
-    const int f = r / NQF, g = r - f * NQF;
-    const int64_t pt = g * nface + v.elem_face[f * ne + e];
-    v.out[pt] = pe_ld<CG>(v.R + pt) + a;
+    v.out[(j % NQF) * nface + fo[j / NQF]] = r[j] + a;
   }
 }
 

@@ -47,6 +47,7 @@
 #include <vector>
 
 #include "ehdg_internal.h"
+#include "fixed_point.cuh"
 #include "sweep_common.cuh"
 
 namespace ehdg {
@@ -97,11 +98,8 @@ struct MdParams {
   IterState* it;
 };
 
-// The same tables in fixed point for the sweep, the equation divided by
-// sigma: coefficient c as the limbs of round(c 2^56)
-struct Cfx {
-  int h, l;
-};
+// The same tables in fixed point for the sweep, the equation divided by sigma
+// (Cfx, fixed_point.cuh).
 
 // The fixed-point sweep splits an element over warps: along the second and
 // third axes the coefficients go in pairs (groups; at P1 = 3 the first group
@@ -161,49 +159,6 @@ __device__ __forceinline__ constexpr int md_idx(int a, int i, int t1, int t2) {
                 : (a == 1 ? t1 + P1 * (i + P1 * t2) : t1 + P1 * (t2 + P1 * i));
 }
 
-// --- fixed point ------------------------------------------------------------
-constexpr int kW = 28;                                  // bits of a low limb
-constexpr long long kHalf = 1LL << (kW - 1);
-
-// t = h 2^28 + l with l in [-2^27, 2^27)
-struct Limb {
-  int h, l;
-};
-__device__ __forceinline__ Limb fx_split(long long t) {
-  Limb x;
-  x.h = (int)((t + kHalf) >> kW);
-  x.l = (int)((unsigned)t - ((unsigned)x.h << kW));
-  return x;
-}
-
-__device__ __forceinline__ long long fx_pack(const Limb& x) {
-  return (long long)((unsigned long long)(unsigned)x.h << 32 | (unsigned)x.l);
-}
-__device__ __forceinline__ Limb fx_limb(long long v) {
-  return Limb{(int)(v >> 32), (int)v};
-}
-
-// a += c x. As mad.wide: from the C++ product and sum the compiler made 10
-// instructions of an Acc::mac, from three of these 6.
-__device__ __forceinline__ void fx_mad(long long& a, int c, int x) {
-  long long r;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(c), "r"(x), "l"(a));
-  a = r;
-}
-
-// a sum of products c x 2^56 as hi 2^56 + mid 2^28 (the products of two low
-// limbs, below a quarter of the last place each, are left out)
-struct Acc {
-  long long hi, mid;
-  __device__ __forceinline__ explicit Acc(long long y) : hi(y), mid(kHalf) {}
-  __device__ __forceinline__ void mac(const Cfx& c, const Limb& x) {
-    fx_mad(hi, c.h, x.h);
-    fx_mad(mid, c.h, x.l);
-    fx_mad(mid, c.l, x.h);
-  }
-  __device__ __forceinline__ long long get() const { return hi + (mid >> kW); }
-};
-
 // the value at byte offset off (below 2^32) of a uniform base
 template <class T>
 __device__ __forceinline__ T& fx_at(T* base, unsigned off) {
@@ -248,15 +203,9 @@ struct Align {
   __device__ __forceinline__ long long operator()(long long m) const { return (m + half) >> s; }
 };
 
-// 2^e as a double, e in [-1022, 1023]
-__device__ __forceinline__ double fx_pow2(int e) { return __hiloint2double((e + 1023) << 20, 0); }
-
 __device__ __forceinline__ double fx_to_double(long long m, int e) {
   if (e == kExpNan) return __hiloint2double(0x7ff80000, 0);
-  if (e == kExpZero) return 0.0;
-  if (e > -1000 && e < 900) return (double)m * fx_pow2(e);
-  const int h = e / 2;
-  return (double)m * fx_pow2(h) * fx_pow2(e - h);
+  return e == kExpZero ? 0.0 : fx_value(m, e);
 }
 
 // a face's coefficients to 62-bit integers; returns the blocks' exponents

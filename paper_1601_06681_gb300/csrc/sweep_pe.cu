@@ -16,13 +16,10 @@ namespace {
 
 template <int NQ>
 __global__ void __launch_bounds__(kPeTile) k_sweep_pe(const __grid_constant__ PeView v,
-                                                      const double* Hy, int graph_mode,
+                                                      const int2* Hx, int graph_mode,
                                                       cudaGraphConditionalHandle handle) {
-  __shared__ double Hsh[NQ * NQ];
-  for (int i = threadIdx.x; i < v.n_rows * NQ; i += kPeTile) {
-    const int j = i / NQ, c = i - j * NQ;
-    Hsh[i] = Hy[v.rows[j] * NQ + c];
-  }
+  __shared__ __align__(16) int2 Hsh[NQ / 2 * NQ];
+  for (int i = threadIdx.x; i < NQ / 2 * NQ; i += kPeTile) Hsh[i] = Hx[i];
   __syncthreads();
   const int kk = v.it->k;                     // read before the last tile advances it
   const int64_t tlen = (int64_t)(NQ / 4) * v.nface;
@@ -34,23 +31,24 @@ __global__ void __launch_bounds__(kPeTile) k_sweep_pe(const __grid_constant__ Pe
 }
 
 template <int NQ>
-cudaError_t launch_pe_t(const PeView& v, const double* Hy, int graph_mode,
+cudaError_t launch_pe_t(const PeView& v, const int2* Hx, int graph_mode,
                         cudaGraphConditionalHandle handle, cudaStream_t s, int* grid_out) {
   const int bpsm = fn_blocks_per_sm((const void*)k_sweep_pe<NQ>, kPeTile, 0);
   const int64_t ntiles = (v.nel + kPeTile - 1) / kPeTile;
   int64_t grid = (int64_t)bpsm * device_sms();
   if (grid > ntiles) grid = ntiles;
   *grid_out = (int)grid;
-  k_sweep_pe<NQ><<<(int)grid, kPeTile, 0, s>>>(v, Hy, graph_mode, handle);
+  k_sweep_pe<NQ><<<(int)grid, kPeTile, 0, s>>>(v, Hx, graph_mode, handle);
   return cudaGetLastError();
 }
 
 template <int NQ>
 __global__ void __launch_bounds__(kPeTile) k_lp_pe(const LpPeView v, const float* Hy32) {
-  __shared__ float Hsh[NQ * NQ];
-  for (int i = threadIdx.x; i < v.n_up * NQ; i += kPeTile) {
+  constexpr int NQF = NQ / 4;
+  __shared__ float Hsh[NQ / 2 * NQ];
+  for (int i = threadIdx.x; i < NQ / 2 * NQ; i += kPeTile) {
     const int j = i / NQ, c = i - j * NQ;
-    Hsh[i] = Hy32[v.rows[j] * NQ + c];
+    Hsh[i] = Hy32[(v.own[j / NQF] * NQF + j % NQF) * NQ + c];
   }
   __syncthreads();
   const int64_t ntiles = (v.nel + kPeTile - 1) / kPeTile;
@@ -69,14 +67,37 @@ cudaError_t launch_lp_pe_t(const LpPeView& v, const float* Hy32, cudaStream_t s)
 
 }  // namespace
 
+// The sweep rows of Hy in row order as fixed-point limbs (one block): Hy =
+// 2^(hs - 56) (h 2^28 + l), hs >= 0 the least with max |Hy| <= 2^(hs + 1), so
+// that a coefficient is below 2 and a row's sums of at most 28 products with
+// 56-bit values stay below 2^63.
+static __global__ void k_pe_limbs(int n_rows, int NQFS, const int* rows, const double* Hy, int2* Hx,
+                           int* hs) {
+  __shared__ int s_e;
+  if (threadIdx.x == 0) s_e = 0;
+  __syncthreads();
+  int em = 0;
+  for (int i = threadIdx.x; i < n_rows * NQFS; i += blockDim.x)
+    em = max(em, fx_exponent(Hy[rows[i / NQFS] * NQFS + i % NQFS]));
+  atomicMax(&s_e, em);
+  __syncthreads();
+  const int s = max(0, s_e - 1023);            // |Hy| < 2^(s_e - 1022)
+  if (threadIdx.x == 0) *hs = s;
+  for (int i = threadIdx.x; i < n_rows * NQFS; i += blockDim.x) {
+    const long long c = __double2ll_rn(scalbn(Hy[rows[i / NQFS] * NQFS + i % NQFS], 56 - s));
+    const Limb x = fx_split(c);
+    Hx[i] = make_int2(x.h, x.l);
+  }
+}
+
 // FP32 correction sweep, one thread per element (quadrilaterals, shared
 // operator, no beta.n = 0 point): every sweep row is an owned point.
 cudaError_t launch_lp_sweep_pe(Ctx& c, const float* in, float* out) {
   LpPeView v;
   v.nel = c.nel;
   v.nface = c.nface;
-  v.n_up = c.n_up;
-  v.rows = c.rows;
+  v.own[0] = c.rows_host[0] / c.Nqf;
+  v.own[1] = c.rows_host[c.Nqf] / c.Nqf;
   v.elem_face = c.geo.elem_face;
   v.R = c.R32;
   v.in = in;
@@ -91,23 +112,32 @@ cudaError_t launch_lp_sweep_pe(Ctx& c, const float* in, float* out) {
   }
 }
 
+cudaError_t build_pe_operator(Ctx& c) {
+  cudaError_t e = dalloc_raw(c, (void**)&c.pe_hx, sizeof(int2) * c.n_rows * c.NQFS);
+  if (e == cudaSuccess) e = dalloc_raw(c, (void**)&c.pe_hs, sizeof(int));
+  if (e != cudaSuccess) return e;
+  k_pe_limbs<<<1, 256, 0, c.stream>>>(c.n_rows, c.NQFS, c.rows, c.Hy,
+                                      reinterpret_cast<int2*>(c.pe_hx), c.pe_hs);
+  return cudaGetLastError();
+}
+
 bool pe_supported(const Ctx& c) {
   return c.pde == EHDG_TRANSPORT && c.dim == 2 && c.shared_op && !c.variable_beta &&
-         c.n_tan == 0 && !c.Hyt && c.NQFS >= 8 && c.NQFS <= 28;
+         c.n_tan == 0 && !c.Hyt && c.NQFS >= 8 && c.NQFS <= 28 && c.n_rows == c.n_up &&
+         2 * c.n_up == c.NQFS;   // the rows are the two outflow faces
 }
 
 PeView pe_view(const Ctx& c, double* fw_dev) {
   PeView v = {};
   v.nel = c.nel;
   v.nface = c.nface;
-  v.n_rows = c.n_rows;
-  v.n_up = c.n_up;
-  v.rows = c.rows;
+  v.own[0] = c.rows_host[0] / c.Nqf;
+  v.own[1] = c.rows_host[c.Nqf] / c.Nqf;
+  v.hs = c.pe_hs;
   v.elem_face = c.geo.elem_face;
   v.face_jf = c.geo.face_jf;
   v.fw = fw_dev;
   v.Gy = c.Gy;
-  v.Y = c.Y;
   v.R_out = c.mixed ? c.R32 : nullptr;
   v.partials = c.partials;
   v.it = c.it;
@@ -121,13 +151,14 @@ PeView pe_view(const Ctx& c, double* fw_dev) {
 
 cudaError_t launch_sweep_pe(Ctx& c, int graph_mode, int* grid_out) {
   const PeView v = pe_view(c, c.pe_fw);
+  const int2* Hx = reinterpret_cast<const int2*>(c.pe_hx);
   switch (c.NQFS) {
-    case 8: return launch_pe_t<8>(v, c.Hy, graph_mode, c.handle, c.stream, grid_out);
-    case 12: return launch_pe_t<12>(v, c.Hy, graph_mode, c.handle, c.stream, grid_out);
-    case 16: return launch_pe_t<16>(v, c.Hy, graph_mode, c.handle, c.stream, grid_out);
-    case 20: return launch_pe_t<20>(v, c.Hy, graph_mode, c.handle, c.stream, grid_out);
-    case 24: return launch_pe_t<24>(v, c.Hy, graph_mode, c.handle, c.stream, grid_out);
-    default: return launch_pe_t<28>(v, c.Hy, graph_mode, c.handle, c.stream, grid_out);
+    case 8: return launch_pe_t<8>(v, Hx, graph_mode, c.handle, c.stream, grid_out);
+    case 12: return launch_pe_t<12>(v, Hx, graph_mode, c.handle, c.stream, grid_out);
+    case 16: return launch_pe_t<16>(v, Hx, graph_mode, c.handle, c.stream, grid_out);
+    case 20: return launch_pe_t<20>(v, Hx, graph_mode, c.handle, c.stream, grid_out);
+    case 24: return launch_pe_t<24>(v, Hx, graph_mode, c.handle, c.stream, grid_out);
+    default: return launch_pe_t<28>(v, Hx, graph_mode, c.handle, c.stream, grid_out);
   }
 }
 
