@@ -1070,6 +1070,8 @@ ehdg_status ehdg_create(const ehdg_mesh_desc* mesh, const ehdg_problem_desc* pro
     CKC(cudaStreamSynchronize(c.stream));
     c.use_pe = true;
   }
+  // their persistent forms launch resident blocks only
+  if (c.use_pe || c.md) c.persist_fits = true;
   if (c.shared_op) {
     c.sweep_rows = (int64_t)c.n_rows * c.nel;
   } else {

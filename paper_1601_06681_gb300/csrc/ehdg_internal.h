@@ -60,6 +60,7 @@ struct IterState {
   unsigned int counter;          // last-block ticket of the residual reduction
   int step;                      // steps finished since the last reset (ehdg_run)
   unsigned int bar;              // grid-barrier arrivals of a persistent sweep
+  unsigned int gen;              // passes of it that have ended
   int abort;                     // a persistent sweep's bounded wait gave up
   double r_last;
 };
@@ -295,6 +296,8 @@ cudaError_t build_tiled_operator(Ctx& c);           // after launch_rows; synchr
 cudaError_t launch_sweep_tiled(Ctx& c, int graph_mode, int* grid_out);
 int tiled_persist_blocks_per_sm(const Ctx& c);      // co-resident blocks of the persistent sweep
 bool persistent_sweep_ok(const Ctx& c);             // whole-step sweep in one launch applies
+cudaError_t launch_sweep_pe_persistent(Ctx& c);
+cudaError_t launch_sweep_md_persistent(Ctx& c);
 cudaError_t launch_sweep_persistent(Ctx& c);        // all iterations of a step, one launch
 cudaError_t launch_final_tiled(Ctx& c);              // u = G + H uhat, per-element H
 cudaError_t launch_lp_sweep_tiled(Ctx& c, const float* in, float* out);   // FP32 correction sweep

@@ -1098,6 +1098,7 @@ __global__ void k_reset(IterState* it) {
   it->status = EHDG_OK;
   it->counter = 0u;
   it->bar = 0u;
+  it->gen = 0u;
   it->abort = 0;
   it->r_last = 0.0;
 }

@@ -59,15 +59,13 @@ struct PeView {
   __host__ __device__ const double* uhat_slot(int s, int64_t tlen) const { return uhat + s * tlen; }
 };
 
-// Hsh: the sweep rows of the operator in row order, limbs, [NQ / 2][NQ] (16-byte
-// aligned). Returns true in the block that did the final reduction.
-template <int NQ, bool CG = false>
-__device__ __forceinline__ bool pe_tile(const PeView& v, const int2* Hsh, const double* src,
-                                        double* dst, int64_t tile, int64_t ntiles, int graph_mode,
-                                        cudaGraphConditionalHandle handle) {
+// The tile's sweep; its residual sum goes to partials[tile] (thread 0). Hsh: the
+// sweep rows of the operator in row order, limbs, [NQ / 2][NQ] (16-byte aligned).
+template <int NQ, bool CG>
+__device__ __forceinline__ void pe_tile_sweep(const PeView& v, const int2* Hsh, const double* src,
+                                              double* dst, int64_t tile) {
   constexpr int NQF = NQ / 4, RN = NQ / 2;
   __shared__ double red[kPeTile / 32];
-  __shared__ bool last;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int64_t ne = v.nel, nface = v.nface;
   const int64_t e = tile * kPeTile + tid;
@@ -120,15 +118,33 @@ __device__ __forceinline__ bool pe_tile(const PeView& v, const int2* Hsh, const 
     }
     res = fma(jf[0], sq[0], jf[1] * sq[1]);
   }
-  // the tile's partial sum, then a ticket
   res = fsum_warp(res);
   if (lane == 0) red[wid] = res;
   __syncthreads();
   if (tid == 0) {
     double s = 0.0;
 #pragma unroll
-    for (int w = 0; w < kPeTile / 32; ++w) s += red[w];
+    for (int w2 = 0; w2 < kPeTile / 32; ++w2) s += red[w2];
     v.partials[tile] = s;
+  }
+}
+
+// the sum of all tiles' partials, in warp 0
+__device__ __forceinline__ double pe_total(const double* partials, int64_t ntiles) {
+  double s = 0.0;
+  for (int64_t t = threadIdx.x & 31; t < ntiles; t += 32) s += __ldcg(partials + t);
+  return fsum_warp(s);
+}
+
+// A tile with its ticket; returns true in the block that did the final reduction.
+template <int NQ, bool CG = false>
+__device__ __forceinline__ bool pe_tile(const PeView& v, const int2* Hsh, const double* src,
+                                        double* dst, int64_t tile, int64_t ntiles, int graph_mode,
+                                        cudaGraphConditionalHandle handle) {
+  __shared__ bool last;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  pe_tile_sweep<NQ, CG>(v, Hsh, src, dst, tile);
+  if (tid == 0) {
     __threadfence();
     last = atomicAdd(&v.it->counter, 1u) == (unsigned int)(ntiles - 1);
   }
@@ -136,9 +152,7 @@ __device__ __forceinline__ bool pe_tile(const PeView& v, const int2* Hsh, const 
   if (!last) return false;
   __threadfence();
   if (wid == 0) {
-    double s = 0.0;
-    for (int64_t t = lane; t < ntiles; t += 32) s += reinterpret_cast<volatile double*>(v.partials)[t];
-    s = fsum_warp(s);
+    const double s = pe_total(v.partials, ntiles);
     if (lane == 0) {
       IterState* it = v.it;
       const double r = v.res_scale * sqrt(s);

@@ -170,6 +170,13 @@ __device__ __forceinline__ const T& fx_at(const T* base, unsigned off) {
 }
 
 // named barriers 1 and 2 of a 128-thread block
+// the same for data that a persistent launch rewrites: through L2 only
+template <bool CG, class T>
+__device__ __forceinline__ T fx_ld(const T* base, unsigned off) {
+  if constexpr (CG) return __ldcg(&fx_at(base, off));
+  else return fx_at(base, off);
+}
+
 template <int ID>
 __device__ __forceinline__ void bar_sync() {
   asm volatile("bar.sync %0, 128;" ::"n"(ID) : "memory");
@@ -374,7 +381,7 @@ __device__ __forceinline__ void md_transform(double (&x)[P1 * P1 * P1],
 // this algorithm on the FP64 pipe). 224 MB are read and 79 MB written to DRAM,
 // 1.2 TB/s: the ALU (a mad.wide is a multiply and a 64-bit add) and the latency
 // of the sums at 12 warps per SM bound it.
-template <int P1, bool SOLO>
+template <int P1, bool SOLO, bool PERSIST>
 __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 : 4)
     k_sweep_fx(const __grid_constant__ FxParams<P1> p, const __grid_constant__ MdResid q) {
   using B = MdBlocks<P1>;
@@ -389,14 +396,15 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
   // (the reduction makes it a uniform value: coefficients by role come from the
   // constant bank through uniform registers)
   const int role0 = (int)__reduce_max_sync(0xffffffffu, (threadIdx.y + blockIdx.x) % S::NW);
-  const int kk = p.it->k;                       // read before the last block advances it
+  int kk = p.it->k;                             // read before the last block advances it
+  const int64_t ntiles = (ne + 31) / 32;
+  int buf = 0;
+  for (unsigned int pass = 0;; ++pass, ++kk) {   // one pass unless PERSIST
   const long long* src = p.tr.m + (int64_t)(kk & 1) * N2 * nface;
   long long* dst = p.tr.m + (int64_t)((kk + 1) & 1) * N2 * nface;
   const unsigned long long* esrc = p.tr.e + (int64_t)(kk & 1) * nface;
   unsigned long long* edst = p.tr.e + (int64_t)((kk + 1) & 1) * nface;
-  const int64_t ntiles = (ne + 31) / 32;
   double res = 0.0;
-  int buf = 0;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= TEAM ? 1 : 0) {
     const bool live = tile * 32 + lane < ne;
     const int64_t e = live ? tile * 32 + lane : ne - 1;
@@ -411,8 +419,8 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
     unsigned m0 = 0x80008000u, m1 = 0x80008000u;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      ei[a] = fx_at(esrc, fi[a]);
-      eo[a] = fx_at(esrc, fo[a]);
+      ei[a] = fx_ld<PERSIST>(esrc, fi[a]);
+      eo[a] = fx_ld<PERSIST>(esrc, fo[a]);
       eg[a] = fx_at(p.tr.Ge + a * ne, e8);
       m0 = __vmaxs2(__vmaxs2(m0, (unsigned)ei[a]), __vmaxs2((unsigned)eo[a], (unsigned)eg[a]));
       m1 = __vmaxs2(__vmaxs2(m1, (unsigned)(ei[a] >> 32)),
@@ -440,8 +448,8 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
         const int j = 2 * J + (u & 1) - OFF, k = 2 * K + (u >> 1) - OFF;
         const bool ok = OFF == 0 || (j >= 0 && k >= 0);
         const int64_t g = ok ? j + P1 * k : 0;
-        xi[u] = fx_split(ok ? ai(fx_at(src + g * nface, fi[0])) : 0);
-        xo[u] = fx_split(ok ? ao(fx_at(src + g * nface, fo[0])) : 0);
+        xi[u] = fx_split(ok ? ai(fx_ld<PERSIST>(src + g * nface, fi[0])) : 0);
+        xo[u] = fx_split(ok ? ao(fx_ld<PERSIST>(src + g * nface, fo[0])) : 0);
       }
 #pragma unroll 1
       for (int i = 0; i < P1; ++i) {
@@ -454,10 +462,10 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
           const int k = 2 * K + u - OFF, j = 2 * J + u - OFF;
           const bool oky = OFF == 0 || k >= 0, okz = OFF == 0 || j >= 0;
           const int64_t gy = oky ? i + P1 * k : 0, gz = okz ? i + P1 * j : 0;
-          ty[0][u] = fx_split(oky ? yi(fx_at(src + gy * nface, fi[1])) : 0);
-          ty[1][u] = fx_split(oky ? yo(fx_at(src + gy * nface, fo[1])) : 0);
-          tz[0][u] = fx_split(okz ? zi(fx_at(src + gz * nface, fi[2])) : 0);
-          tz[1][u] = fx_split(okz ? zo(fx_at(src + gz * nface, fo[2])) : 0);
+          ty[0][u] = fx_split(oky ? yi(fx_ld<PERSIST>(src + gy * nface, fi[1])) : 0);
+          ty[1][u] = fx_split(oky ? yo(fx_ld<PERSIST>(src + gy * nface, fo[1])) : 0);
+          tz[0][u] = fx_split(okz ? zi(fx_ld<PERSIST>(src + gz * nface, fi[2])) : 0);
+          tz[1][u] = fx_split(okz ? zo(fx_ld<PERSIST>(src + gz * nface, fo[2])) : 0);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
@@ -558,7 +566,7 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         if (!ok[t]) continue;
-        const long long d = y[t] - ao(fx_at(src + g[t] * nface, face));
+        const long long d = y[t] - ao(fx_ld<PERSIST>(src + g[t] * nface, face));
         const int d1 = (int)((d + (1 << 29)) >> 30);
         const int d0 = (int)((unsigned)d - ((unsigned)d1 << 30));
         fx_mad(s11, d1, d1);
@@ -645,8 +653,38 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
       res = top == kExpNan ? __hiloint2double(0x7ff80000, 0) : fma(r * sc, sc, res);
     }
   }
-  finish_residual(res, q.partials, blockIdx.x, gridDim.x, p.it, q.hist, q.max_iter, q.tol,
-                  q.res_scale, q.graph_mode, q.handle, gridDim.x);
+  if (!PERSIST) {
+    finish_residual(res, q.partials, blockIdx.x, gridDim.x, p.it, q.hist, q.max_iter, q.tol,
+                    q.res_scale, q.graph_mode, q.handle, gridDim.x);
+    return;
+  }
+  // the same sums as finish_residual
+  __shared__ double red[32];
+  const int nw = blockDim.y, wid = threadIdx.y;
+  res = fsum_warp(res);
+  if (lane == 0) red[wid] = res;
+  __syncthreads();
+  if (wid == 0) {
+    const double v = fsum_warp(lane < nw ? red[lane] : 0.0);
+    if (lane == 0) q.partials[blockIdx.x] = v;
+  }
+  const int state = pass_end(p.it, gridDim.x, pass, q.hist, q.max_iter, q.tol, q.res_scale, [&] {
+    double v = 0.0;
+    for (int i = wid * 32 + lane; i < (int)gridDim.x; i += 32 * nw) v += __ldcg(q.partials + i);
+    v = fsum_warp(v);
+    if (lane == 0) red[wid] = v;
+    __syncthreads();
+    double s = 0.0;
+    for (int w = 0; w < nw; ++w) s += red[w];
+    return s;
+  });
+  if (state == 1) continue;
+  if (state == 0 && lane == 0 && wid == 0) {
+    p.it->status = EHDG_ERR_TIMEOUT;
+    p.it->cont = 0;
+  }
+  return;
+  }
 }
 
 // The step's right-hand side in coefficients: G = (tau + sum c T)^{-1} w with
@@ -1315,8 +1353,28 @@ cudaError_t step_t(Ctx& c) {
   return cudaGetLastError();
 }
 
+// One launch form (SOLO or a team of warps) of the sweep; persist: every
+// iteration of the step, cooperative. The grid does not depend on persist, so
+// the residual is the same sum in both.
+template <int P1, bool SOLO>
+cudaError_t sweep_launch(const FxParams<P1>& p, const MdResid& q, int n_partials, bool persist,
+                         cudaStream_t s) {
+  const int nw = SOLO ? 1 : FxShape<P1>::NW;
+  const int bpsm = std::min(fn_blocks_per_sm((const void*)k_sweep_fx<P1, SOLO, true>, 32 * nw, 0),
+                            fn_blocks_per_sm((const void*)k_sweep_fx<P1, SOLO, false>, 32 * nw, 0));
+  const int grid = (int)std::min<int64_t>(
+      n_partials, std::min<int64_t>((int64_t)bpsm * device_sms(), (p.nel + 31) / 32));
+  if (persist) {
+    void* args[] = {const_cast<FxParams<P1>*>(&p), const_cast<MdResid*>(&q)};
+    return cudaLaunchCooperativeKernel((const void*)k_sweep_fx<P1, SOLO, true>, dim3(grid),
+                                       dim3(32, nw), args, 0, s);
+  }
+  k_sweep_fx<P1, SOLO, false><<<grid, dim3(32, nw), 0, s>>>(p, q);
+  return cudaGetLastError();
+}
+
 template <int P1>
-cudaError_t sweep_t(Ctx& c, int graph_mode) {
+cudaError_t sweep_t(Ctx& c, int graph_mode, bool persist) {
   const FxParams<P1>& p = md_args<P1>(c).x;
   MdResid q;
   q.partials = c.partials;
@@ -1326,24 +1384,13 @@ cudaError_t sweep_t(Ctx& c, int graph_mode) {
   q.max_iter = c.max_iter;
   q.graph_mode = graph_mode;
   q.handle = c.handle;
-  constexpr int NW = FxShape<P1>::NW;
-  const int64_t ntiles = (c.nel + 31) / 32;
   // One warp does all groups of its elements where there are tiles enough to
   // keep 12 warps per SM on full runs: 243 against 265 us at 8,192 tiles (64^3,
   // p = 3). With fewer the team's shorter tile wins: 93 against 109 us per
   // iteration at 2,000 tiles, 31 against 45 at 16.
-  if (NW == 1 || ntiles >= 32 * device_sms()) {
-    const int bpsm = fn_blocks_per_sm((const void*)k_sweep_fx<P1, true>, 32, 0);
-    const int grid = (int)std::min<int64_t>(
-        c.n_partials, std::min<int64_t>((int64_t)bpsm * device_sms(), ntiles));
-    k_sweep_fx<P1, true><<<grid, 32, 0, c.stream>>>(p, q);
-  } else {
-    const int bpsm = fn_blocks_per_sm((const void*)k_sweep_fx<P1, false>, 32 * NW, 0);
-    const int grid = (int)std::min<int64_t>(
-        c.n_partials, std::min<int64_t>((int64_t)bpsm * device_sms(), ntiles));
-    k_sweep_fx<P1, false><<<grid, dim3(32, NW), 0, c.stream>>>(p, q);
-  }
-  return cudaGetLastError();
+  if (FxShape<P1>::NW == 1 || (c.nel + 31) / 32 >= 32 * device_sms())
+    return sweep_launch<P1, true>(p, q, c.n_partials, persist, c.stream);
+  return sweep_launch<P1, false>(p, q, c.n_partials, persist, c.stream);
 }
 
 template <int P1>
@@ -1399,9 +1446,17 @@ cudaError_t launch_step_md(Ctx& c) {
 
 cudaError_t launch_sweep_md(Ctx& c, int graph_mode) {
   switch (c.p) {
-    case 1: return sweep_t<2>(c, graph_mode);
-    case 2: return sweep_t<3>(c, graph_mode);
-    default: return sweep_t<4>(c, graph_mode);
+    case 1: return sweep_t<2>(c, graph_mode, false);
+    case 2: return sweep_t<3>(c, graph_mode, false);
+    default: return sweep_t<4>(c, graph_mode, false);
+  }
+}
+
+cudaError_t launch_sweep_md_persistent(Ctx& c) {
+  switch (c.p) {
+    case 1: return sweep_t<2>(c, 0, true);
+    case 2: return sweep_t<3>(c, 0, true);
+    default: return sweep_t<4>(c, 0, true);
   }
 }
 

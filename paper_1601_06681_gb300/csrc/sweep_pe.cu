@@ -7,6 +7,8 @@
 // match their single-problem runs bit for bit.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "ehdg_internal.h"
 #include "pe_tile.cuh"
 
@@ -40,6 +42,49 @@ cudaError_t launch_pe_t(const PeView& v, const int2* Hx, int graph_mode,
   *grid_out = (int)grid;
   k_sweep_pe<NQ><<<(int)grid, kPeTile, 0, s>>>(v, Hx, graph_mode, handle);
   return cudaGetLastError();
+}
+
+// All iterations of a step in one cooperative launch: one pass over the tiles
+// per iteration, the same tile code and residual sum as k_sweep_pe (so the same
+// iterates and decisions bit for bit), traces read through L2. A pass ends for
+// about 3 us where a launch in the conditional graph loop costs 8: 16 x 16, p = 2
+// is all latency, and at 253 x 187, p = 4 it is a third of the iteration.
+template <int NQ>
+__global__ void __launch_bounds__(kPeTile) k_pe_persist(const __grid_constant__ PeView v,
+                                                        const int2* Hx) {
+  __shared__ __align__(16) int2 Hsh[NQ / 2 * NQ];
+  for (int i = threadIdx.x; i < NQ / 2 * NQ; i += kPeTile) Hsh[i] = Hx[i];
+  __syncthreads();
+  const int64_t tlen = (int64_t)(NQ / 4) * v.nface;
+  const int64_t ntiles = (v.nel + kPeTile - 1) / kPeTile;
+  int k = v.it->k;
+  for (unsigned int pass = 0;; ++pass, ++k) {
+    const double* src = v.uhat_slot(k & 1, tlen);
+    double* dst = const_cast<double*>(v.uhat_slot((k + 1) & 1, tlen));
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      pe_tile_sweep<NQ, true>(v, Hsh, src, dst, tile);
+      __syncthreads();                        // thread 0 has read the tile's warp sums
+    }
+    const int state = pass_end(v.it, gridDim.x, pass, v.hist, v.max_iter, v.tol, v.res_scale, [&] {
+      return threadIdx.x < 32 ? pe_total(v.partials, ntiles) : 0.0;
+    });
+    if (state == 1) continue;
+    if (state == 0 && threadIdx.x == 0) {
+      v.it->status = EHDG_ERR_TIMEOUT;
+      v.it->cont = 0;
+    }
+    return;
+  }
+}
+
+template <int NQ>
+cudaError_t launch_pe_persist_t(const PeView& v, const int2* Hx, cudaStream_t s) {
+  const int bpsm = fn_blocks_per_sm((const void*)k_pe_persist<NQ>, kPeTile, 0);
+  const int64_t ntiles = (v.nel + kPeTile - 1) / kPeTile;
+  const int grid = (int)std::min<int64_t>((int64_t)bpsm * device_sms(), ntiles);
+  void* args[] = {const_cast<PeView*>(&v), &Hx};
+  return cudaLaunchCooperativeKernel((const void*)k_pe_persist<NQ>, dim3(grid), dim3(kPeTile),
+                                     args, 0, s);
 }
 
 template <int NQ>
@@ -147,6 +192,19 @@ PeView pe_view(const Ctx& c, double* fw_dev) {
   v.res_scale = c.res_scale;
   v.uhat = c.uhat;
   return v;
+}
+
+cudaError_t launch_sweep_pe_persistent(Ctx& c) {
+  const PeView v = pe_view(c, c.pe_fw);
+  const int2* Hx = reinterpret_cast<const int2*>(c.pe_hx);
+  switch (c.NQFS) {
+    case 8: return launch_pe_persist_t<8>(v, Hx, c.stream);
+    case 12: return launch_pe_persist_t<12>(v, Hx, c.stream);
+    case 16: return launch_pe_persist_t<16>(v, Hx, c.stream);
+    case 20: return launch_pe_persist_t<20>(v, Hx, c.stream);
+    case 24: return launch_pe_persist_t<24>(v, Hx, c.stream);
+    default: return launch_pe_persist_t<28>(v, Hx, c.stream);
+  }
 }
 
 cudaError_t launch_sweep_pe(Ctx& c, int graph_mode, int* grid_out) {

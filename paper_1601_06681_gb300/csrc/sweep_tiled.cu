@@ -270,10 +270,14 @@ int tiled_persist_blocks_per_sm(const Ctx& c) {
 }
 
 bool persistent_sweep_ok(const Ctx& c) {
-  return c.Hyt && c.persist_fits && c.ppartials && !c.mixed && c.n_tan == 0;
+  if (c.mixed || c.n_tan != 0 || !c.persist_fits) return false;
+  if (c.use_ozaki) return false;
+  return md_active(c) || c.use_pe || (c.Hyt && c.ppartials);
 }
 
 cudaError_t launch_sweep_persistent(Ctx& c) {
+  if (md_active(c)) return launch_sweep_md_persistent(c);
+  if (c.use_pe) return launch_sweep_pe_persistent(c);
   TiledParams p;
   fill_params(c, p, 0);
   p.partials = c.ppartials;
