@@ -91,12 +91,11 @@ struct BInst {
   // once-per-step kernels: right-hand side, initial trace, reconstruction
   int n, KE, cn;
   double ucoef;
-  const double* P;
+  FxOp Px, Hx2, Eyx;            // P / dt, H and Ey in fixed point
   double* u;
   const int* ey_idx;
   const double* ey_val;
   double* G;
-  const double* H;
   double* uhat_n;
   const double* gb;
   double* gb_old;
@@ -992,9 +991,11 @@ __device__ StepParams step_params(const BInst& I) {
   p.n = I.n;
   p.NQFS = I.NQFS;
   p.KE = I.KE;
+  p.nf = 1;
   p.shared = 1;
   p.ucoef = I.ucoef;
-  p.P = I.P;
+  p.Px = I.Px;
+  p.Eyx = I.Eyx;
   p.u = I.u;
   p.ey_idx = I.ey_idx;
   p.ey_val = I.ey_val;
@@ -1009,10 +1010,10 @@ __device__ StepParams step_params(const BInst& I) {
 // the step's right-hand side G = P w, Gy and Y0 (items: 32-element tiles)
 __global__ void __launch_bounds__(32 * kStepT) k_batch_step(const BInst* inst, const int* pre,
                                                             int n_inst, int nmax) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   const int tid = threadIdx.y * 32 + threadIdx.x;
-  double* Psh = sm;                                   // [n][n]
-  double* w = Psh + nmax * nmax;                      // [n][32]
+  int2* Psh = reinterpret_cast<int2*>(sm);            // limbs of P
+  double* w = sm + fx_blocked(nmax, nmax);            // [n][32]
   double* g = w + nmax * 32;                          // [n][32]
   const int n_items = pre[n_inst];
   int cur = -1;
@@ -1021,7 +1022,7 @@ __global__ void __launch_bounds__(32 * kStepT) k_batch_step(const BInst* inst, c
     const BInst& I = inst[i];
     if (i != cur) {   // step_tile starts and ends with barriers around its use of Psh
       __syncthreads();
-      for (int k = tid; k < I.n * I.n; k += 32 * kStepT) Psh[k] = I.P[k];
+      for (int k = tid; k < fx_blocked(I.n, I.n); k += 32 * kStepT) Psh[k] = I.Px.x[k];
       cur = i;
     }
     step_tile(step_params(I), Psh, w, g, nullptr, it - pre[i]);
@@ -1054,10 +1055,10 @@ __global__ void __launch_bounds__(256) k_batch_trace0(const BInst* inst, const i
 // the reconstruction u^{k+1} = G + H uhat^k (items: 32-element tiles)
 __global__ void __launch_bounds__(32 * kStepT) k_batch_final(const BInst* inst, const int* pre,
                                                              int n_inst, int nmax, int nqmax) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   const int tid = threadIdx.y * 32 + threadIdx.x;
-  double* Hsh = sm;                                   // [n][NQFS]
-  double* uh = Hsh + nmax * nqmax;                    // [NQFS][32]
+  int2* Hsh = reinterpret_cast<int2*>(sm);            // limbs of H
+  double* uh = sm + fx_blocked(nmax, nqmax);          // [NQFS][32]
   const int n_items = pre[n_inst];
   int cur = -1;
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
@@ -1065,7 +1066,7 @@ __global__ void __launch_bounds__(32 * kStepT) k_batch_final(const BInst* inst, 
     const BInst& I = inst[i];
     if (i != cur) {
       __syncthreads();
-      for (int k = tid; k < I.n * I.NQFS; k += 32 * kStepT) Hsh[k] = I.H[k];
+      for (int k = tid; k < fx_blocked(I.n, I.NQFS); k += 32 * kStepT) Hsh[k] = I.Hx2.x[k];
       cur = i;
     }
     FinalParams p = {};
@@ -1081,7 +1082,7 @@ __global__ void __launch_bounds__(32 * kStepT) k_batch_final(const BInst* inst, 
     p.uhat = I.uhat;
     p.it = I.it;
     p.G = I.G;
-    p.H = I.H;
+    p.Hx = I.Hx2;
     p.u = I.u;
     const double* src = I.uhat + (int64_t)((I.it->k + 1) & 1) * I.Nqf * I.nface;
     final_tile(p, Hsh, uh, src, it - pre[i]);
@@ -1268,12 +1269,13 @@ cudaError_t BatchLoop::build(const std::vector<Ctx*>& ctxs, unsigned long long* 
     I.KE = c.KE;
     I.cn = (c.scheme == EHDG_CN) ? 1 : 0;
     I.ucoef = (c.scheme == EHDG_STEADY) ? 0.0 : 1.0 / c.dt_eff;
-    I.P = c.P;
+    I.Px = FxOp{static_cast<const int2*>(c.fx_P), c.fx_Ps};
     I.u = c.u;
     I.ey_idx = c.ey_idx;
     I.ey_val = c.ey_val;
     I.G = c.G;
-    I.H = c.H;
+    I.Hx2 = FxOp{static_cast<const int2*>(c.fx_H), c.fx_Hs};
+    I.Eyx = FxOp{static_cast<const int2*>(c.fx_E), c.fx_Es};
     I.uhat_n = c.uhat_n;
     I.gb = c.gb;
     I.gb_old = c.gb_old;
@@ -1409,8 +1411,8 @@ cudaError_t BatchLoop::build(const std::vector<Ctx*>& ctxs, unsigned long long* 
     return std::max(1, std::min(bpsm * device_sms(), items));
   };
   L.sweep_grid = wave(k_batch_sweep, kPeTile, smem, L.n_sweep);
-  L.step_smem = sizeof(double) * ((size_t)L.nmax * L.nmax + 64 * (size_t)L.nmax);
-  L.final_smem = sizeof(double) * ((size_t)L.nmax * L.nqmax + 32 * (size_t)L.nqmax);
+  L.step_smem = sizeof(double) * ((size_t)fx_blocked(L.nmax, L.nmax) + 64 * (size_t)L.nmax);
+  L.final_smem = sizeof(double) * ((size_t)fx_blocked(L.nmax, L.nqmax) + 32 * (size_t)L.nqmax);
   if ((e = cudaFuncSetAttribute(k_batch_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)L.step_smem)) != cudaSuccess)
     return e;

@@ -164,6 +164,10 @@ struct Ctx {
   // transport operator): the element's face traces go to its boundary nodes
   // by two 1D passes per face (Bs), then Dy = Ey A^{-1}[:, bnd] gives the
   // face-point rows and Ab = A^{-1}[:, bnd] the volume values
+  // a shared operator's products in fixed point (fixed_point.cuh): P / dt, H, Ey
+  // and, for shallow water, Hy as limbs with their scales
+  void *fx_P = nullptr, *fx_H = nullptr, *fx_E = nullptr, *fx_Hy = nullptr;
+  int *fx_Ps = nullptr, *fx_Hs = nullptr, *fx_Es = nullptr, *fx_Hys = nullptr;
   bool use_pe = false;           // 2D shared-operator FP64 sweep, one thread per element
   double* pe_fw = nullptr;       // its face Gauss weights [Nqf]
   void* pe_hx = nullptr;         // [n_rows][NQFS] its rows of Hy as fixed-point limbs (int2)
@@ -237,6 +241,7 @@ struct Ctx {
 
 // launchers (kernels.cu)
 cudaError_t launch_assemble(Ctx& c, int n_assemble);
+cudaError_t build_fx_operators(Ctx& c);   // shared operator, after assembly
 cudaError_t launch_face_signs(Ctx& c);
 cudaError_t launch_step(Ctx& c);
 cudaError_t launch_elem(Ctx& c);

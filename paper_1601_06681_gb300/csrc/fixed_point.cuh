@@ -89,4 +89,36 @@ __device__ __forceinline__ long long fx_from_double(double x, int emax) {
   return (v ^ sg) - sg;
 }
 
+// A shared operator's rows as limbs in blocks of four rows, [rows / 4][cols][4]
+// (the last block zero-padded). The columns are in nf groups (the fields of the
+// state, which may differ in size by orders), and each row has a scale for each
+// group, scale[row * nf + f]: entry = 2^(scale - 56) (h 2^28 + l), the limbs'
+// value below 2 and its sum over the group below 32, so that a group's products
+// with 56-bit values sum below 2^62.
+struct FxOp {
+  const int2* x;
+  const int* scale;
+};
+__host__ __device__ inline int64_t fx_blocked(int rows, int cols) {
+  return (int64_t)((rows + 3) / 4) * 4 * cols;
+}
+
+// four rows (blk) times the column of packed limbs X[c * 32]
+__device__ __forceinline__ void fx_rows4(const int2* blk, const long long* X, int cols,
+                                         long long (&y)[4]) {
+  Acc t[4] = {Acc(0), Acc(0), Acc(0), Acc(0)};
+  const int4* b = reinterpret_cast<const int4*>(blk);
+#pragma unroll 4
+  for (int c = 0; c < cols; ++c) {
+    const int4 p = b[2 * c], q = b[2 * c + 1];
+    const Limb x = fx_limb(X[c * 32]);
+    t[0].mac(Cfx{p.x, p.y}, x);
+    t[1].mac(Cfx{p.z, p.w}, x);
+    t[2].mac(Cfx{q.x, q.y}, x);
+    t[3].mac(Cfx{q.z, q.w}, x);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) y[i] = t[i].get();
+}
+
 }  // namespace ehdg

@@ -10,6 +10,7 @@
 #include <cmath>
 
 #include "ehdg_internal.h"
+#include "fixed_point.cuh"
 #include "step_tiles.cuh"
 
 namespace ehdg {
@@ -431,20 +432,66 @@ cudaError_t launch_face_signs(Ctx& c) {
 // Per-step right-hand side: G = P w, Gy = Ey G, Y0 = Ey u^n
 //   w = u^n / dt_eff + f (time-dependent) or w = f (steady)
 // ===========================================================================
+// A shared operator's matrix M [rows][cols] times coef as limbs (FxOp), one
+// block: the scales are the least with the group's largest entry below 2 and
+// its sum of magnitudes below 32. blocked: the layout of FxOp, else row-major.
+__global__ void k_fx_limbs(int rows, int cols, int nf, double coef, const double* M, int blocked,
+                           int2* x, int* scale) {
+  const int np = cols / nf, rows4 = blocked ? (rows + 3) / 4 * 4 : rows;
+  for (int i = threadIdx.x; i < rows4 * nf; i += blockDim.x) {
+    const int r = i / nf, f = i - r * nf;
+    double mx = 0.0, sum = 0.0;
+    if (r < rows)
+      for (int c = f * np; c < (f + 1) * np; ++c) {
+        const double v = fabs(coef * M[r * cols + c]);
+        mx = fmax(mx, v);
+        sum += v;
+      }
+    scale[i] = mx > 0.0 ? max(ilogb(mx), ilogb(sum) + 1 - 5) : 0;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < rows4 * cols; i += blockDim.x) {
+    const int r = i / cols, c = i - r * cols;
+    const double v = r < rows ? coef * M[r * cols + c] : 0.0;
+    const Limb l = fx_split(__double2ll_rn(scalbn(v, 56 - scale[r * nf + c / np])));
+    x[blocked ? ((r / 4) * (int64_t)cols + c) * 4 + r % 4 : i] = make_int2(l.h, l.l);
+  }
+}
+
+cudaError_t build_fx_operators(Ctx& c) {
+  auto make = [&](int rows, int cols, int nf, double coef, const double* M, bool blocked,
+                  void** x, int** scale) {
+    const int r4 = blocked ? (rows + 3) / 4 * 4 : rows;
+    cudaError_t e = dalloc_raw(c, x, sizeof(int2) * r4 * cols);
+    if (e == cudaSuccess) e = dalloc_raw(c, (void**)scale, sizeof(int) * r4 * nf);
+    if (e != cudaSuccess) return e;
+    k_fx_limbs<<<1, 512, 0, c.stream>>>(rows, cols, nf, coef, M, blocked ? 1 : 0,
+                                        static_cast<int2*>(*x), *scale);
+    return cudaGetLastError();
+  };
+  const double uc = c.scheme == EHDG_STEADY ? 1.0 : 1.0 / c.dt_eff;
+  cudaError_t e = make(c.n, c.n, c.nf, uc, c.P, true, &c.fx_P, &c.fx_Ps);
+  if (e == cudaSuccess) e = make(c.n, c.NQFS, 1, 1.0, c.H, true, &c.fx_H, &c.fx_Hs);
+  if (e == cudaSuccess) e = make(c.NQFS, c.KE, 1, 1.0, c.ey_val, false, &c.fx_E, &c.fx_Es);
+  if (e == cudaSuccess && c.pde == EHDG_SW_LINEAR)
+    e = make(c.NQFS, c.NQFS, 1, 1.0, c.Hy, false, &c.fx_Hy, &c.fx_Hys);
+  return e;
+}
+
 // Tile of 32 consecutive elements (threadIdx.x) x kStepT row groups
 // (threadIdx.y); persistent over tiles. w and G of the tile live in shared
 // memory; a shared operator P is staged once per block. The tile body is in
 // step_tiles.cuh (the batched loop runs it too).
 __global__ void __launch_bounds__(32 * kStepT) k_step(const __grid_constant__ StepParams s) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   const int lane = threadIdx.x, t = threadIdx.y, tid = t * 32 + lane;
   const int n = s.n;
-  double* Psh = sm;                                   // n*n if shared
-  double* w = sm + (s.shared ? n * n : 0);            // [n][32]
+  const int64_t np = s.shared && !s.g_ready ? fx_blocked(n, n) : 0;
+  int2* Psh = reinterpret_cast<int2*>(sm);            // the shared operator's limbs
+  double* w = sm + np;                                // [n][32]
   double* g = w + n * 32;                             // [n][32]
   double* sfw = g + n * 32;                           // face passes (sf_ey)
-  if (s.shared)
-    for (int i = tid; i < n * n; i += 32 * kStepT) Psh[i] = s.P[i];
+  for (int64_t i = tid; i < np; i += 32 * kStepT) Psh[i] = s.Px.x[i];
   const int64_t ntiles = (s.nel + 31) / 32;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
     step_tile(s, Psh, w, g, sfw, tile);
@@ -487,9 +534,13 @@ cudaError_t launch_step(Ctx& c) {
   StepParams s;
   s.nel = c.nel;
   s.n = c.n;
+  s.nf = c.nf;
   s.NQFS = c.NQFS;
   s.KE = c.KE;
   s.shared = c.shared_op ? 1 : 0;
+  s.fcoef = (c.scheme == EHDG_STEADY) ? 1.0 : c.dt_eff;
+  s.Px = FxOp{static_cast<const int2*>(c.fx_P), c.fx_Ps};
+  s.Eyx = FxOp{static_cast<const int2*>(c.fx_E), c.fx_Es};
   s.ucoef = (c.scheme == EHDG_STEADY) ? 0.0 : 1.0 / c.dt_eff;
   s.have_force = c.have_force ? 1 : 0;
   s.force_avg = (c.scheme == EHDG_CN) ? 1 : 0;
@@ -516,7 +567,8 @@ cudaError_t launch_step(Ctx& c) {
   }
   step_sf_plan(c, s);
   const size_t smem =
-      sizeof(double) * ((s.shared ? (size_t)c.n * c.n : 0) + 2 * (size_t)c.n * 32 +
+      sizeof(double) * ((s.shared && !s.g_ready ? (size_t)fx_blocked(c.n, c.n) : 0) +
+                        2 * (size_t)c.n * 32 +
                         (s.sf_ey ? (size_t)s.sf_nf * s.sf_p1 * s.sf_p1 * 2 * 32 : 0));
   cudaError_t err = fn_smem((const void*)k_step, smem);
   if (err != cudaSuccess) return err;
@@ -548,6 +600,7 @@ struct ElemParams {
   const IterState* it;
   const double* Gy;             // [slot][nel]
   const double* Hy;             // shared: [NQFS][NQFS]; per element: [slot][NQFS][nel]
+  FxOp Hx;                      // shared operator: Hy as limbs, row-major
   double* Y;                    // [NQFS][nel]
 };
 
@@ -599,6 +652,62 @@ __global__ void __launch_bounds__(32 * kElemT) k_elem(const ElemParams p) {
   }
 }
 
+// The element values of shallow water with one operator for all elements
+// (Y = Gy + Hy phihat, every face point), in fixed point with one thread per
+// element, as the quadrilateral transport sweep (pe_tile.cuh) forms its rows.
+// 512 x 512, p = 3: 122 us on the FP64 pipe (256 products per element).
+template <int NQ>
+__global__ void __launch_bounds__(128) k_elem_fx(const __grid_constant__ ElemParams p) {
+  constexpr int NQF = NQ / 4;
+  __shared__ __align__(16) int2 Hsh[NQ * NQ];
+  __shared__ int s_scale[NQ];
+  for (int i = threadIdx.x; i < NQ * NQ; i += 128) Hsh[i] = p.Hx.x[i];
+  for (int i = threadIdx.x; i < NQ; i += 128) s_scale[i] = p.Hx.scale[i];
+  __syncthreads();
+  const int64_t ne = p.nel;
+  const double* src = p.uhat + (int64_t)(p.it->k & 1) * NQF * p.nface;
+  for (int64_t e = blockIdx.x * 128LL + threadIdx.x; e < ne; e += gridDim.x * 128LL) {
+    double u[NQ], gy[NQ];
+    int64_t face[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) face[f] = p.elem_face[f * ne + e];
+#pragma unroll
+    for (int j = 0; j < NQ; ++j) gy[j] = p.Gy[j * ne + e];
+    int em = 1;
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+#pragma unroll
+      for (int g = 0; g < NQF; ++g) {
+        u[f * NQF + g] = src[g * p.nface + face[f]];
+        em = max(em, fx_exponent(u[f * NQF + g]));
+      }
+    Limb x[NQ];
+#pragma unroll
+    for (int c = 0; c < NQ; ++c) x[c] = fx_split(fx_from_double(u[c], em));
+#pragma unroll
+    for (int j = 0; j < NQ; ++j) {
+      const int4* Hr = reinterpret_cast<const int4*>(Hsh + j * NQ);
+      Acc t(0);
+#pragma unroll
+      for (int c = 0; c < NQ; c += 2) {
+        const int4 h = Hr[c / 2];
+        t.mac(Cfx{h.x, h.y}, x[c]);
+        t.mac(Cfx{h.z, h.w}, x[c + 1]);
+      }
+      const double y = em == 0x7ff ? __hiloint2double(0x7ff80000, 0)
+                                   : fx_value(t.get(), em - 1078 + s_scale[j]);
+      p.Y[(int64_t)j * ne + e] = gy[j] + y;
+    }
+  }
+}
+
+template <int NQ>
+static cudaError_t launch_elem_fx(const ElemParams& p, cudaStream_t s) {
+  const int grid = persistent_grid(k_elem_fx<NQ>, 128, 0, (p.nel + 127) / 128);
+  k_elem_fx<NQ><<<grid, 128, 0, s>>>(p);
+  return cudaGetLastError();
+}
+
 template <int NQ>
 static cudaError_t launch_elem_t(const ElemParams& p, size_t smem, int grid, cudaStream_t s) {
   cudaError_t err = fn_smem((const void*)k_elem<NQ>, smem);
@@ -626,6 +735,17 @@ cudaError_t launch_elem(Ctx& c) {
   p.Gy = c.Gy;
   p.Hy = c.Hy;
   p.Y = c.Y;
+  p.Hx = FxOp{static_cast<const int2*>(c.fx_Hy), c.fx_Hys};
+  if (c.fx_Hy) {   // every shallow-water shape (p <= 5)
+    switch (c.NQFS) {
+      case 8: return launch_elem_fx<8>(p, c.stream);
+      case 12: return launch_elem_fx<12>(p, c.stream);
+      case 16: return launch_elem_fx<16>(p, c.stream);
+      case 20: return launch_elem_fx<20>(p, c.stream);
+      case 24: return launch_elem_fx<24>(p, c.stream);
+      default: break;
+    }
+  }
   const size_t smem = sizeof(double) * ((p.shared ? (size_t)c.NQFS * c.NQFS : 0) + (size_t)c.NQFS * 32);
   const int grid = (int)((c.nel + 31) / 32);
   switch (c.NQFS) {
@@ -903,12 +1023,12 @@ cudaError_t launch_trace0(Ctx& c) {
 // End of step: u^{n+1} = G + H uhat (Crank-Nicolson: 2 v - u^n), trace update
 // ===========================================================================
 __global__ void __launch_bounds__(32 * kStepT) k_final(const FinalParams p) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   const int lane = threadIdx.x, t = threadIdx.y, tid = t * 32 + lane;
-  double* Hsh = sm;
-  double* uh = sm + (p.shared ? p.n * p.NQFS : 0);     // [NQFS][32]
-  if (p.shared)
-    for (int i = tid; i < p.n * p.NQFS; i += 32 * kStepT) Hsh[i] = p.H[i];
+  const int64_t nh = p.shared ? fx_blocked(p.n, p.NQFS) : 0;
+  int2* Hsh = reinterpret_cast<int2*>(sm);
+  double* uh = sm + nh;                                // [NQFS][32]
+  for (int64_t i = tid; i < nh; i += 32 * kStepT) Hsh[i] = p.Hx.x[i];
   const int64_t ntiles = (p.nel + 31) / 32;
   // Algorithm 1 returns u^{k+1}, the local solve with the trace uhat^k
   const double* src = p.uhat + (int64_t)((p.it->k + 1) & 1) * p.Nqf * p.nface;
@@ -955,6 +1075,7 @@ cudaError_t launch_final(Ctx& c) {
   p.it = c.it;
   p.G = c.G;
   p.H = c.H;
+  p.Hx = FxOp{static_cast<const int2*>(c.fx_H), c.fx_Hs};
   p.u = c.u;
   cudaError_t err;
   if (c.use_ozaki && c.oz_final.img) {
@@ -965,7 +1086,7 @@ cudaError_t launch_final(Ctx& c) {
     err = launch_final_sf(c);
   } else {
     const size_t smem =
-        sizeof(double) * ((p.shared ? (size_t)c.n * c.NQFS : 0) + (size_t)c.NQFS * 32);
+        sizeof(double) * ((p.shared ? (size_t)fx_blocked(c.n, c.NQFS) : 0) + (size_t)c.NQFS * 32);
     err = fn_smem((const void*)k_final, smem);
     if (err != cudaSuccess) return err;
     const int grid = persistent_grid(k_final, 32 * kStepT, smem, (c.nel + 31) / 32);

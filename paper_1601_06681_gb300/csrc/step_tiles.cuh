@@ -4,11 +4,18 @@
 // reconstruction u^{k+1} = G + H uhat^k (Crank-Nicolson: 2 v - u^n). The
 // single-problem kernels and the batched step run this code, so their
 // results agree bit for bit.
+//
+// With one operator for all elements the products P w, Ey G and H uhat run in
+// fixed point on the integer pipe (fixed_point.cuh), the element's inputs
+// aligned to the largest of them: on the FP64 pipe (1.6 operations per clock
+// and SM) they bounded the step, 48 x 48 and 48 x 16 products per element for
+// shallow water at p = 3.
 #pragma once
 
 #include <cuda_runtime.h>
 
 #include "ehdg_internal.h"
+#include "fixed_point.cuh"
 
 namespace ehdg {
 
@@ -16,10 +23,13 @@ constexpr int kStepT = 4;
 
 struct StepParams {
   int64_t nel;
-  int n, NQFS, KE, shared;
+  int n, nf, NQFS, KE, shared;
   double ucoef;                 // 1/dt_eff, or 0 for steady
+  double fcoef;                 // shared operator: w / ucoef = u + fcoef f (steady: f)
   int have_force, force_avg;    // force_avg: use 0.5 (f_old + f) (Crank-Nicolson)
-  const double* P;
+  const double* P;              // per-element operator
+  FxOp Px;                      // shared operator: ucoef P (steady: P)
+  FxOp Eyx;                     // shared operator: Ey, [NQFS][KE] (not blocked)
   const double* u;
   const double* force;
   const double* force_old;
@@ -45,9 +55,73 @@ struct StepParams {
   const int* warm;
 };
 
-// Psh: a shared operator P [n][n]; w, g: [n][32] scratch; sfw: the face
+// the largest biased exponent over a tile's warps of each lane's values, >= 1
+__device__ __forceinline__ int tile_max(int v) {
+  __shared__ int s_max[kStepT][32];
+  s_max[threadIdx.y][threadIdx.x] = v;
+  __syncthreads();
+  int m = 1;
+#pragma unroll
+  for (int t = 0; t < kStepT; ++t) m = max(m, s_max[t][threadIdx.x]);
+  __syncthreads();
+  return m;
+}
+
+// values v[c * 32] (c0 <= c < c1) of a lane to packed limbs in place, in units
+// of 2^(emax - 1078); returns emax (0x7ff: a value is not finite)
+__device__ __forceinline__ int tile_limbs(double* v, int c0, int c1) {
+  const int lane = threadIdx.x, t = threadIdx.y;
+  int em = 1;
+  for (int c = c0 + t; c < c1; c += kStepT) em = max(em, fx_exponent(v[c * 32 + lane]));
+  em = tile_max(em);
+  long long* x = reinterpret_cast<long long*>(v);
+  for (int c = c0 + t; c < c1; c += kStepT)
+    x[c * 32 + lane] = fx_pack(fx_split(fx_from_double(v[c * 32 + lane], em)));
+  __syncthreads();
+  return em;
+}
+
+// Rows b*4 .. b*4+3 of a shared operator (limbs in osh) times a tile's columns:
+// X the packed limbs, nf groups of cols / nf columns in units of 2^(em[f] - 1078).
+// The groups' sums are aligned to the coarsest unit of the row's groups.
+__device__ __forceinline__ void tile_rows4(const FxOp& op, const int2* osh, const double* X, int b,
+                                           int cols, int nf, const int (&em)[3], double (&out)[4]) {
+  const int np = cols / nf;
+  const long long* x = reinterpret_cast<const long long*>(X) + threadIdx.x;
+  const int* sc = op.scale + b * 4 * nf;
+  long long sum[4] = {0, 0, 0, 0};
+  int L[4];
+  bool nan = false;
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    if (f >= nf) break;
+    long long y[4];
+    fx_rows4(osh + ((int64_t)b * cols + f * np) * 4, x + f * np * 32, np, y);
+    nan |= em[f] == 0x7ff;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int Lf = em[f] - 1078 + sc[i * nf + f];
+      if (f == 0) {
+        L[i] = Lf;
+        sum[i] = y[i];
+      } else if (Lf > L[i]) {
+        const int sh = min(63, Lf - L[i]);
+        sum[i] = ((sum[i] + ((1LL << sh) >> 1)) >> sh) + y[i];
+        L[i] = Lf;
+      } else {
+        const int sh = min(63, L[i] - Lf);
+        sum[i] += (y[i] + ((1LL << sh) >> 1)) >> sh;
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    out[i] = nan ? __hiloint2double(0x7ff80000, 0) : fx_value(sum[i], L[i]);
+}
+
+// Psh: a shared operator's blocked limbs; w, g: [n][32] scratch; sfw: the face
 // passes' scratch [sf_nf q][p+1][2][32] (sf_ey only).
-__device__ __forceinline__ void step_tile(const StepParams& s, const double* Psh, double* w,
+__device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, double* w,
                                           double* g, double* sfw, int64_t tile) {
   const int lane = threadIdx.x, t = threadIdx.y;
   const int n = s.n;
@@ -62,25 +136,37 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const double* Psh
     for (int c = t; c < n; c += kStepT) {
       double v = 0.0;
       if (live) {
-        v = s.u[c * ne + e] * s.ucoef;
-        if (s.have_force)
-          v += s.force_avg ? 0.5 * (s.force[c * ne + e] + s.force_old[c * ne + e])
-                           : s.force[c * ne + e];
+        v = s.shared ? (s.ucoef != 0.0 ? s.u[c * ne + e] : 0.0) : s.u[c * ne + e] * s.ucoef;
+        if (s.have_force) {
+          const double f = s.force_avg ? 0.5 * (s.force[c * ne + e] + s.force_old[c * ne + e])
+                                       : s.force[c * ne + e];
+          v = s.shared ? fma(s.fcoef, f, v) : v + f;
+        }
       }
       w[c * 32 + lane] = v;
     }
     __syncthreads();
-    for (int r = t; r < n; r += kStepT) {
-      double a0 = 0.0, a1 = 0.0;
-      if (s.shared) {
-        const double* Pr = Psh + r * n;
-        int c = 0;
-        for (; c + 1 < n; c += 2) {
-          a0 = fma(Pr[c], w[c * 32 + lane], a0);
-          a1 = fma(Pr[c + 1], w[(c + 1) * 32 + lane], a1);
+    if (s.shared) {
+      const int np = n / s.nf;
+      int em[3] = {1, 1, 1};
+#pragma unroll
+      for (int f = 0; f < 3; ++f)
+        if (f < s.nf) em[f] = tile_limbs(w, f * np, (f + 1) * np);
+      for (int b = t; b * 4 < n; b += kStepT) {
+        double v[4];
+        tile_rows4(s.Px, Psh, w, b, n, s.nf, em, v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = b * 4 + i;
+          if (r >= n) break;
+          if (live) s.G[r * ne + e] = v[i];
+          g[r * 32 + lane] = v[i];
         }
-        if (c < n) a0 = fma(Pr[c], w[c * 32 + lane], a0);
-      } else if (live) {
+      }
+    }
+    for (int r = t; r < (s.shared ? 0 : n); r += kStepT) {
+      double a0 = 0.0, a1 = 0.0;
+      if (live) {
         const double* Pr = s.P + (int64_t)r * n * ne + e;
         int c = 0;
         for (; c + 1 < n; c += 2) {
@@ -145,6 +231,8 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const double* Psh
     }
     return;
   }
+  const bool limbs = s.shared && !s.g_ready;
+  const int ge = limbs ? tile_limbs(g, 0, n) : 0;
   if (!live) return;
   // the rows the sweep computes (upwind and tangential points; every point
   // for shallow water): Gy in the sweep's slot order, and the element
@@ -154,6 +242,22 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const double* Psh
   for (int j = t; j < nr; j += kStepT) {
     const int r = s.shared ? s.rows[j] : s.rowid[j * ne + e];
     double y0 = 0.0, gy = 0.0;
+    if (limbs) {
+      const long long* gx = reinterpret_cast<const long long*>(g) + lane;
+      Acc a(0);
+      for (int k2 = 0; k2 < s.KE; ++k2) {
+        const int2 c = s.Eyx.x[r * s.KE + k2];
+        a.mac(Cfx{c.x, c.y}, fx_limb(gx[s.ey_idx[r * s.KE + k2] * 32]));
+      }
+      s.Gy[j * ne + e] = ge == 0x7ff ? __hiloint2double(0x7ff80000, 0)
+                                     : fx_value(a.get(), ge - 1078 + s.Eyx.scale[r]);
+      if (want_y0) {
+        for (int k2 = 0; k2 < s.KE; ++k2)
+          y0 = fma(s.ey_val[r * s.KE + k2], s.u[s.ey_idx[r * s.KE + k2] * ne + e], y0);
+        s.Y[r * ne + e] = y0;
+      }
+      continue;
+    }
     if (want_y0) {
       for (int k2 = 0; k2 < s.KE; ++k2) {
         const double wv = s.ey_val[r * s.KE + k2];
@@ -177,39 +281,50 @@ struct FinalParams {
   const double* uhat;           // [2][Nqf][nface]
   const IterState* it;
   const double* G;
-  const double* H;
+  const double* H;              // per-element operator
+  FxOp Hx;                      // shared operator
   double* u;
 };
 
-// Hsh: a shared operator H [n][NQFS]; uh: [NQFS][32] scratch; src: the trace
+// Hsh: a shared operator's blocked limbs; uh: [NQFS][32] scratch; src: the trace
 // the last sweep read.
-__device__ __forceinline__ void final_tile(const FinalParams& p, const double* Hsh, double* uh,
+__device__ __forceinline__ void final_tile(const FinalParams& p, const int2* Hsh, double* uh,
                                            const double* src, int64_t tile) {
   const int lane = threadIdx.x, t = threadIdx.y;
   const int64_t ne = p.nel;
   const int64_t e = tile * 32 + lane;
   const bool live = e < ne;
   __syncthreads();
-  if (live) {
-    for (int f = 0; f < p.F; ++f) {
-      const int64_t face = p.elem_face[f * ne + e];
-      for (int g = t; g < p.Nqf; g += kStepT)
-        uh[(f * p.Nqf + g) * 32 + lane] = src[g * p.nface + face];
-    }
+  for (int f = 0; f < p.F; ++f) {
+    const int64_t face = live ? p.elem_face[f * ne + e] : 0;
+    for (int g = t; g < p.Nqf; g += kStepT)
+      uh[(f * p.Nqf + g) * 32 + lane] = live ? src[g * p.nface + face] : 0.0;
   }
   __syncthreads();
+  if (p.shared) {
+    const int em[3] = {tile_limbs(uh, 0, p.NQFS), 1, 1};
+    for (int b = t; b * 4 < p.n; b += kStepT) {
+      double g[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        g[i] = live && b * 4 + i < p.n ? p.G[(b * 4 + i) * ne + e] : 0.0;
+      double v[4];
+      tile_rows4(p.Hx, Hsh, uh, b, p.NQFS, 1, em, v);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = b * 4 + i;
+        if (r >= p.n || !live) break;
+        double acc = g[i] + v[i];
+        if (p.cn) acc = 2.0 * acc - p.u[r * ne + e];
+        p.u[r * ne + e] = acc;
+      }
+    }
+    return;
+  }
   if (!live) return;
   for (int r = t; r < p.n; r += kStepT) {
     double a0 = p.G[r * ne + e], a1 = 0.0;
-    if (p.shared) {
-      const double* Hr = Hsh + r * p.NQFS;
-      int c = 0;
-      for (; c + 1 < p.NQFS; c += 2) {
-        a0 = fma(Hr[c], uh[c * 32 + lane], a0);
-        a1 = fma(Hr[c + 1], uh[(c + 1) * 32 + lane], a1);
-      }
-      if (c < p.NQFS) a0 = fma(Hr[c], uh[c * 32 + lane], a0);
-    } else {
+    {
       const double* Hr = p.H + (int64_t)r * p.NQFS * ne + e;
       int c = 0;
       for (; c + 1 < p.NQFS; c += 2) {
