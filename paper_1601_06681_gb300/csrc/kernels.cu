@@ -841,101 +841,36 @@ struct FaceParams {
 };
 
 constexpr int kFaceBlock = 256;
-// one wave: 4 resident 256-thread blocks per SM; each thread strides over
-// several faces, so the reduction's adds are spread over more points
-constexpr int kFaceMaxBlocks = 608;
+constexpr int kFaceMaxBlocks = 608;   // one wave: 4 resident 256-thread blocks per SM
 
-// Grid: x strides over faces, y = face point. Block partials are reduced in a
-// fixed order by the last block to finish (deterministic).
+// A step's initial trace: the trace formula of u^n at every face point, in both
+// slots (points no sweep rewrites keep it). Grid: x strides over faces, y =
+// face point.
 __global__ void __launch_bounds__(kFaceBlock) k_face(const FaceParams p) {
-  __shared__ double red[kFaceBlock / 32];
-  __shared__ bool last;
-  const int64_t nface = p.geo.nface, nel = p.geo.nel;
-  const int64_t total = (int64_t)p.Nqf * nface;
-  const int gf = blockIdx.y;
-  // every block reads the counter before the last block advances it
-  const int kk = (p.mode == kFaceIterate) ? p.it->k : 0;
-  const double* uh_old = p.uhat + (int64_t)(kk & 1) * total + (int64_t)gf * nface;
-  double* uh_new = p.uhat + (int64_t)((p.mode == kFaceIterate ? kk + 1 : 0) & 1) * total +
-                   (int64_t)gf * nface;
-  const double wg = p.fw[gf];
-  const int64_t ym_off = (int64_t)gf * nel;   // + (local face * Nqf) * nel + elem
   // warm start: slot 0 holds the previous step's final trace, the trace
   // formula of u^n at every point but the inflow boundary ones, which
   // k_trace0_warm sets (every other point of slot 1 is written by the first
   // sweep before any sweep reads it)
-  if (p.mode != kFaceIterate && p.warm && *p.warm) return;
-  double acc = 0.0;
+  if (p.warm && *p.warm) return;
+  const int64_t nface = p.geo.nface, nel = p.geo.nel;
+  const int64_t total = (int64_t)p.Nqf * nface;
+  const int gf = blockIdx.y;
+  double* uh_new = p.uhat + (int64_t)gf * nface;
+  const int64_t ym_off = (int64_t)gf * nel;   // + (local face * Nqf) * nel + elem
   for (int64_t face = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; face < nface;
        face += (int64_t)gridDim.x * blockDim.x) {
-    const int em = p.geo.face_elem[face];
-    const int ep = p.geo.face_elem[nface + face];
-    const int fm = p.geo.face_local[face];
-    const int fpl = p.geo.face_local[nface + face];
     double uh;
     if (p.pde == EHDG_TRANSPORT) {
       uh = transport_trace_point(nel, nface, p.Nqf, p.cn, p.geo.face_elem, p.geo.face_local,
                                  p.sgn, p.Y, p.gb, p.gb_old, gf, face);
     } else {
+      const int em = p.geo.face_elem[face], ep = p.geo.face_elem[nface + face];
+      const int fm = p.geo.face_local[face], fpl = p.geo.face_local[nface + face];
       const double ym = p.Y[ym_off + (int64_t)fm * p.Nqf * nel + em];
       uh = (ep >= 0) ? ym + p.Y[ym_off + (int64_t)fpl * p.Nqf * nel + ep] : 2.0 * ym;
     }
-    if (p.mode == kFaceIterate) {
-      // the point weight wg is the block's; it multiplies the sum once below
-      const double d = uh - uh_old[face];
-      acc = fma(p.geo.face_jf[face] * d, d, acc);
-      if (p.R_out) p.R_out[(int64_t)gf * nface + face] = (float)d;
-    } else {
-      uh_new[total + face] = uh;     // both slots: points no sweep rewrites keep this value
-    }
+    uh_new[total + face] = uh;
     uh_new[face] = uh;
-  }
-  if (p.mode != kFaceIterate) return;
-
-  // deterministic reduction: warp -> block -> partials[block] -> last block
-  const unsigned int nblocks = gridDim.x * gridDim.y;
-  const unsigned int bid = blockIdx.y * gridDim.x + blockIdx.x;
-  acc = warp_sum(acc * wg);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = acc;
-  __syncthreads();
-  if (wid == 0) {
-    double v = (lane < (int)(blockDim.x >> 5)) ? red[lane] : 0.0;
-    v = warp_sum(v);
-    if (lane == 0) {
-      p.partials[bid] = v;
-      __threadfence();
-      const unsigned int ticket = atomicAdd(&p.it->counter, 1u);
-      last = (ticket == nblocks - 1);
-    }
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double v = 0.0;
-  for (unsigned int i = threadIdx.x; i < nblocks; i += blockDim.x)
-    v += reinterpret_cast<volatile double*>(p.partials)[i];
-  v = warp_sum(v);
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sum = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
-    const double r = p.res_scale * sqrt(sum);
-    IterState* it = p.it;
-    const int k = it->k;
-    if (k < p.max_iter) p.hist[k] = r;
-    it->k = k + 1;
-    it->r_last = r;
-    it->counter = 0u;
-    int cont = 1, status = EHDG_OK;
-    if (!isfinite(r)) { cont = 0; status = EHDG_ERR_DIVERGED; }
-    else if (r < p.tol) { cont = 0; status = EHDG_OK; }
-    else if (k + 1 >= p.max_iter) { cont = 0; status = EHDG_ERR_NOT_CONVERGED; }
-    it->cont = cont;
-    it->status = status;
-    __threadfence();
-    if (p.graph_mode) cudaGraphSetConditional(p.handle, (unsigned int)cont);
   }
 }
 
@@ -971,6 +906,104 @@ int face_launches(const Ctx& c, int mode) {
   return (mode == kFaceInitial && c.warm_ok && c.pde == EHDG_TRANSPORT && c.n_bface > 0) ? 2 : 1;
 }
 
+// The shallow-water trace update of an iteration, one thread per face: the
+// trace formula and the residual at its NQF points. The FP64 pipe bounds it
+// (k_face: four operations a point, 38 us at 512 x 512, p = 3, 0.69 of the
+// pipe), so the squares of faces with the same Jacobian are summed per point
+// index first and weighted once: three operations a point.
+template <int NQF>
+__global__ void __launch_bounds__(128) k_face_sw(const __grid_constant__ FaceParams p) {
+  __shared__ double red[4];
+  __shared__ bool last;
+  const int64_t nel = p.geo.nel, nface = p.geo.nface;
+  const int kk = p.it->k;                        // read before the last block advances it
+  const int64_t total = (int64_t)NQF * nface;
+  const double* old = p.uhat + (int64_t)(kk & 1) * total;
+  double* out = p.uhat + (int64_t)((kk + 1) & 1) * total;
+  double acc[NQF], res = 0.0, jf = 0.0;
+#pragma unroll
+  for (int g = 0; g < NQF; ++g) acc[g] = 0.0;
+  auto flush = [&] {
+    double s = 0.0;
+#pragma unroll
+    for (int g = 0; g < NQF; ++g) {
+      s = fma(p.fw[g], acc[g], s);
+      acc[g] = 0.0;
+    }
+    res = fma(jf, s, res);
+  };
+  for (int64_t face = blockIdx.x * 128LL + threadIdx.x; face < nface; face += gridDim.x * 128LL) {
+    const int em = p.geo.face_elem[face], ep = p.geo.face_elem[nface + face];
+    const int fm = p.geo.face_local[face], fp = p.geo.face_local[nface + face];
+    const double j = p.geo.face_jf[face];
+    const double* ym = p.Y + (int64_t)fm * NQF * nel + em;
+    const double* yp = ep >= 0 ? p.Y + (int64_t)fp * NQF * nel + ep : ym;   // wall: the mirror state
+    double a[NQF], b[NQF], o[NQF];
+#pragma unroll
+    for (int g = 0; g < NQF; ++g) {
+      a[g] = ym[g * nel];
+      b[g] = yp[g * nel];
+      o[g] = old[g * nface + face];
+    }
+    if (j != jf) {
+      flush();
+      jf = j;
+    }
+#pragma unroll
+    for (int g = 0; g < NQF; ++g) {
+      const double uh = a[g] + b[g], d = uh - o[g];
+      acc[g] = fma(d, d, acc[g]);
+      out[g * nface + face] = uh;
+      if (p.R_out) p.R_out[g * nface + face] = (float)d;
+    }
+  }
+  flush();
+  // deterministic reduction: warp -> block -> partials[block] -> last block
+  res = warp_sum(res);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane == 0) red[wid] = res;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    p.partials[blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
+    __threadfence();
+    last = atomicAdd(&p.it->counter, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double v = 0.0;
+  for (unsigned int i = threadIdx.x; i < gridDim.x; i += 128) v += __ldcg(p.partials + i);
+  v = warp_sum(v);
+  __syncthreads();
+  if (lane == 0) red[wid] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double r = p.res_scale * sqrt((red[0] + red[1]) + (red[2] + red[3]));
+    IterState* it = p.it;
+    const int k = it->k;
+    if (k < p.max_iter) p.hist[k] = r;
+    it->k = k + 1;
+    it->r_last = r;
+    it->counter = 0u;
+    int cont = 1, status = EHDG_OK;
+    if (!isfinite(r)) { cont = 0; status = EHDG_ERR_DIVERGED; }
+    else if (r < p.tol) { cont = 0; status = EHDG_OK; }
+    else if (k + 1 >= p.max_iter) { cont = 0; status = EHDG_ERR_NOT_CONVERGED; }
+    it->cont = cont;
+    it->status = status;
+    __threadfence();
+    if (p.graph_mode) cudaGraphSetConditional(p.handle, (unsigned int)cont);
+  }
+}
+
+template <int NQF>
+static cudaError_t launch_face_sw(const Ctx& c, const FaceParams& p) {
+  const int grid = std::min(persistent_grid(k_face_sw<NQF>, 128, 0, (c.nface + 127) / 128),
+                            c.n_partials);
+  k_face_sw<NQF><<<grid, 128, 0, c.stream>>>(p);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_face(Ctx& c, int mode, int graph_mode) {
   FaceParams p;
   p.graph_mode = graph_mode;
@@ -1002,6 +1035,16 @@ cudaError_t launch_face(Ctx& c, int mode, int graph_mode) {
   p.partials = c.partials;
   p.it = c.it;
   p.hist = c.hist;
+  if (mode == kFaceIterate) {
+    switch (c.Nqf) {   // shallow water, p <= 5 (transport sweeps write their own traces)
+      case 2: return launch_face_sw<2>(c, p);
+      case 3: return launch_face_sw<3>(c, p);
+      case 4: return launch_face_sw<4>(c, p);
+      case 5: return launch_face_sw<5>(c, p);
+      case 6: return launch_face_sw<6>(c, p);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   const dim3 grid(face_grid_x(c.nface, c.Nqf), c.Nqf);
   k_face<<<grid, kFaceBlock, 0, c.stream>>>(p);
   cudaError_t err = cudaGetLastError();
