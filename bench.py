@@ -1382,6 +1382,8 @@ def batch_variants(args, variants, tol, profile_loop=True):
             b.set_loop(False)
         elif opt == "persistent":
             b.set_loop("persistent")
+        elif opt == "":
+            b.set_loop(True)                          # the loop of launches
         setup = time.perf_counter() - t0
         inputs = start(b)
 

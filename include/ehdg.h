@@ -329,8 +329,10 @@ ehdg_status ehdg_batch_set_chains(ehdg_batch b, int k);
  * completes a stage of an instance (its FP64 sweep, a correction sweep, the
  * FP64 update) publishes the next stage's work items to a ring in device
  * memory, and every block takes the next item of the ring; waits on the ring
- * are bounded (a wait that gives up makes the step EHDG_ERR_TIMEOUT). The
- * graph is recaptured at the next run. EHDG_ERR_INVALID for a NULL batch or
+ * are bounded (a wait that gives up makes the step EHDG_ERR_TIMEOUT). Until
+ * this call or ehdg_batch_autotune_schedule chooses, a batch takes the
+ * persistent form where it applies and every looped instance is FP64, else the
+ * loop of launches. The graph is recaptured at the next run. EHDG_ERR_INVALID for a NULL batch or
  * a mode outside 0..2. */
 ehdg_status ehdg_batch_set_loop(ehdg_batch b, int on);
 /* Kernel accounting of the batched loop (a diagnostic; the paper has no

@@ -220,7 +220,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // One FP64 sweep of every instance that still iterates: items = (instance,
 // 128-element tile) from the lists; the instance's own single-problem tile
 // body, reduction and stopping test.
-__global__ void __launch_bounds__(kPeTile) k_batch_sweep(const BInst* inst, const int4* counts,
+// (five blocks per SM, 102 registers: 15.7 ms for the 48-instance mix, two at
+// the 250 registers of the unconstrained p = 6 body 18.0)
+__global__ void __launch_bounds__(kPeTile, 5) k_batch_sweep(const BInst* inst, const int4* counts,
                                                           int* lists, int n_inst,
                                                           unsigned int* ticket, int graph_mode,
                                                           cudaGraphConditionalHandle handle) {
@@ -826,10 +828,10 @@ __device__ __forceinline__ void q_corr_item(const BInst& I, const float* Hsh32, 
   lp_pe_tile<NQ, true>(v, Hsh32, tile);
 }
 
-// five resident blocks per SM (96 registers; four at the unconstrained 128):
-// the blocks spend much of an item at barriers while one thread takes the
-// next item or counts the stage, so more blocks keep the pipes busier
-__global__ void __launch_bounds__(kPeTile, 5) k_batch_persist(const BInst* inst, BQueue* q,
+// three resident blocks per SM (168 registers): 11.3 ms for a mix of 48 FP64
+// instances, 12.7 at five blocks, whose 96 registers spill 3 KB of the
+// fixed-point tile, 12.3 at two
+__global__ void __launch_bounds__(kPeTile, 3) k_batch_persist(const BInst* inst, BQueue* q,
                                                            long long* seq, int2* items,
                                                            int* stage_cnt, unsigned int limit) {
   __shared__ int2 s_item;

@@ -16,8 +16,11 @@ namespace ehdg {
 
 namespace {
 
+// three blocks per SM from p = 4 on, four below: 253 x 187, p = 4 (370 tiles)
+// then runs in one wave (6.75 ms for ten Crank-Nicolson steps; 7.74 at two
+// blocks, 6.95 at four, which spill)
 template <int NQ>
-__global__ void __launch_bounds__(kPeTile) k_sweep_pe(const __grid_constant__ PeView v,
+__global__ void __launch_bounds__(kPeTile, NQ >= 20 ? 3 : 4) k_sweep_pe(const __grid_constant__ PeView v,
                                                       const int2* Hx, int graph_mode,
                                                       cudaGraphConditionalHandle handle) {
   __shared__ __align__(16) int2 Hsh[NQ / 2 * NQ];
@@ -50,7 +53,7 @@ cudaError_t launch_pe_t(const PeView& v, const int2* Hx, int graph_mode,
 // about 3 us where a launch in the conditional graph loop costs 8: 16 x 16, p = 2
 // is all latency, and at 253 x 187, p = 4 it is a third of the iteration.
 template <int NQ>
-__global__ void __launch_bounds__(kPeTile) k_pe_persist(const __grid_constant__ PeView v,
+__global__ void __launch_bounds__(kPeTile, NQ >= 20 ? 3 : 4) k_pe_persist(const __grid_constant__ PeView v,
                                                         const int2* Hx) {
   __shared__ __align__(16) int2 Hsh[NQ / 2 * NQ];
   for (int i = threadIdx.x; i < NQ / 2 * NQ; i += kPeTile) Hsh[i] = Hx[i];
