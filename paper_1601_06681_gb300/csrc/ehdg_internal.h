@@ -117,7 +117,8 @@ struct Ctx {
   int64_t sweep_rows = 0;        // rows computed per sweep, all elements
   // per-element transport operator, tile-major (32 elements per tile): the
   // rows each tile needs, NQFS x 32 doubles each, streamed by the tiled sweep
-  double* Hyt = nullptr;
+  double* Hyt = nullptr;         // (limbs of the entries, fixed_point.cuh)
+  int16_t* row_scale = nullptr;   // [slot][nel] scale of each row
   int32_t* tile_row0 = nullptr;  // [ntiles] first row of a tile in Hyt
   uint8_t* tile_nrows = nullptr; // [ntiles] rows of a tile (max over its elements)
   int64_t ntiles = 0;

@@ -5,6 +5,12 @@
 // through a ring of shared-memory stages filled by cp.async.bulk, one
 // mbarrier per stage, every wait bounded.
 //
+// The rows are fixed-point limbs (fixed_point.cuh), 8 bytes an entry like the
+// doubles they come from, with one scale per row and element: their products
+// run on the integer pipe, aligned to the element's largest trace. In double
+// the FP64 pipe bounded the pass (58.7 us at 256 x 256, p = 4, with the 240 MB
+// it has to stream at 0.60 of the copy rate); now it takes 44.9 us, 0.79 of it.
+//
 // Ring bookkeeping: sequence number q holds row J0 + (q mod L), L = J1 - J0,
 // in stage q mod S and completes phase (q / S) & 1 of that stage's mbarrier.
 // q_done counts the sequence numbers consumed, qp the ones issued; a pass
@@ -16,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "ehdg_internal.h"
+#include "fixed_point.cuh"
 #include "tiled_common.cuh"
 
 namespace ehdg {
@@ -64,7 +71,8 @@ struct TiledParams {
   const int32_t* elem_face;      // [F][nel]
   const double* face_jf;
   double fw[kMaxQ * kMaxQ];
-  const double* Hyt;             // tile-major rows
+  const int2* Hyt;               // tile-major rows, limbs
+  const int16_t* row_scale;       // [slot][nel] their scales
   const int32_t* tile_row0;      // [ntiles] first row of each tile in Hyt
   const uint8_t* tile_nrows;     // [ntiles] rows of each tile
   double* uhat;                  // [2][Nqf][nface]
@@ -92,7 +100,7 @@ struct TiledParams {
 // read through L2 only (it is rewritten by other SMs during a persistent
 // launch). Returns false if a bounded wait gave up.
 template <int F, int NQF, bool CG>
-__device__ __forceinline__ bool sweep_pass(const TiledParams& p, double* stages, uint32_t mbar0,
+__device__ __forceinline__ bool sweep_pass(const TiledParams& p, int2* stages, uint32_t mbar0,
                                            int lane, int64_t gw, int64_t J0, int64_t J1,
                                            int64_t q0, int64_t& q_done, int64_t& qp,
                                            int64_t qp_end, const double* src, double* dst,
@@ -106,7 +114,9 @@ __device__ __forceinline__ bool sweep_pass(const TiledParams& p, double* stages,
   int nr_t = 0, nr_e = 0, nu_e = 0;
   int64_t e = 0;
   int fid[F];
-  double jf[F], u[NQ];
+  double jf[F];
+  Limb x[NQ];                                    // the element's traces, in units of 2^L
+  int em = 1;
   // per-tile values of tile t, loaded as soon as t is known (one row before
   // the warp enters the tile): face ids, row counts
   int fid_n[F], nr_e_n = 0, nu_e_n = 0, nr_t_n = 0;
@@ -124,10 +134,11 @@ __device__ __forceinline__ bool sweep_pass(const TiledParams& p, double* stages,
   // the next row's Gy value and point id are loaded one row ahead (slots
   // beyond an element's rows exist in both arrays and are never used)
   double gy_n = 0.0;
-  int rid_n = 0;
+  int rid_n = 0, sc_n = 0;
   if (t * 32 + lane < ne) {
     gy_n = p.Gy[(int64_t)j * ne + t * 32 + lane];
     rid_n = p.rowid[(int64_t)j * ne + t * 32 + lane];
+    sc_n = p.row_scale[(int64_t)j * ne + t * 32 + lane];
   }
   for (int64_t i = 0; i < L; ++i) {
     if (fresh) {
@@ -139,6 +150,8 @@ __device__ __forceinline__ bool sweep_pass(const TiledParams& p, double* stages,
       nu_e = nu_e_n;
 #pragma unroll
       for (int f = 0; f < F; ++f) fid[f] = fid_n[f];
+      double u[NQ];
+      em = 1;
 #pragma unroll
       for (int f = 0; f < F; ++f) {
         jf[f] = live ? p.face_jf[fid[f]] : 0.0;
@@ -146,14 +159,30 @@ __device__ __forceinline__ bool sweep_pass(const TiledParams& p, double* stages,
         for (int g = 0; g < NQF; ++g) {
           const double* a = src + (int64_t)g * nface + fid[f];
           u[f * NQF + g] = live ? (CG ? __ldcg(a) : *a) : 0.0;
+          em = max(em, fx_exponent(u[f * NQF + g]));
         }
       }
+#pragma unroll
+      for (int c = 0; c < NQ; ++c) x[c] = fx_split(fx_from_double(u[c], em));
       fresh = false;
     }
     const bool row_live = j < nr_e;
     const double gy = gy_n;
     const int rid = rid_n;
+    const int L2 = em - 1078 + sc_n;
     const int j_cur = j;
+    // the row's point and the trace there now, for the increment
+    const int rf = rid / NQF, rg = rid - rf * NQF;
+    int face = 0;
+    double jfv = 0.0, uk = 0.0;
+#pragma unroll
+    for (int q2 = 0; q2 < F; ++q2)
+      if (q2 == rf) {
+        face = fid[q2];
+        jfv = jf[q2];
+      }
+    const int64_t pt = (int64_t)rg * nface + face;
+    if (row_live) uk = CG ? __ldcg(src + pt) : src[pt];
     // advance to the next row (and tile) and start its Gy / point-id loads
     if (++j == nr_t) {
       j = 0;
@@ -166,6 +195,7 @@ __device__ __forceinline__ bool sweep_pass(const TiledParams& p, double* stages,
     if (i + 1 < L && t * 32 + lane < ne) {
       gy_n = p.Gy[(int64_t)j * ne + t * 32 + lane];
       rid_n = p.rowid[(int64_t)j * ne + t * 32 + lane];
+      sc_n = p.row_scale[(int64_t)j * ne + t * 32 + lane];
     }
 
     const int64_t q = q0 + i;
@@ -175,36 +205,22 @@ __device__ __forceinline__ bool sweep_pass(const TiledParams& p, double* stages,
       return false;
     }
     q_done = q + 1;
-    const double* Hs = stages + (size_t)st * NQ * 32;
-    double a[kCH];
-    a[0] = row_live ? gy : 0.0;
+    const int2* Hs = stages + (size_t)st * NQ * 32;
+    Acc a(0);
 #pragma unroll
-    for (int c2 = 1; c2 < kCH; ++c2) a[c2] = 0.0;
-#pragma unroll
-    for (int c = 0; c < NQ; ++c) a[c % kCH] = fma(Hs[c * 32 + lane], u[c], a[c % kCH]);
-    double acc = a[0];
-    if constexpr (kCH == 2) acc = a[0] + a[1];
-    if constexpr (kCH == 4) acc = (a[0] + a[1]) + (a[2] + a[3]);
+    for (int c = 0; c < NQ; ++c) {
+      const int2 h = Hs[c * 32 + lane];
+      a.mac(Cfx{h.x, h.y}, x[c]);
+    }
+    const double acc =
+        gy + (em == 0x7ff ? __hiloint2double(0x7ff80000, 0) : fx_value(a.get(), L2));
     __syncwarp();                                // every lane has read the stage
     ring_fill(p.Hyt, stages, mbar0, kTS, NQ, lane, J0, L, q_done, qp, qp_end);
     if (row_live) {
-      const int f = rid / NQF, g = rid - f * NQF;
-      int face = 0;
-      double jfv = 0.0, uk = 0.0;
-#pragma unroll
-      for (int q2 = 0; q2 < F; ++q2)
-        if (q2 == f) {
-          face = fid[q2];
-          jfv = jf[q2];
-        }
-#pragma unroll
-      for (int c = 0; c < NQ; ++c)
-        if (c == rid) uk = u[c];
       if (j_cur < nu_e) {
-        const int64_t pt = (int64_t)g * nface + face;
         dst[pt] = acc;
         const double d = acc - uk;
-        acc_res = fma(jfv * p.fw[g] * d, d, acc_res);
+        acc_res = fma(jfv * p.fw[rg] * d, d, acc_res);
         if (p.R_out) p.R_out[pt] = (float)d;
       } else {
         p.Y[(int64_t)rid * ne + e] = acc;

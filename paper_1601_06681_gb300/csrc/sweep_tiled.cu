@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(32 * kTW, (F * NQF <= 28) ? EHDG_TILED_MINB : 
   extern __shared__ __align__(256) unsigned char tsm[];
   __shared__ __align__(8) uint64_t mbar[kTW][kTS];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  double* stages = reinterpret_cast<double*>(tsm) + (size_t)w * kTS * NQ * 32;
+  int2* stages = reinterpret_cast<int2*>(tsm) + (size_t)w * kTS * NQ * 32;
   const uint32_t mbar0 = saddr(&mbar[w][0]);
   const int kk = p.it->k;                        // read before the last block advances it
   const int64_t tlen = (int64_t)NQF * p.nface;
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(32 * kTW, (F * NQF <= 28) ? EHDG_TILED_MINB : 
   __shared__ double s_r;
   __shared__ int s_cont, s_status;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  double* stages = reinterpret_cast<double*>(tsm) + (size_t)w * kTS * NQ * 32;
+  int2* stages = reinterpret_cast<int2*>(tsm) + (size_t)w * kTS * NQ * 32;
   const uint32_t mbar0 = saddr(&mbar[w][0]);
   const int k0 = p.it->k;
   const int64_t tlen = (int64_t)NQF * p.nface;
@@ -235,7 +235,8 @@ static void fill_params(Ctx& c, TiledParams& p, int graph_mode) {
   p.elem_face = c.geo.elem_face;
   p.face_jf = c.geo.face_jf;
   fill_face_weights(c, p.fw);
-  p.Hyt = c.Hyt;
+  p.Hyt = reinterpret_cast<const int2*>(c.Hyt);
+  p.row_scale = c.row_scale;
   p.tile_row0 = c.tile_row0;
   p.tile_nrows = c.tile_nrows;
   p.uhat = c.uhat;

@@ -225,6 +225,33 @@ __global__ void k_tile_hy(int64_t nel, int nq, int64_t ntiles, const int32_t* ti
   }
 }
 
+// The tile-major rows of the sweep to fixed-point limbs in place, entry =
+// 2^(scale - 56) (h 2^28 + l), one scale per row and element: the least with the
+// row's largest entry below 2 and its sum of magnitudes below 32 (so that its
+// products with 56-bit values sum below 2^62). One warp per row.
+__global__ void k_tile_limbs(int64_t nel, int nq, int64_t ntiles, const int32_t* tile_row0,
+                             const uint8_t* tile_nrows, double* Hyt, int16_t* row_scale) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; t < ntiles; t += nw) {
+    const int64_t e = t * 32 + lane;
+    for (int j = 0; j < tile_nrows[t]; ++j) {
+      double* row = Hyt + ((int64_t)tile_row0[t] + j) * nq * 32 + lane;
+      double mx = 0.0, sum = 0.0;
+      for (int c = 0; c < nq; ++c) {
+        mx = fmax(mx, fabs(row[c * 32]));
+        sum += fabs(row[c * 32]);
+      }
+      const int s = mx > 0.0 ? max(ilogb(mx), ilogb(sum) + 1 - 5) : 0;
+      if (e < nel) row_scale[(int64_t)j * nel + e] = (int16_t)s;
+      for (int c = 0; c < nq; ++c) {
+        const Limb l = fx_split(__double2ll_rn(scalbn(row[c * 32], 56 - s)));
+        reinterpret_cast<int2*>(row)[c * 32] = make_int2(l.h, l.l);
+      }
+    }
+  }
+}
+
 template <int F, int NQF>
 cudaError_t final_config(int64_t total_rows, int64_t ntiles, int* grid, size_t* smem_out) {
   return tiled_shape_of(k_final_tiled<F, NQF>, F * NQF, total_rows, ntiles, grid, smem_out);
@@ -384,7 +411,12 @@ cudaError_t build_tiled_operator(Ctx& c) {
                           cudaMemcpyHostToDevice)) != cudaSuccess)
       return err;
   }
-  return cudaSuccess;
+  // last, since the low-precision copies are rounded from the doubles
+  if ((err = dalloc_raw(c, (void**)&c.row_scale, sizeof(int16_t) * c.NQFS * c.nel)) != cudaSuccess)
+    return err;
+  k_tile_limbs<<<152 * 8, 128, 0, c.stream>>>(c.nel, c.NQFS, ntiles, c.tile_row0, c.tile_nrows,
+                                              c.Hyt, c.row_scale);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_lp_sweep_tiled(Ctx& c, const float* in, float* out) {

@@ -13,15 +13,12 @@ namespace ehdg {
 namespace {
 
 // compile-time tuning: warps per block (independent of each other), stages
-// per warp, independent FMA chains per row
+// per warp
 #ifndef EHDG_TILED_TW
 #define EHDG_TILED_TW 4
 #endif
 #ifndef EHDG_TILED_TS
 #define EHDG_TILED_TS 2
-#endif
-#ifndef EHDG_TILED_CH
-#define EHDG_TILED_CH 1
 #endif
 // minimum resident blocks per SM asked of the compiler (instances with up
 // to 28 face points per element)
@@ -30,8 +27,6 @@ namespace {
 #endif
 constexpr int kTW = EHDG_TILED_TW;
 constexpr int kTS = EHDG_TILED_TS;
-constexpr int kCH = EHDG_TILED_CH;
-static_assert(kCH == 1 || kCH == 2 || kCH == 4, "FMA chains per row: 1, 2 or 4");
 constexpr uint32_t kTileWaitLimit = 1u << 22; // mbarrier polls before giving up
 constexpr uint32_t kBarrierPolls = 1u << 22;  // grid-barrier polls before giving up
 constexpr int kTiledMaxBlocks = 4096;         // same bound as the other transport sweep
