@@ -76,8 +76,11 @@ typedef enum { EHDG_BE = 0, EHDG_CN = 1, EHDG_STEADY = 2 } ehdg_scheme;
  * equation delta = R + S H delta and the FP64 update uhat += delta; the fixed
  * point and the stopping rule are those of the FP64 iteration. MIXED_FP32 uses
  * float32 operands and accumulation on the CUDA cores.
- * FP64_EMULATED: every sweep FP64-accurate, with the element products on the
- * BF16 tensor cores by the Ozaki splitting -- each element's traces and each
+ * FP64_EMULATED: every sweep FP64-accurate without the FP64 pipe's products:
+ * in fixed point on the integer pipe where that form exists (as EHDG_FP64
+ * there: transport on quadrilaterals and hexahedra without a beta.n = 0 point,
+ * shallow water), otherwise on the BF16 tensor cores by the Ozaki splitting
+ * -- each element's traces and each
  * operator row in 49-bit fixed point against their largest exponent, split
  * into seven 7-bit digits whose products are summed exactly (integers below
  * 2^24 in FP32 accumulators) and recombined in 64-bit integers; the trace
@@ -142,10 +145,10 @@ typedef struct {
   double coriolis_ym;
   double friction;
   /* MIXED_* precisions: nonzero runs the outer FP64 sweeps (the FP64
-   * residual R and the convergence test) as FP64_EMULATED sweeps on the BF16
-   * tensor cores, under the same conditions as FP64_EMULATED (otherwise
-   * ehdg_create returns EHDG_ERR_UNSUPPORTED). Zero: DFMA sweeps. Ignored by
-   * FP64 and FP64_EMULATED. */
+   * residual R and the convergence test) as FP64_EMULATED sweeps (on the BF16
+   * tensor cores for hexahedra), under the same conditions as FP64_EMULATED
+   * (otherwise ehdg_create returns EHDG_ERR_UNSUPPORTED). Zero: the sweeps of
+   * EHDG_FP64. Ignored by FP64 and FP64_EMULATED. */
   int emulated_outer;
 } ehdg_problem_desc;
 
@@ -259,11 +262,9 @@ ehdg_status ehdg_autotune_inner_sweeps(ehdg_ctx ctx, const int* candidates, int 
                                        int* best, double* best_ms);
 /* Autotuner for the FP64 path of a context that has both (FP64_EMULATED, or a
  * MIXED_* precision with emulated_outer): runs one implicit step from the
- * current state with the DFMA kernels and one with the tensor-core kernels
- * (restoring the state after each), keeps the faster, and reports both times;
- * the state is left as it was. Both paths are FP64-accurate; the tensor cores
- * pay on large shared-operator problems, the DFMA kernels on small ones (a
- * tensor-core launch has a fixed setup). A batch recaptures its graph after
+ * current state with the kernels of EHDG_FP64 and one with the tensor-core
+ * kernels (restoring the state after each), keeps the faster, and reports both
+ * times; the state is left as it was. Both paths are FP64-accurate. A batch recaptures its graph after
  * an instance's path changed. EHDG_ERR_INVALID for a context without the
  * tensor-core path. The paper has no counterpart. */
 ehdg_status ehdg_autotune_fp64_path(ehdg_ctx ctx, int* tensor_cores, double* ms_dfma,

@@ -1076,6 +1076,13 @@ ehdg_status ehdg_create(const ehdg_mesh_desc* mesh, const ehdg_problem_desc* pro
     CKC(cudaStreamSynchronize(c.stream));
     c.use_pe = true;
   }
+  // The tensor-core products stay where no fixed-point form exists (mixed
+  // precision on hexahedra, beta.n = 0 points). Elsewhere fixed point is at least
+  // as accurate (2^-56 of the largest value against 2^-49) and faster: 37 x 29 x
+  // 31 hexahedra, p = 3: 51 against 65 us per iteration, 64^3: 243 against 297 a
+  // sweep; shallow water, 512 x 512, p = 3: 46 against 66 us of element values.
+  // ehdg_autotune_fp64_path still compares the two.
+  if (c.use_pe || c.md || c.pde == EHDG_SW_LINEAR) c.use_ozaki = false;
   // their persistent forms launch resident blocks only
   if (c.use_pe || c.md) c.persist_fits = true;
   if (c.shared_op) {

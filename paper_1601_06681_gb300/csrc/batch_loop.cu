@@ -1027,7 +1027,7 @@ __global__ void __launch_bounds__(32 * kStepT) k_batch_step(const BInst* inst, c
       for (int k = tid; k < fx_blocked(I.n, I.n); k += 32 * kStepT) Psh[k] = I.Px.x[k];
       cur = i;
     }
-    step_tile(step_params(I), Psh, w, g, nullptr, it - pre[i]);
+    step_tile<true>(step_params(I), Psh, w, g, nullptr, it - pre[i]);
   }
 }
 

@@ -482,11 +482,12 @@ cudaError_t build_fx_operators(Ctx& c) {
 // (threadIdx.y); persistent over tiles. w and G of the tile live in shared
 // memory; a shared operator P is staged once per block. The tile body is in
 // step_tiles.cuh (the batched loop runs it too).
+template <bool SHARED>
 __global__ void __launch_bounds__(32 * kStepT) k_step(const __grid_constant__ StepParams s) {
   extern __shared__ __align__(16) double sm[];
   const int lane = threadIdx.x, t = threadIdx.y, tid = t * 32 + lane;
   const int n = s.n;
-  const int64_t np = s.shared && !s.g_ready ? fx_blocked(n, n) : 0;
+  const int64_t np = SHARED && !s.g_ready ? fx_blocked(n, n) : 0;
   int2* Psh = reinterpret_cast<int2*>(sm);            // the shared operator's limbs
   double* w = sm + np;                                // [n][32]
   double* g = w + n * 32;                             // [n][32]
@@ -494,7 +495,7 @@ __global__ void __launch_bounds__(32 * kStepT) k_step(const __grid_constant__ St
   for (int64_t i = tid; i < np; i += 32 * kStepT) Psh[i] = s.Px.x[i];
   const int64_t ntiles = (s.nel + 31) / 32;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-    step_tile(s, Psh, w, g, sfw, tile);
+    step_tile<SHARED>(s, Psh, w, g, sfw, tile);
 }
 
 // The sum-factorised face-point pass of the step (hexahedra, one shared
@@ -570,10 +571,11 @@ cudaError_t launch_step(Ctx& c) {
       sizeof(double) * ((s.shared && !s.g_ready ? (size_t)fx_blocked(c.n, c.n) : 0) +
                         2 * (size_t)c.n * 32 +
                         (s.sf_ey ? (size_t)s.sf_nf * s.sf_p1 * s.sf_p1 * 2 * 32 : 0));
-  cudaError_t err = fn_smem((const void*)k_step, smem);
+  auto kern = s.shared ? k_step<true> : k_step<false>;
+  cudaError_t err = fn_smem((const void*)kern, smem);
   if (err != cudaSuccess) return err;
-  const int grid = persistent_grid(k_step, 32 * kStepT, smem, (c.nel + 31) / 32);
-  k_step<<<grid, dim3(32, kStepT), smem, c.stream>>>(s);
+  const int grid = persistent_grid(kern, 32 * kStepT, smem, (c.nel + 31) / 32);
+  kern<<<grid, dim3(32, kStepT), smem, c.stream>>>(s);
   return cudaGetLastError();
 }
 

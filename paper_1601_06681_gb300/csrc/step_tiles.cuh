@@ -121,6 +121,7 @@ __device__ __forceinline__ void tile_rows4(const FxOp& op, const int2* osh, cons
 
 // Psh: a shared operator's blocked limbs; w, g: [n][32] scratch; sfw: the face
 // passes' scratch [sf_nf q][p+1][2][32] (sf_ey only).
+template <bool SHARED>
 __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, double* w,
                                           double* g, double* sfw, int64_t tile) {
   const int lane = threadIdx.x, t = threadIdx.y;
@@ -136,17 +137,17 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
     for (int c = t; c < n; c += kStepT) {
       double v = 0.0;
       if (live) {
-        v = s.shared ? (s.ucoef != 0.0 ? s.u[c * ne + e] : 0.0) : s.u[c * ne + e] * s.ucoef;
+        v = SHARED ? (s.ucoef != 0.0 ? s.u[c * ne + e] : 0.0) : s.u[c * ne + e] * s.ucoef;
         if (s.have_force) {
           const double f = s.force_avg ? 0.5 * (s.force[c * ne + e] + s.force_old[c * ne + e])
                                        : s.force[c * ne + e];
-          v = s.shared ? fma(s.fcoef, f, v) : v + f;
+          v = SHARED ? fma(s.fcoef, f, v) : v + f;
         }
       }
       w[c * 32 + lane] = v;
     }
     __syncthreads();
-    if (s.shared) {
+    if (SHARED) {
       const int np = n / s.nf;
       int em[3] = {1, 1, 1};
 #pragma unroll
@@ -164,7 +165,7 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
         }
       }
     }
-    for (int r = t; r < (s.shared ? 0 : n); r += kStepT) {
+    for (int r = t; r < (SHARED ? 0 : n); r += kStepT) {
       double a0 = 0.0, a1 = 0.0;
       if (live) {
         const double* Pr = s.P + (int64_t)r * n * ne + e;
@@ -231,16 +232,16 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
     }
     return;
   }
-  const bool limbs = s.shared && !s.g_ready;
+  const bool limbs = SHARED && !s.g_ready;
   const int ge = limbs ? tile_limbs(g, 0, n) : 0;
   if (!live) return;
   // the rows the sweep computes (upwind and tangential points; every point
   // for shallow water): Gy in the sweep's slot order, and the element
   // values Y0 = Ey u^n there, which are all the initial trace reads (it
   // takes the upwind side, or both sides of a tangential point)
-  const int nr = s.shared ? s.n_rows : s.nrows[e];
+  const int nr = SHARED ? s.n_rows : s.nrows[e];
   for (int j = t; j < nr; j += kStepT) {
-    const int r = s.shared ? s.rows[j] : s.rowid[j * ne + e];
+    const int r = SHARED ? s.rows[j] : s.rowid[j * ne + e];
     double y0 = 0.0, gy = 0.0;
     if (limbs) {
       const long long* gx = reinterpret_cast<const long long*>(g) + lane;

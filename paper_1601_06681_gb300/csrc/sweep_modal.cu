@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
         xi[u] = fx_split(ok ? ai(fx_ld<PERSIST>(src + g * nface, fi[0])) : 0);
         xo[u] = fx_split(ok ? ao(fx_ld<PERSIST>(src + g * nface, fo[0])) : 0);
       }
-#pragma unroll 1
+#pragma unroll (SOLO || P1 == 4 ? 1 : P1)
       for (int i = 0; i < P1; ++i) {
         const int by = S::group(i) + 2 * K, bz = S::group(i) + 2 * J;
         const Align yi(L, fx_field(ei[1], by)), yo(L, fx_field(eo[1], by));
@@ -948,10 +948,10 @@ bool md_1d(const Ref1D& R, Md1D* o) {
   // real eigenvalues in [0, 64) by bisection on the sign of det(D - x I), in
   // decreasing order; their real parts lie in (0, 36] for p <= 6
   std::vector<ld> lam;
-  const int steps = 4096;
+  const int steps = 512;
   ld x1 = 64.0L, d1 = det_shift(n, D, x1);
   for (int s = steps - 1; s >= 0 && (int)lam.size() <= nr; --s) {
-    // an irrational offset keeps the grid off the eigenvalues
+    // the offset keeps the grid off the eigenvalues, which are over 1 apart
     const ld x0 = 64.0L * s / steps + 0.00312345L, d0 = det_shift(n, D, x0);
     if ((d0 > 0) != (d1 > 0)) {
       ld a = x0, b = x1;
