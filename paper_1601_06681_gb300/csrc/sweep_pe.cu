@@ -50,8 +50,8 @@ cudaError_t launch_pe_t(const PeView& v, const int2* Hx, int graph_mode,
 // All iterations of a step in one cooperative launch: one pass over the tiles
 // per iteration, the same tile code and residual sum as k_sweep_pe (so the same
 // iterates and decisions bit for bit), traces read through L2. A pass ends for
-// about 3 us where a launch in the conditional graph loop costs 8: 16 x 16, p = 2
-// is all latency, and at 253 x 187, p = 4 it is a third of the iteration.
+// about 3 us where a launch in the conditional graph loop costs 8. Taken by
+// meshes with more tiles than resident blocks; k_pe_resident has the others.
 template <int NQ>
 __global__ void __launch_bounds__(kPeTile, NQ >= 20 ? 3 : 4) k_pe_persist(const __grid_constant__ PeView v,
                                                         const int2* Hx) {
@@ -80,12 +80,200 @@ __global__ void __launch_bounds__(kPeTile, NQ >= 20 ? 3 : 4) k_pe_persist(const 
   }
 }
 
+// the barrier of a cluster's threads (all of them, every time), with release
+// and acquire at cluster scope
+__device__ __forceinline__ void pe_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
+// *p = x in the shared memory of block `rank` of the cluster
+__device__ __forceinline__ void pe_cluster_store(double* p, int rank, double x) {
+  asm volatile(
+      "{\n .reg .b32 a;\n mapa.shared::cluster.u32 a, %0, %1;\n st.shared::cluster.f64 [a], %2;\n}\n" ::
+          "r"((uint32_t)__cvta_generic_to_shared(p)),
+      "r"(rank), "d"(x)
+      : "memory");
+}
+
+// The same where every tile has a block of its own: what does not change
+// between passes (face ids, Gy, weights, Jacobians) stays in registers, and so
+// do the traces on the element's outflow faces, which its own thread wrote; a
+// pass loads the NQ / 2 inflow values in one round through L2. The operator's
+// columns are staged in the order outflow, inflow.
+//
+// CL: the grid is one cluster (up to kPeCluster tiles). Its hardware barrier
+// ends a pass, every block holds all partial sums in shared memory and decides
+// for itself: such a mesh is all latency, and the counter and the polled word
+// in L2 cost more than the pass. 16 x 16, p = 2, 10 steps: 2.62 -> 1.42 ms with
+// the cluster; 253 x 187, p = 4 with a block per tile 6.96 -> 6.38. The sums are those of pe_total, so iterates,
+// residuals and decisions are bit for bit the same in every form.
+constexpr int kPeCluster = 16;
+
+template <int NQ, bool CL>
+__global__ void __launch_bounds__(kPeTile, CL ? 1 : (NQ >= 20 ? 3 : 4))
+    k_pe_resident(const __grid_constant__ PeView v, const int2* Hx) {
+  constexpr int NQF = NQ / 4, RN = NQ / 2;
+  __shared__ __align__(16) int2 Hsh[RN * NQ];
+  __shared__ double red[kPeTile / 32];
+  __shared__ double parts[CL ? 2 : 1][CL ? kPeCluster : 1];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int i = tid; i < RN * NQ; i += kPeTile) {
+    const int j = i / NQ, c = i - j * NQ, b = c / NQF;
+    const int f = b < 2 ? v.own[b] : v.own[b - 2] ^ 1;
+    Hsh[i] = Hx[j * NQ + f * NQF + c - b * NQF];
+  }
+  const int ntiles = (int)gridDim.x;
+  const int64_t ne = v.nel, nface = v.nface, tlen = (int64_t)NQF * nface;
+  const int64_t e = (int64_t)blockIdx.x * kPeTile + tid;
+  const bool live = e < ne;
+  int k = v.it->k;
+  double uo[RN], gy[RN], w[NQF], jf[2] = {0.0, 0.0};
+  int64_t fo[2] = {0, 0}, fi[2] = {0, 0};
+  int eg = 1;
+  const int hs = *v.hs;
+#pragma unroll
+  for (int g = 0; g < NQF; ++g) w[g] = v.fw[g];
+#pragma unroll
+  for (int b = 0; b < 2; ++b) {
+    if (live) {
+      fo[b] = v.elem_face[v.own[b] * ne + e];
+      fi[b] = v.elem_face[(v.own[b] ^ 1) * ne + e];
+      jf[b] = v.face_jf[fo[b]];
+    }
+#pragma unroll
+    for (int g = 0; g < NQF; ++g) {
+      gy[b * NQF + g] = live ? v.Gy[(b * NQF + g) * ne + e] : 0.0;
+      uo[b * NQF + g] = live ? v.uhat_slot(k & 1, tlen)[g * nface + fo[b]] : 0.0;
+      eg = max(eg, fx_exponent(gy[b * NQF + g]));
+    }
+  }
+  __syncthreads();
+  // (a block's shared memory is written by the others once all have started)
+  if (CL) pe_cluster_sync();
+  for (unsigned int pass = 0;; ++pass, ++k) {
+    const double* src = v.uhat_slot(k & 1, tlen);
+    double* dst = const_cast<double*>(v.uhat_slot((k + 1) & 1, tlen));
+    double res = 0.0;
+    if (live) {
+      double ui[RN];
+#pragma unroll
+      for (int j = 0; j < RN; ++j) ui[j] = __ldcg(src + (j % NQF) * nface + fi[j / NQF]);
+      int emax = eg;
+#pragma unroll
+      for (int j = 0; j < RN; ++j) emax = max(emax, fx_exponent(uo[j]));
+#pragma unroll
+      for (int j = 0; j < RN; ++j) emax = max(emax, fx_exponent(ui[j]));
+      Limb x[NQ];
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {
+        x[j] = fx_split(fx_from_double(uo[j], emax));
+        x[RN + j] = fx_split(fx_from_double(ui[j], emax));
+      }
+      double sq[2] = {0.0, 0.0};
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {
+        const int4* Hr = reinterpret_cast<const int4*>(Hsh + j * NQ);
+        Acc t(fx_from_double(gy[j], emax + hs));
+#pragma unroll
+        for (int c = 0; c < NQ; c += 2) {
+          const int4 h = Hr[c / 2];
+          t.mac(Cfx{h.x, h.y}, x[c]);
+          t.mac(Cfx{h.z, h.w}, x[c + 1]);
+        }
+        double acc = fx_value(t.get(), emax - 1078 + hs);
+        if (emax == 0x7ff) acc = __hiloint2double(0x7ff80000, 0);
+        const int b = j / NQF, g = j - b * NQF;
+        const double d = acc - uo[j];
+        dst[g * nface + fo[b]] = acc;
+        uo[j] = acc;
+        sq[b] = fma(w[g], d * d, sq[b]);
+      }
+      res = fma(jf[0], sq[0], jf[1] * sq[1]);
+    }
+    res = fsum_warp(res);
+    if (lane == 0) red[wid] = res;
+    __syncthreads();
+    if (!CL) {
+      if (tid == 0) {
+        double s = 0.0;
+#pragma unroll
+        for (int i = 0; i < kPeTile / 32; ++i) s += red[i];
+        v.partials[blockIdx.x] = s;
+      }
+      const int state = pass_end(v.it, gridDim.x, pass, v.hist, v.max_iter, v.tol, v.res_scale,
+                                 [&] { return tid < 32 ? pe_total(v.partials, ntiles) : 0.0; });
+      if (state == 1) continue;
+      if (state == 0 && tid == 0) {
+        v.it->status = EHDG_ERR_TIMEOUT;
+        v.it->cont = 0;
+      }
+      return;
+    }
+    double* mine = &parts[CL ? pass & 1 : 0][CL ? blockIdx.x : 0];
+    if (tid < ntiles) {
+      double s = 0.0;
+#pragma unroll
+      for (int i = 0; i < kPeTile / 32; ++i) s += red[i];
+      pe_cluster_store(mine, tid, s);
+    }
+    pe_cluster_sync();
+    const double r =
+        v.res_scale * sqrt(fsum_warp(lane < ntiles ? parts[CL ? pass & 1 : 0][CL ? lane : 0] : 0.0));
+    int cont = 1, status = EHDG_OK;
+    if (!isfinite(r)) { cont = 0; status = EHDG_ERR_DIVERGED; }
+    else if (r < v.tol) { cont = 0; status = EHDG_OK; }
+    else if (k + 1 >= v.max_iter) { cont = 0; status = EHDG_ERR_NOT_CONVERGED; }
+    if (blockIdx.x == 0 && tid == 0) {
+      if (k < v.max_iter) v.hist[k] = r;
+      if (!cont) {
+        v.it->k = k + 1;
+        v.it->r_last = r;
+        v.it->status = status;
+        v.it->cont = 0;
+      }
+    }
+    if (!cont) return;
+  }
+}
+
+// One cluster of all tiles, where the device takes a cluster of that size.
+template <int NQ>
+cudaError_t launch_pe_cluster_t(const PeView& v, const int2* Hx, int ntiles, cudaStream_t s) {
+  cudaError_t e = ntiles > 8 ? cudaFuncSetAttribute((const void*)k_pe_resident<NQ, true>,
+                                                    cudaFuncAttributeNonPortableClusterSizeAllowed, 1)
+                             : cudaSuccess;
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned int)ntiles;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned int)ntiles);
+  cfg.blockDim = dim3(kPeTile);
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int fits = 0;
+  e = cudaOccupancyMaxActiveClusters(&fits, k_pe_resident<NQ, true>, &cfg);
+  if (e != cudaSuccess) return e;
+  if (fits < 1) return cudaErrorLaunchOutOfResources;
+  return cudaLaunchKernelEx(&cfg, k_pe_resident<NQ, true>, v, Hx);
+}
+
 template <int NQ>
 cudaError_t launch_pe_persist_t(const PeView& v, const int2* Hx, cudaStream_t s) {
-  const int bpsm = fn_blocks_per_sm((const void*)k_pe_persist<NQ>, kPeTile, 0);
   const int64_t ntiles = (v.nel + kPeTile - 1) / kPeTile;
-  const int grid = (int)std::min<int64_t>((int64_t)bpsm * device_sms(), ntiles);
+  if (ntiles <= kPeCluster) {
+    if (launch_pe_cluster_t<NQ>(v, Hx, (int)ntiles, s) == cudaSuccess) return cudaSuccess;
+    cudaGetLastError();
+  }
   void* args[] = {const_cast<PeView*>(&v), &Hx};
+  const void* resident = (const void*)k_pe_resident<NQ, false>;
+  if (ntiles <= (int64_t)fn_blocks_per_sm(resident, kPeTile, 0) * device_sms())
+    return cudaLaunchCooperativeKernel(resident, dim3((unsigned int)ntiles), dim3(kPeTile), args, 0,
+                                       s);
+  const int bpsm = fn_blocks_per_sm((const void*)k_pe_persist<NQ>, kPeTile, 0);
+  const int grid = (int)std::min<int64_t>((int64_t)bpsm * device_sms(), ntiles);
   return cudaLaunchCooperativeKernel((const void*)k_pe_persist<NQ>, dim3(grid), dim3(kPeTile),
                                      args, 0, s);
 }
