@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "dependent_launch.cuh"
 #include "ehdg_internal.h"
 #include "sweep_pass.cuh"
 #include "tiled_common.cuh"
@@ -95,7 +96,10 @@ __device__ __forceinline__ bool lp_pass(const LpTParams& p, T* stages, uint32_t 
   const T* rows = static_cast<const T*>(p.Hyt_lp);
   const int64_t ne = p.nel, nface = p.nface;
   const int64_t L = J1 - J0;
-  if (L <= 0) return true;
+  if (L <= 0) {
+    dep_wait();
+    return true;
+  }
   auto ptid_at = [&](const RowPos& r) -> int {
     const int64_t ee = r.t * 32 + lane;
     return (r.t < p.ntiles && ee < ne) ? p.ptid[(int64_t)r.j * ne + ee] : 0;
@@ -110,14 +114,18 @@ __device__ __forceinline__ bool lp_pass(const LpTParams& p, T* stages, uint32_t 
   rowpos_next(p, ahead2);
   int pt_cur = ptid_at(cur);
   int pt_nxt = L > 1 ? ptid_at(ahead1) : 0;
-  float rv_cur = CG ? __ldcg(p.R + pt_cur) : p.R[pt_cur];
   int nr_e = 0, nu_e = 0;
   int64_t e = 0, t_gathered = -1;
   float d[NQ];
   // face ids of the tile the next row enters, loaded a row early
   int fid_n[F];
-  int64_t fid_tile = -1;
+  int64_t fid_tile = cur.t;
+#pragma unroll
+  for (int f = 0; f < F; ++f)
+    fid_n[f] = cur.t * 32 + lane < ne ? p.elem_face[(int64_t)f * ne + cur.t * 32 + lane] : 0;
   int rid_n = (cur.t * 32 + lane < ne) ? p.rowid[(int64_t)cur.j * ne + cur.t * 32 + lane] : 0;
+  dep_wait();                                    // R and the correction from here on
+  float rv_cur = CG ? __ldcg(p.R + pt_cur) : p.R[pt_cur];
   for (int64_t i = 0; i < L; ++i) {
     if (cur.t != t_gathered) {
       // the tile's correction values at each element's face points

@@ -14,6 +14,7 @@
 // operator is kept as an FP32 copy of Hy in the sweep's slot layout.
 #include <cuda_runtime.h>
 
+#include "dependent_launch.cuh"
 #include "ehdg_internal.h"
 
 namespace ehdg {
@@ -183,6 +184,8 @@ __global__ void k_face_lp_sw(int64_t nel, int64_t nface, int Nqf, const int32_t*
 
 // uhat <- uhat + delta in FP64: slot K&1 = slot (K+1)&1 + delta, K = it->k
 __global__ void k_apply(int64_t total, const IterState* it, double* uhat, const float* delta) {
+  dep_trigger();
+  dep_wait();
   const int K = it->k;
   double* dst = uhat + (int64_t)(K & 1) * total;
   const double* src = uhat + (int64_t)((K + 1) & 1) * total;
@@ -313,8 +316,8 @@ cudaError_t launch_lp_sweep(Ctx& c, const float* in, float* out, bool fuse_apply
 
 cudaError_t launch_apply(Ctx& c, const float* delta) {
   const int64_t total = (int64_t)c.Nqf * c.nface;
-  k_apply<<<grid1d(total, 256, 152 * 16), 256, 0, c.stream>>>(total, c.it, c.uhat, delta);
-  return cudaGetLastError();
+  return launch_dependent(k_apply, dim3(grid1d(total, 256, 152 * 16)), dim3(256), 0, c.stream, total,
+                          c.it, c.uhat, delta);
 }
 
 // Kernels of one low-precision sweep (the element kernel plus the trace

@@ -22,6 +22,7 @@
 // block waits (bounded again) for its copies still in flight before it ends.
 #include <cuda_runtime.h>
 
+#include "dependent_launch.cuh"
 #include "ehdg_internal.h"
 #include "sweep_common.cuh"
 #include "tiled_common.cuh"
@@ -42,15 +43,17 @@ __global__ void __launch_bounds__(32 * kTW, (F * NQF <= 28) ? EHDG_TILED_MINB : 
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int2* stages = reinterpret_cast<int2*>(tsm) + (size_t)w * kTS * NQ * 32;
   const uint32_t mbar0 = saddr(&mbar[w][0]);
-  const int kk = p.it->k;                        // read before the last block advances it
-  const int64_t tlen = (int64_t)NQF * p.nface;
-  const double* src = p.uhat + (int64_t)(kk & 1) * tlen;
-  double* dst = p.uhat + (int64_t)((kk + 1) & 1) * tlen;
+  dep_trigger();
   const int64_t nwarps = (int64_t)gridDim.x * kTW, gw = (int64_t)blockIdx.x * kTW + w;
   const int64_t J0 = p.total_rows * gw / nwarps, J1 = p.total_rows * (gw + 1) / nwarps;
   int64_t qp = 0, q_done = 0;
   ring_init(mbar0, kTS, lane);
   ring_fill(p.Hyt, stages, mbar0, kTS, NQ, lane, J0, J1 - J0, 0, qp, J1 - J0);
+  dep_wait();
+  const int kk = p.it->k;                        // read before the last block advances it
+  const int64_t tlen = (int64_t)NQF * p.nface;
+  const double* src = p.uhat + (int64_t)(kk & 1) * tlen;
+  double* dst = p.uhat + (int64_t)((kk + 1) & 1) * tlen;
   double acc_res = 0.0;
   sweep_pass<F, NQF, false>(p, stages, mbar0, lane, gw, J0, J1, 0, q_done, qp, J1 - J0, src, dst,
                             acc_res);
@@ -160,8 +163,7 @@ cudaError_t tiled_config(int64_t total_rows, int64_t ntiles, int* grid, size_t* 
 
 template <int F, int NQF>
 cudaError_t tiled_launch(const TiledParams& p, int grid, size_t smem, cudaStream_t s) {
-  k_sweep_tiled<F, NQF><<<grid, 32 * kTW, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_dependent(k_sweep_tiled<F, NQF>, dim3(grid), dim3(32 * kTW), smem, s, p);
 }
 
 // blocks of the persistent kernel that fit on one SM (0 on error)

@@ -112,7 +112,8 @@ __device__ __forceinline__ void fx_tile(const TcFxParams& p, unsigned char* As, 
   const int64_t e = tile * kFxM + row;
   const bool live = e < ne;
   const uint32_t nface = p.nface;
-  // every load of the tile first: R at the owned points, then the K range
+  // every load of the tile first: R at the owned points, then the K range (not
+  // through the read-only path: they may not move above a dependent launch's wait)
   float rv[NUP][GN];
   int fo[NUP];
 #pragma unroll
@@ -120,14 +121,14 @@ __device__ __forceinline__ void fx_tile(const TcFxParams& p, unsigned char* As, 
     fo[i] = fx_pick<F_>(fid, p.rfs[i]);
 #pragma unroll
     for (int q = 0; q < GN; ++q)
-      rv[i][q] = i < p.n_up_f ? __ldg(p.R + ((uint32_t)(G0 + q) * nface + (uint32_t)fo[i])) : 0.f;
+      rv[i][q] = i < p.n_up_f ? p.R[(uint32_t)(G0 + q) * nface + (uint32_t)fo[i]] : 0.f;
   }
   float v[S::KQ];
 #pragma unroll
   for (int j = 0; j < S::KQ; ++j) {
     const int k = Q * S::KQ + j;
     const int f = k / NQF, g = k - (k / NQF) * NQF;
-    v[j] = k < S::NQFS ? __ldg(p.in + ((uint32_t)g * nface + (uint32_t)fid[f < F_ ? f : 0])) : 0.f;
+    v[j] = k < S::NQFS ? p.in[(uint32_t)g * nface + (uint32_t)fid[f < F_ ? f : 0]] : 0.f;
   }
   unsigned char* Arow = As + (uint32_t)(row >> 3) * S::SBO + (uint32_t)(row & 7) * 16u;
 #pragma unroll

@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <vector>
 
+#include "dependent_launch.cuh"
 #include "ehdg_internal.h"
 #include "tiled_common.cuh"
 #include "lp_pass.cuh"
@@ -41,6 +42,7 @@ __global__ void __launch_bounds__(32 * kTW) k_sweep_lp_tiled(const LpTParams p) 
   const int64_t nwarps = (int64_t)gridDim.x * kTW, gw = (int64_t)blockIdx.x * kTW + w;
   const int64_t J0 = p.total_rows * gw / nwarps, J1 = p.total_rows * (gw + 1) / nwarps;
   int64_t qp = 0, q_done = 0;
+  dep_trigger();
   ring_init(mbar0, S, lane);
   ring_fill(static_cast<const T*>(p.Hyt_lp), stages, mbar0, S, NQ, lane, J0, J1 - J0, 0, qp,
             J1 - J0);
@@ -272,8 +274,7 @@ cudaError_t lp_config(int64_t total_rows, int64_t ntiles, int* grid, size_t* sme
 
 template <int F, int NQF, class T>
 cudaError_t lp_launch(const LpTParams& p, int grid, size_t smem, cudaStream_t s) {
-  k_sweep_lp_tiled<F, NQF, T><<<grid, 32 * kTW, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_dependent(k_sweep_lp_tiled<F, NQF, T>, dim3(grid), dim3(32 * kTW), smem, s, p);
 }
 
 struct AuxOps {
