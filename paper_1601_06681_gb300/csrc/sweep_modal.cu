@@ -252,32 +252,6 @@ __device__ __forceinline__ unsigned long long fx_face(const double (&x)[P1 * P1]
   return ex;
 }
 
-// v = sum_a c_a (l X_in + r X_out)
-template <int P1>
-__device__ __forceinline__ void md_lift(double (&v)[P1 * P1 * P1], const MdParams<P1>& p,
-                                        int slot, int64_t e) {
-  constexpr int RC = MdBlocks<P1>::RC, N2 = P1 * P1;
-  const int64_t nface = p.nface;
-  const long long* src = p.tr.m + (int64_t)slot * N2 * nface;
-  const unsigned long long* ee = p.tr.e + (int64_t)slot * nface;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const int fi = p.elem_face[p.fin[a] * p.nel + e], fo = p.elem_face[p.fout[a] * p.nel + e];
-    const unsigned long long ei = ee[fi], eo = ee[fo];
-#pragma unroll
-    for (int g = 0; g < N2; ++g) {
-      const double xi = fx_to_double(src[g * nface + fi], fx_field(ei, fx_block<P1>(g)));
-      const double xo = fx_to_double(src[g * nface + fo], fx_field(eo, fx_block<P1>(g)));
-#pragma unroll
-      for (int i = 0; i < P1; ++i) {
-        double& t = v[md_idx<P1>(a, i, g % P1, g / P1)];
-        t = a == 0 ? p.cl[a][i] * xi : fma(p.cl[a][i], xi, t);
-        if (i < RC) t = fma(p.cr[a][i], xo, t);
-      }
-    }
-  }
-}
-
 // v <- (tau + sum_a c_a T_a)^{-1} v, last block first
 template <int P1>
 __device__ __forceinline__ void md_solve(double (&v)[P1 * P1 * P1], const MdParams<P1>& p) {
@@ -365,6 +339,174 @@ __device__ __forceinline__ void md_transform(double (&x)[P1 * P1 * P1],
     }
 }
 
+// an element's faces, its exponents and the unit of its values
+struct FxElem {
+  unsigned e8, fi[3], fo[3];                   // byte offsets of the first coefficients
+  unsigned long long ei[3], eo[3], eg[3];
+  int top, L;                                  // values in units of 2^L: the largest has p.ib bits
+};
+
+template <int P1, bool CG>
+__device__ __forceinline__ FxElem fx_element(const FxParams<P1>& p, int64_t e,
+                                             const unsigned long long* esrc) {
+  const int64_t ne = p.nel;
+  FxElem x;
+  x.e8 = 8u * (unsigned)e;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    x.fi[a] = 8u * (unsigned)p.elem_face[p.fin[a] * ne + e];
+    x.fo[a] = 8u * (unsigned)p.elem_face[p.fout[a] * ne + e];
+  }
+  unsigned m0 = 0x80008000u, m1 = 0x80008000u;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    x.ei[a] = fx_ld<CG>(esrc, x.fi[a]);
+    x.eo[a] = fx_ld<CG>(esrc, x.fo[a]);
+    x.eg[a] = fx_at(p.tr.Ge + a * ne, x.e8);
+    m0 = __vmaxs2(__vmaxs2(m0, (unsigned)x.ei[a]), __vmaxs2((unsigned)x.eo[a], (unsigned)x.eg[a]));
+    m1 = __vmaxs2(__vmaxs2(m1, (unsigned)(x.ei[a] >> 32)),
+                  __vmaxs2((unsigned)(x.eo[a] >> 32), (unsigned)(x.eg[a] >> 32)));
+  }
+  m0 = __vmaxs2(m0, m1);
+  x.top = max((int)(short)m0, (int)(short)(m0 >> 16));
+  x.L = x.top + 62 - p.ib;
+  return x;
+}
+
+// One role's unknowns from the trace src: packed limbs in units of 2^L in
+// Mt[role]. TEAM: the other roles run in the block's other warps.
+template <int P1, bool TEAM, bool SOLO, bool CG>
+__device__ __forceinline__ void fx_solve(const FxParams<P1>& p, const FxElem& el,
+                                         const long long* src,
+                                         long long (*Mt)[P1 * 4][32], int role, int lane) {
+  using B = MdBlocks<P1>;
+  using S = FxShape<P1>;
+  constexpr int NG = S::NG, OFF = S::OFF;
+  const int J = role % NG, K = role / NG, L = el.L;
+  const int64_t nface = p.tr.nface;
+  const unsigned(&fi)[3] = el.fi, (&fo)[3] = el.fo;
+  const unsigned long long(&ei)[3] = el.ei, (&eo)[3] = el.eo;
+  long long(*M)[32] = Mt[role];
+  // lifts
+  {
+    Limb xi[4], xo[4];
+    const int b0 = J + 2 * K;
+    const Align ai(L, fx_field(ei[0], b0)), ao(L, fx_field(eo[0], b0));
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = 2 * J + (u & 1) - OFF, k = 2 * K + (u >> 1) - OFF;
+      const bool ok = OFF == 0 || (j >= 0 && k >= 0);
+      const int64_t g = ok ? j + P1 * k : 0;
+      xi[u] = fx_split(ok ? ai(fx_ld<CG>(src + g * nface, fi[0])) : 0);
+      xo[u] = fx_split(ok ? ao(fx_ld<CG>(src + g * nface, fo[0])) : 0);
+    }
+#pragma unroll (SOLO || P1 == 4 ? 1 : P1)
+    for (int i = 0; i < P1; ++i) {
+      const int by = S::group(i) + 2 * K, bz = S::group(i) + 2 * J;
+      const Align yi(L, fx_field(ei[1], by)), yo(L, fx_field(eo[1], by));
+      const Align zi(L, fx_field(ei[2], bz)), zo(L, fx_field(eo[2], bz));
+      Limb ty[2][2], tz[2][2];                  // [in, out][index in the group]
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int k = 2 * K + u - OFF, j = 2 * J + u - OFF;
+        const bool oky = OFF == 0 || k >= 0, okz = OFF == 0 || j >= 0;
+        const int64_t gy = oky ? i + P1 * k : 0, gz = okz ? i + P1 * j : 0;
+        ty[0][u] = fx_split(oky ? yi(fx_ld<CG>(src + gy * nface, fi[1])) : 0);
+        ty[1][u] = fx_split(oky ? yo(fx_ld<CG>(src + gy * nface, fo[1])) : 0);
+        tz[0][u] = fx_split(okz ? zi(fx_ld<CG>(src + gz * nface, fi[2])) : 0);
+        tz[1][u] = fx_split(okz ? zo(fx_ld<CG>(src + gz * nface, fo[2])) : 0);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int jj = u & 1, kz = u >> 1;
+        Acc t(0);
+        t.mac(p.clx[i], xi[u]);
+        t.mac(p.crx[i], xo[u]);
+        t.mac(p.cl[0][2 * J + jj], ty[0][kz]);
+        t.mac(p.cr[0][2 * J + jj], ty[1][kz]);
+        t.mac(p.cl[1][2 * K + kz], tz[0][jj]);
+        t.mac(p.cr[1][2 * K + kz], tz[1][jj]);
+        M[i * 4 + u][lane] = t.get();
+      }
+    }
+  }
+  // couplings from the warps of higher groups
+  // barrier 1: (1, 1) has published; barrier 2: (0, 1) and (1, 0) have.
+  // Every warp meets both once per tile and waits only for what it reads,
+  // and (1, 1) at the end of its tile for barrier 2, so that no warp comes to
+  // a barrier a second time before its first phase has ended: (1, 1) and, by
+  // barrier 1, the next two need barrier 2 of the tile before, (0, 0) waits
+  // for it itself. The same order lets a buffer be written again two tiles on.
+  if (NG > 1 && !(J && K)) {
+    if (TEAM) {
+      if (J || K) {
+        bar_sync<1>();
+      } else {
+        bar_arrive<1>();
+        bar_sync<2>();
+      }
+    }
+    const long long(*VJ)[32] = Mt[(1 + NG * K) % S::NW];   // (1, K)
+    const long long(*VK)[32] = Mt[(J + NG) % S::NW];       // (J, 1)
+#pragma unroll 1
+    for (int i = 0; i < P1; ++i) {
+      Acc t[4] = {Acc(M[i * 4][lane]), Acc(M[i * 4 + 1][lane]), Acc(M[i * 4 + 2][lane]),
+                  Acc(M[i * 4 + 3][lane])};
+      if (J == 0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {           // (c, kz)
+          const Limb x = fx_limb(VJ[i * 4 + u][lane]);
+          t[u & 2].mac(p.T[0][0][u & 1], x);
+          t[(u & 2) + 1].mac(p.T[0][1][u & 1], x);
+        }
+      }
+      if (K == 0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {           // (jj, c)
+          const Limb x = fx_limb(VK[i * 4 + u][lane]);
+          t[u & 1].mac(p.T[1][0][u >> 1], x);
+          t[(u & 1) + 2].mac(p.T[1][1][u >> 1], x);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) M[i * 4 + u][lane] = t[u].get();
+    }
+  }
+  // the blocks along the first axis, last first
+  const Cfx* inv = p.inv[role];
+#pragma unroll
+  for (int I = B::NB - 1; I >= 0; --I) {
+    const int si = B::size(I), m = 4 * si;
+    Limb b[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      if (x >= m) continue;
+      const int i = I + x / 4;
+      long long y = M[i * 4 + (x & 3)][lane];
+      if (I + si < P1) {
+        Acc t(y);
+#pragma unroll
+        for (int c = 0; c < P1; ++c)
+          if (c >= I + si) t.mac(p.Tx[i][c], fx_limb(M[c * 4 + (x & 3)][lane]));
+        y = t.get();
+      }
+      b[x] = fx_split(y);
+    }
+#pragma unroll 4
+    for (int x = 0; x < m; ++x) {
+      Acc t(0);
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (c < m) t.mac(inv[S::off(I) + x * m + c], b[c]);
+      M[I * 4 + x][lane] = fx_pack(fx_split(t.get()));
+    }
+  }
+  if (TEAM && (J || K)) {
+    if (J && K) bar_arrive<1>();
+    else bar_arrive<2>();
+  }
+}
+
 // The sweep in fixed point: 32 elements per tile. Role (J, K) holds the unknowns
 // of group J of the second and K of the third axis and solves them as dense
 // blocks (4 x the first axis's block) after it has taken the couplings from the
@@ -384,9 +526,8 @@ __device__ __forceinline__ void md_transform(double (&x)[P1 * P1 * P1],
 template <int P1, bool SOLO, bool PERSIST>
 __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 : 4)
     k_sweep_fx(const __grid_constant__ FxParams<P1> p, const __grid_constant__ MdResid q) {
-  using B = MdBlocks<P1>;
   using S = FxShape<P1>;
-  constexpr int N2 = P1 * P1, NG = S::NG, OFF = S::OFF, RC = B::RC;
+  constexpr int N2 = P1 * P1, NG = S::NG, OFF = S::OFF, RC = MdBlocks<P1>::RC;
   // each warp's right-hand sides, then its solved limbs, at [i * 4 + jj + 2 kz];
   // two buffers (alternate tiles), since other warps read the solved values
   constexpr bool TEAM = NG > 1 && !SOLO;       // warps of a block share an element
@@ -408,28 +549,11 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= TEAM ? 1 : 0) {
     const bool live = tile * 32 + lane < ne;
     const int64_t e = live ? tile * 32 + lane : ne - 1;
-    const unsigned e8 = 8u * (unsigned)e;
-    unsigned fi[3], fo[3];                     // byte offsets of the faces' first coefficients
-    unsigned long long ei[3], eo[3], eg[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      fi[a] = 8u * (unsigned)p.elem_face[p.fin[a] * ne + e];
-      fo[a] = 8u * (unsigned)p.elem_face[p.fout[a] * ne + e];
-    }
-    unsigned m0 = 0x80008000u, m1 = 0x80008000u;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      ei[a] = fx_ld<PERSIST>(esrc, fi[a]);
-      eo[a] = fx_ld<PERSIST>(esrc, fo[a]);
-      eg[a] = fx_at(p.tr.Ge + a * ne, e8);
-      m0 = __vmaxs2(__vmaxs2(m0, (unsigned)ei[a]), __vmaxs2((unsigned)eo[a], (unsigned)eg[a]));
-      m1 = __vmaxs2(__vmaxs2(m1, (unsigned)(ei[a] >> 32)),
-                    __vmaxs2((unsigned)(eo[a] >> 32), (unsigned)(eg[a] >> 32)));
-    }
-    m0 = __vmaxs2(m0, m1);
-    const int top = max((int)(short)m0, (int)(short)(m0 >> 16));
-    // values in units of 2^L: the largest has p.ib bits
-    const int L = top + 62 - p.ib;
+    const FxElem el = fx_element<P1, PERSIST>(p, e, esrc);
+    const unsigned e8 = el.e8;
+    const unsigned(&fo)[3] = el.fo;
+    const unsigned long long(&eo)[3] = el.eo, (&eg)[3] = el.eg;
+    const int top = el.top, L = el.L;
 
     double r = 0.0;
 #pragma unroll 1
@@ -438,124 +562,7 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
     const int role = SOLO ? S::NW - 1 - step : role0;
     const int J = role % NG, K = role / NG;
     long long(*M)[32] = Msh[buf][role];
-    // lifts
-    {
-      Limb xi[4], xo[4];
-      const int b0 = J + 2 * K;
-      const Align ai(L, fx_field(ei[0], b0)), ao(L, fx_field(eo[0], b0));
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = 2 * J + (u & 1) - OFF, k = 2 * K + (u >> 1) - OFF;
-        const bool ok = OFF == 0 || (j >= 0 && k >= 0);
-        const int64_t g = ok ? j + P1 * k : 0;
-        xi[u] = fx_split(ok ? ai(fx_ld<PERSIST>(src + g * nface, fi[0])) : 0);
-        xo[u] = fx_split(ok ? ao(fx_ld<PERSIST>(src + g * nface, fo[0])) : 0);
-      }
-#pragma unroll (SOLO || P1 == 4 ? 1 : P1)
-      for (int i = 0; i < P1; ++i) {
-        const int by = S::group(i) + 2 * K, bz = S::group(i) + 2 * J;
-        const Align yi(L, fx_field(ei[1], by)), yo(L, fx_field(eo[1], by));
-        const Align zi(L, fx_field(ei[2], bz)), zo(L, fx_field(eo[2], bz));
-        Limb ty[2][2], tz[2][2];                  // [in, out][index in the group]
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int k = 2 * K + u - OFF, j = 2 * J + u - OFF;
-          const bool oky = OFF == 0 || k >= 0, okz = OFF == 0 || j >= 0;
-          const int64_t gy = oky ? i + P1 * k : 0, gz = okz ? i + P1 * j : 0;
-          ty[0][u] = fx_split(oky ? yi(fx_ld<PERSIST>(src + gy * nface, fi[1])) : 0);
-          ty[1][u] = fx_split(oky ? yo(fx_ld<PERSIST>(src + gy * nface, fo[1])) : 0);
-          tz[0][u] = fx_split(okz ? zi(fx_ld<PERSIST>(src + gz * nface, fi[2])) : 0);
-          tz[1][u] = fx_split(okz ? zo(fx_ld<PERSIST>(src + gz * nface, fo[2])) : 0);
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int jj = u & 1, kz = u >> 1;
-          Acc t(0);
-          t.mac(p.clx[i], xi[u]);
-          t.mac(p.crx[i], xo[u]);
-          t.mac(p.cl[0][2 * J + jj], ty[0][kz]);
-          t.mac(p.cr[0][2 * J + jj], ty[1][kz]);
-          t.mac(p.cl[1][2 * K + kz], tz[0][jj]);
-          t.mac(p.cr[1][2 * K + kz], tz[1][jj]);
-          M[i * 4 + u][lane] = t.get();
-        }
-      }
-    }
-    // couplings from the warps of higher groups
-    // barrier 1: (1, 1) has published; barrier 2: (0, 1) and (1, 0) have.
-    // Every warp meets both once per tile and waits only for what it reads,
-    // and (1, 1) at the end of its tile for barrier 2, so that no warp comes to
-    // a barrier a second time before its first phase has ended: (1, 1) and, by
-    // barrier 1, the next two need barrier 2 of the tile before, (0, 0) waits
-    // for it itself. The same order lets a buffer be written again two tiles on.
-    if (NG > 1 && !(J && K)) {
-      if (TEAM) {
-        if (J || K) {
-          bar_sync<1>();
-        } else {
-          bar_arrive<1>();
-          bar_sync<2>();
-        }
-      }
-      const long long(*VJ)[32] = Msh[buf][(1 + NG * K) % S::NW];   // (1, K)
-      const long long(*VK)[32] = Msh[buf][(J + NG) % S::NW];       // (J, 1)
-#pragma unroll 1
-      for (int i = 0; i < P1; ++i) {
-        Acc t[4] = {Acc(M[i * 4][lane]), Acc(M[i * 4 + 1][lane]), Acc(M[i * 4 + 2][lane]),
-                    Acc(M[i * 4 + 3][lane])};
-        if (J == 0) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {           // (c, kz)
-            const Limb x = fx_limb(VJ[i * 4 + u][lane]);
-            t[u & 2].mac(p.T[0][0][u & 1], x);
-            t[(u & 2) + 1].mac(p.T[0][1][u & 1], x);
-          }
-        }
-        if (K == 0) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {           // (jj, c)
-            const Limb x = fx_limb(VK[i * 4 + u][lane]);
-            t[u & 1].mac(p.T[1][0][u >> 1], x);
-            t[(u & 1) + 2].mac(p.T[1][1][u >> 1], x);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) M[i * 4 + u][lane] = t[u].get();
-      }
-    }
-    // the blocks along the first axis, last first
-    const Cfx* inv = p.inv[role];
-#pragma unroll
-    for (int I = B::NB - 1; I >= 0; --I) {
-      const int si = B::size(I), m = 4 * si;
-      Limb b[8];
-#pragma unroll
-      for (int x = 0; x < 8; ++x) {
-        if (x >= m) continue;
-        const int i = I + x / 4;
-        long long y = M[i * 4 + (x & 3)][lane];
-        if (I + si < P1) {
-          Acc t(y);
-#pragma unroll
-          for (int c = 0; c < P1; ++c)
-            if (c >= I + si) t.mac(p.Tx[i][c], fx_limb(M[c * 4 + (x & 3)][lane]));
-          y = t.get();
-        }
-        b[x] = fx_split(y);
-      }
-#pragma unroll 4
-      for (int x = 0; x < m; ++x) {
-        Acc t(0);
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-          if (c < m) t.mac(inv[S::off(I) + x * m + c], b[c]);
-        M[I * 4 + x][lane] = fx_pack(fx_split(t.get()));
-      }
-    }
-    if (TEAM && (J || K)) {
-      if (J && K) bar_arrive<1>();
-      else bar_arrive<2>();
-    }
+    fx_solve<P1, TEAM, SOLO, PERSIST>(p, el, src, Msh[buf], role, lane);
     // outflow coefficients: residual, normalisation, store
     // sums of squares D = d1 2^30 + d0 per axis
     long long s11, s10, s00;
@@ -728,26 +735,78 @@ __global__ void __launch_bounds__(128) k_step_md(const __grid_constant__ MdParam
 }
 
 // u^{k+1} = G + (tau + sum c T)^{-1} (lifts of uhat^k), the trace the last
-// sweep read, back to nodal values (Crank-Nicolson: 2 v - u^n)
-template <int P1>
-__global__ void __launch_bounds__(128) k_final_md(const __grid_constant__ MdParams<P1> p,
-                                                  const __grid_constant__ MdVolume<P1> s) {
-  constexpr int N2 = P1 * P1, N3 = P1 * N2;
-  const int64_t ne = p.nel;
+// sweep read, back to nodal values (Crank-Nicolson: 2 v - u^n). The lifts and
+// the solve are the sweep's, in fixed point; the sum with G and the transform
+// (3 P1^4 products) run in double, in place in the shared memory that holds the
+// unknowns. In double throughout, one thread per element, it was bound by the
+// FP64 pipe on large meshes (964 us at 64^3, p = 3) and by fetching its
+// straight-line code on small ones (59 us at 17 x 12 x 9, p = 2).
+template <int P1, bool SOLO>
+__global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 : 4)
+    k_final_fx(const __grid_constant__ FxParams<P1> p, const __grid_constant__ MdVolume<P1> s) {
+  using S = FxShape<P1>;
+  constexpr int N2 = P1 * P1, N3 = P1 * N2, NG = S::NG, OFF = S::OFF;
+  constexpr bool TEAM = NG > 1 && !SOLO;
+  constexpr int WARPS = TEAM ? S::NW : 1;
+  __shared__ long long Msh[TEAM ? 2 : 1][S::NW][P1 * 4][32];
+  const int64_t ne = p.nel, ntiles = (ne + 31) / 32;
+  const int lane = threadIdx.x, wid = threadIdx.y;
+  const int role0 = (int)__reduce_max_sync(0xffffffffu, threadIdx.y);
   const int slot = (p.it->k + 1) & 1;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    double v[N3];
-    md_lift<P1>(v, p, slot, e);
-    md_solve<P1>(v, p);
+  const long long* src = p.tr.m + (int64_t)slot * N2 * p.tr.nface;
+  const unsigned long long* esrc = p.tr.e + (int64_t)slot * p.tr.nface;
+  int buf = 0;
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, buf ^= TEAM ? 1 : 0) {
+    const bool live = tile * 32 + lane < ne;
+    const int64_t e = live ? tile * 32 + lane : ne - 1;
+    const FxElem el = fx_element<P1, false>(p, e, esrc);
+#pragma unroll 1
+    for (int step = 0; step < (TEAM ? 1 : S::NW); ++step) {
+      const int role = TEAM ? role0 : S::NW - 1 - step;
+      fx_solve<P1, TEAM, SOLO, false>(p, el, src, Msh[buf], role, lane);
+      if (TEAM && role % NG && role / NG) bar_sync<2>();
+    }
+    auto sync = [] {
+      if (TEAM) __syncthreads();
+      else __syncwarp();
+    };
+    auto at = [&](int i, int j, int k) -> long long& {
+      return Msh[buf][S::group(j) + NG * S::group(k)]
+                [i * 4 + ((j + OFF) & 1) + 2 * ((k + OFF) & 1)][lane];
+    };
+    sync();
+#pragma unroll 4
+    for (int c = wid; c < N3; c += WARPS) {
+      long long& m = at(c % P1, (c / P1) % P1, c / N2);
+      const Limb x = fx_limb(m);
+      double v = fx_value(((long long)x.h << kW) + x.l, el.L);
+      if (el.top == kExpNan) v = __hiloint2double(0x7ff80000, 0);
+      m = __double_as_longlong(v + s.G[c * ne + e]);
+    }
+    sync();
+#pragma unroll 1
+    for (int a = 0; a < 3; ++a) {
+#pragma unroll 1
+      for (int g = wid; g < N2; g += WARPS) {
+        const int t1 = g % P1, t2 = g / P1;
+        double x[P1];
 #pragma unroll
-    for (int c = 0; c < N3; ++c) v[c] += s.G[c * ne + e];
-    md_transform<P1>(v, s.Q);
+        for (int c = 0; c < P1; ++c)
+          x[c] = __longlong_as_double(a == 0 ? at(c, t1, t2) : (a == 1 ? at(t1, c, t2) : at(t1, t2, c)));
 #pragma unroll
-    for (int c = 0; c < N3; ++c) {
-      double x = v[c];
-      if (s.cn) x = 2.0 * x - s.u[c * ne + e];
-      s.u[c * ne + e] = x;
+        for (int i = 0; i < P1; ++i) {
+          double y = s.Q[a][i][0] * x[0];
+#pragma unroll
+          for (int c = 1; c < P1; ++c) y = fma(s.Q[a][i][c], x[c], y);
+          if (a < 2) {
+            (a == 0 ? at(i, t1, t2) : at(t1, i, t2)) = __double_as_longlong(y);
+          } else if (live) {
+            double* u = s.u + (int64_t)(g + N2 * i) * ne + e;
+            *u = s.cn ? 2.0 * y - *u : y;
+          }
+        }
+      }
+      sync();
     }
   }
 }
@@ -770,6 +829,15 @@ struct MdFace {
   int* warm;
   int cn;
 };
+
+// The tables in shared memory, indexed by a face's axes: one copy of the
+// transform's code instead of one per axis, and half the registers.
+template <int P1>
+__device__ __forceinline__ void md_stage(const double (&m)[3][P1][P1], double (&tab)[3][P1][P1]) {
+  for (int i = threadIdx.x; i < 3 * P1 * P1; i += blockDim.x)
+    tab[i / (P1 * P1)][(i / P1) % P1][i % P1] = m[i / (P1 * P1)][(i / P1) % P1][i % P1];
+  __syncthreads();
+}
 
 template <int P1>
 __device__ __forceinline__ void md_face_transform(double (&x)[P1 * P1], const double (&m1)[P1][P1],
@@ -804,6 +872,8 @@ __device__ __forceinline__ void md_face_transform(double (&x)[P1 * P1], const do
 template <int P1>
 __global__ void __launch_bounds__(128) k_bnd_md(const __grid_constant__ MdFace<P1> p) {
   constexpr int N2 = P1 * P1;
+  __shared__ double tab[3][P1][P1];
+  md_stage<P1>(p.C, tab);
   const int64_t nface = p.nface;
   for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < p.n_bface;
        b += (int64_t)gridDim.x * blockDim.x) {
@@ -814,9 +884,7 @@ __global__ void __launch_bounds__(128) k_bnd_md(const __grid_constant__ MdFace<P
     for (int g = 0; g < N2; ++g)
       x[g] = p.cn ? 0.5 * (p.gb[g * nface + f] + p.gb_old[g * nface + f]) : p.gb[g * nface + f];
     const int ax = p.face_local[f] >> 1;
-    if (ax == 0) md_face_transform<P1>(x, p.C[1], p.C[2]);
-    else if (ax == 1) md_face_transform<P1>(x, p.C[0], p.C[2]);
-    else md_face_transform<P1>(x, p.C[0], p.C[1]);
+    md_face_transform<P1>(x, tab[ax == 0 ? 1 : 0], tab[ax == 2 ? 1 : 2]);
     long long m[N2];
     const unsigned long long ex = fx_face<P1>(x, m);
 #pragma unroll
@@ -832,8 +900,10 @@ __global__ void __launch_bounds__(128) k_bnd_md(const __grid_constant__ MdFace<P
 // The final trace uhat^K back to the face Gauss points in slot 0 of uhat
 // (Crank-Nicolson: 2 vhat - uhat^n, with the previous-level copies updated)
 template <int P1>
-__global__ void __launch_bounds__(128) k_trace_end_md(const __grid_constant__ MdFace<P1> p) {
+__global__ void __launch_bounds__(128, 4) k_trace_end_md(const __grid_constant__ MdFace<P1> p) {
   constexpr int N2 = P1 * P1;
+  __shared__ double tab[3][P1][P1];
+  md_stage<P1>(p.V, tab);
   const int64_t nface = p.nface;
   const int slot = p.it->k & 1;
   const long long* fin = p.tr.m + (int64_t)slot * N2 * nface;
@@ -845,9 +915,7 @@ __global__ void __launch_bounds__(128) k_trace_end_md(const __grid_constant__ Md
 #pragma unroll
     for (int g = 0; g < N2; ++g) x[g] = fx_to_double(fin[g * nface + f], fx_field(ex, fx_block<P1>(g)));
     const int ax = p.face_local[f] >> 1;
-    if (ax == 0) md_face_transform<P1>(x, p.V[1], p.V[2]);
-    else if (ax == 1) md_face_transform<P1>(x, p.V[0], p.V[2]);
-    else md_face_transform<P1>(x, p.V[0], p.V[1]);
+    md_face_transform<P1>(x, tab[ax == 0 ? 1 : 0], tab[ax == 2 ? 1 : 2]);
 #pragma unroll
     for (int g = 0; g < N2; ++g) {
       const int64_t t = g * nface + f;
@@ -1353,6 +1421,21 @@ cudaError_t step_t(Ctx& c) {
   return cudaGetLastError();
 }
 
+// One warp does all groups of its elements where there are tiles enough to
+// keep 12 warps per SM on full runs: 243 against 265 us at 8,192 tiles (64^3,
+// p = 3). With fewer the team's shorter tile wins: 93 against 109 us per
+// iteration at 2,000 tiles, 31 against 45 at 16.
+bool fx_solo(int64_t nel) { return (nel + 31) / 32 >= 32 * device_sms(); }
+
+template <int P1, bool SOLO>
+cudaError_t final_launch(const FxParams<P1>& x, const MdVolume<P1>& v, cudaStream_t s) {
+  const int nw = SOLO ? 1 : FxShape<P1>::NW;
+  const int bpsm = fn_blocks_per_sm((const void*)k_final_fx<P1, SOLO>, 32 * nw, 0);
+  const int grid = (int)std::min<int64_t>((int64_t)bpsm * device_sms(), (x.nel + 31) / 32);
+  k_final_fx<P1, SOLO><<<std::max(grid, 1), dim3(32, nw), 0, s>>>(x, v);
+  return cudaGetLastError();
+}
+
 // One launch form (SOLO or a team of warps) of the sweep; persist: every
 // iteration of the step, cooperative. The grid does not depend on persist, so
 // the residual is the same sum in both.
@@ -1384,11 +1467,7 @@ cudaError_t sweep_t(Ctx& c, int graph_mode, bool persist) {
   q.max_iter = c.max_iter;
   q.graph_mode = graph_mode;
   q.handle = c.handle;
-  // One warp does all groups of its elements where there are tiles enough to
-  // keep 12 warps per SM on full runs: 243 against 265 us at 8,192 tiles (64^3,
-  // p = 3). With fewer the team's shorter tile wins: 93 against 109 us per
-  // iteration at 2,000 tiles, 31 against 45 at 16.
-  if (FxShape<P1>::NW == 1 || (c.nel + 31) / 32 >= 32 * device_sms())
+  if (FxShape<P1>::NW == 1 || fx_solo(c.nel))
     return sweep_launch<P1, true>(p, q, c.n_partials, persist, c.stream);
   return sweep_launch<P1, false>(p, q, c.n_partials, persist, c.stream);
 }
@@ -1396,12 +1475,9 @@ cudaError_t sweep_t(Ctx& c, int graph_mode, bool persist) {
 template <int P1>
 cudaError_t final_t(Ctx& c) {
   const MdKernelArgs<P1>& t = md_args<P1>(c);
-  const MdParams<P1>& p = t.p;
-  const MdVolume<P1>& s = t.s;
   const MdFace<P1>& f = t.f;
-  const int th = md_threads(c.nel);
-  k_final_md<P1><<<md_grid(k_final_md<P1>, th, c.nel), th, 0, c.stream>>>(p, s);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = FxShape<P1>::NW == 1 || fx_solo(c.nel) ? final_launch<P1, true>(t.x, t.s, c.stream)
+                                                        : final_launch<P1, false>(t.x, t.s, c.stream);
   if (e != cudaSuccess) return e;
   const int tf = md_threads(c.nface);
   k_trace_end_md<P1><<<md_grid(k_trace_end_md<P1>, tf, c.nface), tf, 0, c.stream>>>(f);

@@ -128,3 +128,24 @@ def test_zero_and_non_finite_states(p):
         s.run(1)
         u, uh = s.get_state()
         assert np.abs(u - 1).max() < 1e-12 and np.abs(uh - 1).max() < 1e-12
+
+
+@pytest.mark.parametrize("n,p", [((55, 54, 53), 1), ((55, 54, 53), 2), ((33, 34, 35), 2),
+                                 ((33, 34, 35), 3), ((3, 1, 11), 3)])
+def test_crank_nicolson_keeps_a_linear_solution(n, p):
+    """The same linear solution under Crank-Nicolson, which is exact for it too:
+    the reconstruction 2 v - u^n in its three forms (one warp per tile, a team per
+    tile, p = 1). Two steps; tolerance as above, twice for the factor 2."""
+    beta, a, dt = np.array([0.7, -0.4, 0.6]), np.array([0.3, -0.2, 0.5]), 5e-3
+    sol = lambda x, t: 1.0 + x @ a - (a @ beta) * t      # noqa: E731
+    with E.Solver(E.ehdg_mesh_structured(n), p, scheme="cn", dt=dt, tol=1e-13, max_iter=500,
+                  beta_const=beta) as s:
+        x, xf = s.node_coords(), s.face_point_coords()
+        s.set_boundary(sol(xf, 0.0))
+        s.set_state(sol(x, 0.0)[:, None, :])
+        for k in (1, 2):
+            s.set_boundary(sol(xf, k * dt))
+            s.run(1)
+        u, uh = s.get_state()
+    assert np.abs(u[:, 0] - sol(x, 2 * dt)).max() < 2e-11
+    assert np.abs(uh - sol(xf, 2 * dt)).max() < 2e-11
