@@ -614,7 +614,7 @@ def run_2d(args, ws, dev, stream, standalone=False):
     # roofline of the dominant kernel (k_sweep_persist, the persistent form of
     # k_sweep_tiled that runs a step's iterations in one launch; figures per
     # sweep): per element and sweep it reads its operator rows (rows x NQFS
-    # doubles), Gy and the point id of each row, the trace at its NQFS face
+    # limb pairs of 8 bytes), Gy and the point id of each row, the trace at its NQFS face
     # points, its 4 face ids and face Jacobians and its two row counts, and
     # writes one value per row; flops = 2 x rows x NQFS
     info = solver.info
@@ -634,7 +634,7 @@ def run_2d(args, ws, dev, stream, standalone=False):
                                 "face for this per-node velocity (p+1 = 5 counted)",
         "iterations_per_run": iters_total / reps, "setup_s": round(setup_s, 3),
         "fp64_rel_l2_vs_fp64_fixed_point": rel_l2(u_fp64, u_fix),
-        "roofline": {"kernel": "k_sweep_persist", "bound": "alu",
+        "roofline": {"kernel": "k_sweep_persist", "bound": "hbm",
                      "achieved_tflops": flops / (avg_ms * 1e-3) / 1e12,
                      "flops_per_sweep": flops, "alg_bytes_per_sweep": alg_bytes,
                      "avg_sweep_us": avg_ms * 1e3, "sweeps": int(prof_sweeps),
@@ -688,6 +688,26 @@ def fp64_sweep(info):
     return "k_sweep_sf", 2.0 * fma, dense
 
 
+# Products per element and sweep of the fixed-point Schur sweep (k_sweep_fx,
+# padded groups included) at p = 3, each three 32 x 32 + 64 integer
+# multiply-adds; 57 of those per clock and SM measured.
+SCHUR_PRODUCTS = {4: 1140}
+MULTIPLY_ADDS_PER_CLOCK = 57.0
+SM_MAX_MHZ = 2070.0
+
+
+def schur_roofline(info, sweeps, ms, sms, mhz):
+    """The integer-pipe view of `sweeps` iterations that took `ms` in all (the
+    persistent form: one launch per step)."""
+    t = ms * 1e-3 / max(sweeps, 1)
+    mads = 3.0 * SCHUR_PRODUCTS[info["q"]] * info["n_elem"]
+    peak = MULTIPLY_ADDS_PER_CLOCK * sms * mhz * 1e6 / 1e12
+    return {"kernel": "k_sweep_fx", "bound": "alu", "achieved": mads / t / 1e12, "peak": peak,
+            "unit": "T integer multiply-adds/s", "frac": mads / t / 1e12 / peak,
+            "peak_source": f"{sms} SMs x {MULTIPLY_ADDS_PER_CLOCK:.0f} per clock (measured) x {mhz:.0f} MHz",
+            "multiply_adds_per_sweep": mads, "avg_sweep_us": t * 1e6, "sweeps": int(sweeps)}
+
+
 # the dominant kernel of each kind the profiling run times, per path
 def _kernel_name(kind, precision, emulated_outer, info=None):
     emulated = precision == "fp64_emulated" or emulated_outer
@@ -700,7 +720,7 @@ def _kernel_name(kind, precision, emulated_outer, info=None):
 
 
 def dominant_roofline(stats, info, precision, emulated_outer, fp64_peak_tf, fp64_src, peaks,
-                      peak_src):
+                      peak_src, sweeps=0, sms=0, mhz=0.0):
     """Roofline of the kind with the largest share of a profiled run:
     FP64 sweep on the DFMA pipe (alu), FP64-accurate sweep on the BF16 tensor
     pipe (tensor, executed digit MMAs), correction sweep (hbm)."""
@@ -708,6 +728,9 @@ def dominant_roofline(stats, info, precision, emulated_outer, fp64_peak_tf, fp64
     nel, nq, rows = info["n_elem"], 2 * info["dim"] * info["Nqf"], info["sweep_rows"]
     share = kernel_shares(stats).get(kind, 0.0)
     launches, ms = stats[kind]
+    if kind == "elem" and sweeps and precision in ("fp64", "fp64_emulated"):
+        return {"kind": kind, "share": share, "launches": int(launches),
+                **schur_roofline(info, sweeps, ms, sms, mhz)}
     name = _kernel_name(kind, precision, emulated_outer, info)
     out = {"kernel": name, "kind": kind, "share": share, "launches": int(launches)}
     if kind == "elem" and name in ("k_sweep_fused", "k_sweep_sf"):
@@ -856,23 +879,20 @@ def run_headline(args):
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     peak_tf, peak_txt, probe_tf, derived_tf, sms = fp64_peak(ehdg, stream, clocks.get("sm_mhz"))
     nq, rows, nel = 2 * info["dim"] * info["Nqf"], info["sweep_rows"], info["n_elem"]
-    n_sweep, sweep_ms = stats["elem"]
-    avg_ms = sweep_ms / max(n_sweep, 1)
-    sweep_kernel, flops, dense_flops = fp64_sweep(info)
+    sweep_ms = stats["elem"][1]
+    avg_ms = sweep_ms / max(prof_sweeps, 1)
+    _, _, dense_flops = fp64_sweep(info)
     alg_bytes = ALG_BYTES_PER_ELEM_3D * nel
     # bytes the fused sweep must move: the trace at the element's NQFS points
     # (each shared by the two elements of its face), Gy at its rows, the new
     # trace at its owned rows, its face ids
     own_bytes = nel * (8 * nq // 2 + 8 * 2 * (rows // nel) + 4 * 2 * info["dim"])
     roofline = {
-        "kernel": sweep_kernel, "bound": "alu",
-        "achieved": flops / (avg_ms * 1e-3) / 1e12, "peak": peak_tf, "unit": "TFLOP/s",
-        "frac": flops / (avg_ms * 1e-3) / 1e12 / peak_tf, "peak_source": peak_txt,
+        **schur_roofline(info, prof_sweeps, sweep_ms, sms, clocks.get("sm_mhz") or SM_MAX_MHZ),
         "fp64_probe_tflops": probe_tf, "fp64_derived_tflops": derived_tf, "sms": sms,
-        "traffic": kernel_traffic(f"{sweep_kernel}@transport3d_{n}x{n}x{n}_p3_be"),
-        "flops_per_sweep": flops, "dense_form_flops_per_sweep": dense_flops,
+        "traffic": kernel_traffic(f"k_sweep_fx@transport3d_{n}x{n}x{n}_p3_be"),
+        "dense_form_flops_per_sweep": dense_flops,
         "dense_form_equivalent_tflops": dense_flops / (avg_ms * 1e-3) / 1e12,
-        "avg_sweep_us": avg_ms * 1e3, "sweeps": int(n_sweep),
         "hbm_view": {"alg_bytes_per_sweep": alg_bytes,
                      "alg_bytes_definition": "8 (n + 2 T_own) per element, n = 64, T_own = 48",
                      "achieved_gbs": alg_bytes / (avg_ms * 1e-3) / 1e9, "peak_gbs": hbm,
@@ -931,7 +951,8 @@ def run_headline(args):
                    "rel_l2_trace_vs_fp64_fixed_point": rel_l2(uh, uh_fix),
                    "kernel_time_share": kernel_shares(st),
                    "dominant_kernel": dominant_roofline(st, s.info, prec, eo, peak_tf, peak_txt,
-                                                        peaks, peak_src)}
+                                                        peaks, peak_src, its, sms,
+                                                        clocks.get("sm_mhz") or SM_MAX_MHZ)}
             if prec in ("tf32", "bf16"):
                 ent["inner_sweeps"] = m_kept or args.inner_sweeps
                 if tried:
@@ -1023,10 +1044,10 @@ def run_2d_line(args):
     with ClockSampler(local) as clk:
         res = run_2d(args, ws, dev, stream, standalone=True)
     clocks = clk.summary()
-    peak_tf, peak_txt, probe_tf, derived_tf, sms = fp64_peak(ehdg, stream, clocks.get("sm_mhz"))
     r = res["roofline"]
-    r.update({"achieved": r["achieved_tflops"], "peak": peak_tf, "unit": "TFLOP/s",
-              "frac": r["achieved_tflops"] / peak_tf, "peak_source": peak_txt})
+    v = r["hbm_view"]
+    r.update({"achieved": v["achieved_gbs"], "peak": v["peak_gbs"], "unit": "GB/s",
+              "frac": v["frac"], "peak_source": v["peak_source"]})
     if rank == 0:
         line = {"metric": METRIC, "value": res["value"], "unit": UNIT, "n_gpus": ws,
                 "steps": args.steps, "warmup": args.warmup, "ms_per_step": res["ms_per_run"],
