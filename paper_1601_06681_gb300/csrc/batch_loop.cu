@@ -130,7 +130,7 @@ struct ListView {
 // counts[i] = (sweep items, 1 if mixed precision, correction tiles, update
 // chunks) of instance i.
 __device__ void build_lists(const BInst* inst, const int4* counts, int n_inst, int* L) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   const ListView v{n_inst};
   const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
   int* part = reinterpret_cast<int*>(sm);           // [5][nt]: per-thread sums, then offsets
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kPeTile, 5) k_batch_sweep(const BInst* inst, c
                                                           int* lists, int n_inst,
                                                           unsigned int* ticket, int graph_mode,
                                                           cudaGraphConditionalHandle handle) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) double sm[];
   const int tid = threadIdx.x;
   const ListView lv{n_inst};
   const int n_act = lists[0];
