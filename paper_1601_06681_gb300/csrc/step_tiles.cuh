@@ -105,12 +105,10 @@ __device__ __forceinline__ void tile_rows4(const FxOp& op, const int2* osh, cons
         L[i] = Lf;
         sum[i] = y[i];
       } else if (Lf > L[i]) {
-        const int sh = min(63, Lf - L[i]);
-        sum[i] = ((sum[i] + ((1LL << sh) >> 1)) >> sh) + y[i];
+        sum[i] = fx_shift(sum[i], Lf - L[i]) + y[i];
         L[i] = Lf;
       } else {
-        const int sh = min(63, L[i] - Lf);
-        sum[i] += (y[i] + ((1LL << sh) >> 1)) >> sh;
+        sum[i] += fx_shift(y[i], L[i] - Lf);
       }
     }
   }
