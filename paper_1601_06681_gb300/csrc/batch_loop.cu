@@ -54,8 +54,7 @@ struct BInst {
   const double* Gy;
   double* Y;
   float* R_out;
-  const int2* Hx;               // the sweep rows of Hy in row order, fixed-point limbs
-  const int* hs;
+  const int2* Hx;               // the sweep rows of Hy in fixed point (pe_tile.cuh)
   int own[2];                   // their local faces
   double* uhat;
   IterState* it;
@@ -234,7 +233,7 @@ __global__ void __launch_bounds__(kPeTile, 5) k_batch_sweep(const BInst* inst, c
   const int* pre = lv.pre_sw(lists);
   const int n_items = n_act > 0 ? pre[n_act] : 0;
   int cur = -1;
-  int2* Hsh = reinterpret_cast<int2*>(sm);            // the instance's sweep rows [n_rows][NQ]
+  int2* Hsh = reinterpret_cast<int2*>(sm);            // the instance's sweep rows
   for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
     // every listed instance iterates; its state cannot change before all its
     // work items are done
@@ -244,7 +243,7 @@ __global__ void __launch_bounds__(kPeTile, 5) k_batch_sweep(const BInst* inst, c
     const BInst& I = inst[idx];
     const int nq = I.NQFS;
     if (idx != cur) {   // the previous item's threads are past its last barrier
-      for (int i = tid; i < I.n_rows * nq; i += kPeTile) Hsh[i] = I.Hx[i];
+      for (int i = tid; i < pe_operator_len(nq); i += kPeTile) Hsh[i] = I.Hx[i];
       __syncthreads();
       cur = idx;
     }
@@ -255,7 +254,6 @@ __global__ void __launch_bounds__(kPeTile, 5) k_batch_sweep(const BInst* inst, c
     v.nface = I.nface;
     v.own[0] = I.own[0];
     v.own[1] = I.own[1];
-    v.hs = I.hs;
     v.elem_face = I.elem_face;
     v.face_jf = I.face_jf;
     v.fw = I.fw;
@@ -792,7 +790,6 @@ __device__ __forceinline__ bool q_sweep_item(const BInst& I, const int2* Hsh, in
   v.nface = I.nface;
   v.own[0] = I.own[0];
   v.own[1] = I.own[1];
-  v.hs = I.hs;
   v.elem_face = I.elem_face;
   v.face_jf = I.face_jf;
   v.fw = I.fw;
@@ -1253,7 +1250,6 @@ cudaError_t BatchLoop::build(const std::vector<Ctx*>& ctxs, unsigned long long* 
     I.Y = c.Y;
     I.R_out = c.mixed ? c.R32 : nullptr;
     I.Hx = reinterpret_cast<const int2*>(c.pe_hx);
-    I.hs = c.pe_hs;
     I.own[0] = c.rows_host[0] / c.Nqf;
     I.own[1] = c.rows_host[c.Nqf] / c.Nqf;
     I.uhat = c.uhat;
@@ -1293,7 +1289,7 @@ cudaError_t BatchLoop::build(const std::vector<Ctx*>& ctxs, unsigned long long* 
     L.nch += (int)(((int64_t)c.Nqf * c.nface + kApplyChunk - 1) / kApplyChunk);
     L.nmax = std::max(L.nmax, c.n);
     L.nqmax = std::max(L.nqmax, c.NQFS);
-    smem = std::max(smem, sizeof(double) * (size_t)c.n_rows * c.NQFS);
+    smem = std::max(smem, sizeof(int2) * (size_t)pe_operator_len(c.NQFS));
     L.n_sweep += I.n_tiles_pe;
     if (c.mixed) {
       I.tc = 1;

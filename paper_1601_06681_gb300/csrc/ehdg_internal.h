@@ -171,8 +171,7 @@ struct Ctx {
   int *fx_Ps = nullptr, *fx_Hs = nullptr, *fx_Es = nullptr, *fx_Hys = nullptr;
   bool use_pe = false;           // 2D shared-operator FP64 sweep, one thread per element
   double* pe_fw = nullptr;       // its face Gauss weights [Nqf]
-  void* pe_hx = nullptr;         // [n_rows][NQFS] its rows of Hy as fixed-point limbs (int2)
-  int* pe_hs = nullptr;          // [1] their scale
+  void* pe_hx = nullptr;         // its rows of Hy as fixed-point limbs, with their scales (pe_tile.cuh)
   bool use_sf = false;
   int sf_NB = 0;                 // boundary nodes per element
   int* sf_bnd = nullptr;         // [NB] their node indices

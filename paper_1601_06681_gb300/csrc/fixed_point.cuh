@@ -147,6 +147,9 @@ struct FxOp {
   const int2* x;
   const int* scale;
 };
+// the scale of a group of columns that are zero, so low that its values do not
+// raise the others' unit
+constexpr int kZeroGroup = -4096;
 __host__ __device__ inline int64_t fx_blocked(int rows, int cols) {
   return (int64_t)((rows + 3) / 4) * 4 * cols;
 }

@@ -5,8 +5,14 @@
 // of the two faces it is upwind of (NQ / 2 rows; no point has beta.n = 0),
 // writes the new trace there and adds w (uhat^{k+1} - uhat^k)^2 to the residual.
 //
-// The products run in fixed point on the integer pipe (fixed_point.cuh), the
-// element's traces and Gy aligned to the largest of them with 56 bits: the FP64
+// The products run in fixed point on the integer pipe (fixed_point.cuh). The
+// operator is equilibrated: Hy[j][c] = 2^(s_j + t_a) Hx[j][c], t_a for the columns
+// of axis a's faces, s_j for row j, both of either sign, since the columns go with
+// |beta_a| / h_a and all entries with dt where that is small. The element's traces
+// times 2^t_a are aligned to the largest of them with 56 bits, a row's sum and its
+// Gy to the larger of the two. (One scale for the whole operator, not below one,
+// lost 2.6e-13 of a trace at 16 x 16, p = 2, dt = 1e-6, in an element fed from rest;
+// the present form 5e-17, an FMA chain 8e-17.) The FP64
 // pipe, 1.6 operations per clock and SM, bounded the double form (NQ^2 / 2
 // products per element, 200 at p = 4). What is left there is four operations
 // per row: the conversion of the result, the increment, its square, the sum.
@@ -44,7 +50,6 @@ __device__ __forceinline__ T pe_ld(const T* p) {
 struct PeView {
   int64_t nel, nface;
   int own[2];                   // the local faces of the sweep rows: 0 or 1, 2 or 3
-  const int* hs;                // [1] scale: Hy = 2^(hs - 56) x the limbs below
   const int32_t* elem_face;     // [4][nel]
   const double* face_jf;        // [nface]
   const double* fw;             // face Gauss weight of each face point
@@ -59,8 +64,27 @@ struct PeView {
   __host__ __device__ const double* uhat_slot(int s, int64_t tlen) const { return uhat + s * tlen; }
 };
 
+// The operator in limbs: the sweep rows in row order, [NQ / 2][NQ], then (t_0, t_1)
+// and the NQ / 2 scales of the rows.
+__host__ __device__ constexpr int pe_operator_len(int NQ) { return NQ / 2 * NQ + 1 + NQ / 4; }
+
+// Gy + the sum of a row's products, x in units of 2^(unit - 1078) with the row's scale
+template <int NQ>
+__device__ __forceinline__ double pe_row(const int2* Hrow, const Limb (&x)[NQ], int unit, double gy) {
+  const int4* Hr = reinterpret_cast<const int4*>(Hrow);
+  Acc t(0);
+#pragma unroll
+  for (int c = 0; c < NQ; c += 2) {
+    const int4 h = Hr[c / 2];
+    t.mac(Cfx{h.x, h.y}, x[c]);
+    t.mac(Cfx{h.z, h.w}, x[c + 1]);
+  }
+  const int L = max(unit, max(fx_exponent(gy), 1));
+  return fx_value(fx_shift(t.get(), L - unit) + fx_from_double(gy, L), L - 1078);
+}
+
 // The tile's sweep; its residual sum goes to partials[tile] (thread 0). Hsh: the
-// sweep rows of the operator in row order, limbs, [NQ / 2][NQ] (16-byte aligned).
+// operator as above (16-byte aligned).
 template <int NQ, bool CG>
 __device__ __forceinline__ void pe_tile_sweep(const PeView& v, const int2* Hsh, const double* src,
                                               double* dst, int64_t tile) {
@@ -77,7 +101,8 @@ __device__ __forceinline__ void pe_tile_sweep(const PeView& v, const int2* Hsh, 
     for (int f = 0; f < 4; ++f) face[f] = v.elem_face[f * ne + e];
 #pragma unroll
     for (int j = 0; j < RN; ++j) gy[j] = v.Gy[j * ne + e];
-    const int hs = *v.hs;
+    const int2 tc = Hsh[RN * NQ];
+    const int* sc = reinterpret_cast<const int*>(Hsh + RN * NQ + 1);
 #pragma unroll
     for (int g = 0; g < NQF; ++g) w[g] = v.fw[g];
 #pragma unroll
@@ -86,28 +111,22 @@ __device__ __forceinline__ void pe_tile_sweep(const PeView& v, const int2* Hsh, 
       for (int g = 0; g < NQF; ++g) u[f * NQF + g] = pe_ld<CG>(src + g * nface + face[f]);
     const int64_t fo[2] = {v.own[0] ? face[1] : face[0], v.own[1] == 3 ? face[3] : face[2]};
     const double jf[2] = {v.face_jf[fo[0]], v.face_jf[fo[1]]};
-    int emax = 1;
+    int ea[2] = {1, 1}, eg = 1;
 #pragma unroll
-    for (int c = 0; c < NQ; ++c) emax = max(emax, fx_exponent(u[c]));
+    for (int c = 0; c < NQ; ++c) ea[c / (2 * NQF)] = max(ea[c / (2 * NQF)], fx_exponent(u[c]));
 #pragma unroll
-    for (int j = 0; j < RN; ++j) emax = max(emax, fx_exponent(gy[j]));
+    for (int j = 0; j < RN; ++j) eg = max(eg, fx_exponent(gy[j]));
+    const int em = max(ea[0] + tc.x, ea[1] + tc.y);
     double sq[2] = {0.0, 0.0};
     Limb x[NQ];
 #pragma unroll
-    for (int c = 0; c < NQ; ++c) x[c] = fx_split(fx_from_double(u[c], emax));
+    for (int c = 0; c < NQ; ++c)
+      x[c] = fx_split(fx_from_double(u[c], em - (c < 2 * NQF ? tc.x : tc.y)));
 #pragma unroll
     for (int j = 0; j < RN; ++j) {
-      const int4* Hr = reinterpret_cast<const int4*>(Hsh + j * NQ);
-      // the sum in units of 2^(emax - 1078 + hs), Gy aligned to it
-      Acc t(fx_from_double(gy[j], emax + hs));
-#pragma unroll
-      for (int c = 0; c < NQ; c += 2) {
-        const int4 h = Hr[c / 2];
-        t.mac(Cfx{h.x, h.y}, x[c]);
-        t.mac(Cfx{h.z, h.w}, x[c + 1]);
-      }
-      double acc = fx_value(t.get(), emax - 1078 + hs);
-      if (emax == 0x7ff) acc = __hiloint2double(0x7ff80000, 0);   // an input is not finite
+      double acc = pe_row<NQ>(Hsh + j * NQ, x, em + sc[j], gy[j]);
+      if (max(max(ea[0], ea[1]), eg) == 0x7ff)   // an input is not finite
+        acc = __hiloint2double(0x7ff80000, 0);
       const int b = j / NQF, g = j - b * NQF;
       const int64_t pt = g * nface + fo[b];
       const double old = v.own[b] & 1 ? u[(2 * b + 1) * NQF + g] : u[2 * b * NQF + g];

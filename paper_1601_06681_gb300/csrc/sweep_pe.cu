@@ -23,8 +23,8 @@ template <int NQ>
 __global__ void __launch_bounds__(kPeTile, NQ >= 20 ? 3 : 4) k_sweep_pe(const __grid_constant__ PeView v,
                                                       const int2* Hx, int graph_mode,
                                                       cudaGraphConditionalHandle handle) {
-  __shared__ __align__(16) int2 Hsh[NQ / 2 * NQ];
-  for (int i = threadIdx.x; i < NQ / 2 * NQ; i += kPeTile) Hsh[i] = Hx[i];
+  __shared__ __align__(16) int2 Hsh[pe_operator_len(NQ)];
+  for (int i = threadIdx.x; i < pe_operator_len(NQ); i += kPeTile) Hsh[i] = Hx[i];
   __syncthreads();
   const int kk = v.it->k;                     // read before the last tile advances it
   const int64_t tlen = (int64_t)(NQ / 4) * v.nface;
@@ -55,8 +55,8 @@ cudaError_t launch_pe_t(const PeView& v, const int2* Hx, int graph_mode,
 template <int NQ>
 __global__ void __launch_bounds__(kPeTile, NQ >= 20 ? 3 : 4) k_pe_persist(const __grid_constant__ PeView v,
                                                         const int2* Hx) {
-  __shared__ __align__(16) int2 Hsh[NQ / 2 * NQ];
-  for (int i = threadIdx.x; i < NQ / 2 * NQ; i += kPeTile) Hsh[i] = Hx[i];
+  __shared__ __align__(16) int2 Hsh[pe_operator_len(NQ)];
+  for (int i = threadIdx.x; i < pe_operator_len(NQ); i += kPeTile) Hsh[i] = Hx[i];
   __syncthreads();
   const int64_t tlen = (int64_t)(NQ / 4) * v.nface;
   const int64_t ntiles = (v.nel + kPeTile - 1) / kPeTile;
@@ -113,7 +113,7 @@ template <int NQ, bool CL>
 __global__ void __launch_bounds__(kPeTile, CL ? 1 : (NQ >= 20 ? 3 : 4))
     k_pe_resident(const __grid_constant__ PeView v, const int2* Hx) {
   constexpr int NQF = NQ / 4, RN = NQ / 2;
-  __shared__ __align__(16) int2 Hsh[RN * NQ];
+  __shared__ __align__(16) int2 Hsh[pe_operator_len(NQ)];
   __shared__ double red[kPeTile / 32];
   __shared__ double parts[CL ? 2 : 1][CL ? kPeCluster : 1];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(kPeTile, CL ? 1 : (NQ >= 20 ? 3 : 4))
     const int f = b < 2 ? v.own[b] : v.own[b - 2] ^ 1;
     Hsh[i] = Hx[j * NQ + f * NQF + c - b * NQF];
   }
+  for (int i = RN * NQ + tid; i < pe_operator_len(NQ); i += kPeTile) Hsh[i] = Hx[i];
   const int ntiles = (int)gridDim.x;
   const int64_t ne = v.nel, nface = v.nface, tlen = (int64_t)NQF * nface;
   const int64_t e = (int64_t)blockIdx.x * kPeTile + tid;
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(kPeTile, CL ? 1 : (NQ >= 20 ? 3 : 4))
   double uo[RN], gy[RN], w[NQF], jf[2] = {0.0, 0.0};
   int64_t fo[2] = {0, 0}, fi[2] = {0, 0};
   int eg = 1;
-  const int hs = *v.hs;
+  const int2 tc = Hx[RN * NQ];
 #pragma unroll
   for (int g = 0; g < NQF; ++g) w[g] = v.fw[g];
 #pragma unroll
@@ -158,30 +159,24 @@ __global__ void __launch_bounds__(kPeTile, CL ? 1 : (NQ >= 20 ? 3 : 4))
       double ui[RN];
 #pragma unroll
       for (int j = 0; j < RN; ++j) ui[j] = __ldcg(src + (j % NQF) * nface + fi[j / NQF]);
-      int emax = eg;
+      int ea[2] = {1, 1};
 #pragma unroll
-      for (int j = 0; j < RN; ++j) emax = max(emax, fx_exponent(uo[j]));
-#pragma unroll
-      for (int j = 0; j < RN; ++j) emax = max(emax, fx_exponent(ui[j]));
+      for (int j = 0; j < RN; ++j)
+        ea[j / NQF] = max(ea[j / NQF], max(fx_exponent(uo[j]), fx_exponent(ui[j])));
+      const int em = max(ea[0] + tc.x, ea[1] + tc.y);
       Limb x[NQ];
 #pragma unroll
       for (int j = 0; j < RN; ++j) {
-        x[j] = fx_split(fx_from_double(uo[j], emax));
-        x[RN + j] = fx_split(fx_from_double(ui[j], emax));
+        const int ej = em - (j < NQF ? tc.x : tc.y);
+        x[j] = fx_split(fx_from_double(uo[j], ej));
+        x[RN + j] = fx_split(fx_from_double(ui[j], ej));
       }
       double sq[2] = {0.0, 0.0};
+      const int* sc = reinterpret_cast<const int*>(Hsh + RN * NQ + 1);
 #pragma unroll
       for (int j = 0; j < RN; ++j) {
-        const int4* Hr = reinterpret_cast<const int4*>(Hsh + j * NQ);
-        Acc t(fx_from_double(gy[j], emax + hs));
-#pragma unroll
-        for (int c = 0; c < NQ; c += 2) {
-          const int4 h = Hr[c / 2];
-          t.mac(Cfx{h.x, h.y}, x[c]);
-          t.mac(Cfx{h.z, h.w}, x[c + 1]);
-        }
-        double acc = fx_value(t.get(), emax - 1078 + hs);
-        if (emax == 0x7ff) acc = __hiloint2double(0x7ff80000, 0);
+        double acc = pe_row<NQ>(Hsh + j * NQ, x, em + sc[j], gy[j]);
+        if (max(max(ea[0], ea[1]), eg) == 0x7ff) acc = __hiloint2double(0x7ff80000, 0);
         const int b = j / NQF, g = j - b * NQF;
         const double d = acc - uo[j];
         dst[g * nface + fo[b]] = acc;
@@ -303,27 +298,41 @@ cudaError_t launch_lp_pe_t(const LpPeView& v, const float* Hy32, cudaStream_t s)
 
 }  // namespace
 
-// The sweep rows of Hy in row order as fixed-point limbs (one block): Hy =
-// 2^(hs - 56) (h 2^28 + l), hs >= 0 the least with max |Hy| <= 2^(hs + 1), so
-// that a coefficient is below 2 and a row's sums of at most 28 products with
-// 56-bit values stay below 2^63.
-static __global__ void k_pe_limbs(int n_rows, int NQFS, const int* rows, const double* Hy, int2* Hx,
-                           int* hs) {
-  __shared__ int s_e;
-  if (threadIdx.x == 0) s_e = 0;
+// The sweep rows of Hy in row order as fixed-point limbs, equilibrated (one block):
+// t_a the exponent of the largest entry in the columns of axis a's faces, s_j then
+// the least with row j's largest entry below 2 and its sum of magnitudes below 32,
+// so that its sum with 56-bit values stays below 2^62.
+static __global__ void k_pe_limbs(int NQFS, const int* rows, const double* Hy, int2* Hx) {
+  __shared__ int s_t[2], s_s[kMaxQ * 2];
+  const int n_rows = NQFS / 2, tid = threadIdx.x;
+  if (tid < 2) s_t[tid] = kZeroGroup;
   __syncthreads();
-  int em = 0;
-  for (int i = threadIdx.x; i < n_rows * NQFS; i += blockDim.x)
-    em = max(em, fx_exponent(Hy[rows[i / NQFS] * NQFS + i % NQFS]));
-  atomicMax(&s_e, em);
+  for (int i = tid; i < n_rows * NQFS; i += blockDim.x) {
+    const double h = Hy[rows[i / NQFS] * NQFS + i % NQFS];
+    if (h != 0.0) atomicMax(&s_t[(i % NQFS) / n_rows], min(1000, max(-1000, ilogb(h))));
+  }
   __syncthreads();
-  const int s = max(0, s_e - 1023);            // |Hy| < 2^(s_e - 1022)
-  if (threadIdx.x == 0) *hs = s;
-  for (int i = threadIdx.x; i < n_rows * NQFS; i += blockDim.x) {
-    const long long c = __double2ll_rn(scalbn(Hy[rows[i / NQFS] * NQFS + i % NQFS], 56 - s));
-    const Limb x = fx_split(c);
+  auto entry = [&](int j, int c) {
+    const int t = s_t[c / n_rows];
+    return t == kZeroGroup ? 0.0 : Hy[rows[j] * NQFS + c] * fx_pow2(-t);
+  };
+  if (tid < n_rows) {
+    double mx = 0.0, sum = 0.0;
+    for (int c = 0; c < NQFS; ++c) {
+      mx = fmax(mx, fabs(entry(tid, c)));
+      sum += fabs(entry(tid, c));
+    }
+    s_s[tid] = mx > 0.0 ? max(ilogb(mx), ilogb(sum) + 1 - 5) : 0;
+  }
+  __syncthreads();
+  for (int i = tid; i < n_rows * NQFS; i += blockDim.x) {
+    const int j = i / NQFS;
+    const Limb x = fx_split(__double2ll_rn(scalbn(entry(j, i - j * NQFS), 56 - s_s[j])));
     Hx[i] = make_int2(x.h, x.l);
   }
+  int* scales = reinterpret_cast<int*>(Hx + n_rows * NQFS);
+  if (tid < 2) scales[tid] = s_t[tid];
+  if (tid < n_rows) scales[2 + tid] = s_s[tid];
 }
 
 // FP32 correction sweep, one thread per element (quadrilaterals, shared
@@ -349,11 +358,9 @@ cudaError_t launch_lp_sweep_pe(Ctx& c, const float* in, float* out) {
 }
 
 cudaError_t build_pe_operator(Ctx& c) {
-  cudaError_t e = dalloc_raw(c, (void**)&c.pe_hx, sizeof(int2) * c.n_rows * c.NQFS);
-  if (e == cudaSuccess) e = dalloc_raw(c, (void**)&c.pe_hs, sizeof(int));
+  cudaError_t e = dalloc_raw(c, (void**)&c.pe_hx, sizeof(int2) * pe_operator_len(c.NQFS));
   if (e != cudaSuccess) return e;
-  k_pe_limbs<<<1, 256, 0, c.stream>>>(c.n_rows, c.NQFS, c.rows, c.Hy,
-                                      reinterpret_cast<int2*>(c.pe_hx), c.pe_hs);
+  k_pe_limbs<<<1, 256, 0, c.stream>>>(c.NQFS, c.rows, c.Hy, reinterpret_cast<int2*>(c.pe_hx));
   return cudaGetLastError();
 }
 
@@ -369,7 +376,6 @@ PeView pe_view(const Ctx& c, double* fw_dev) {
   v.nface = c.nface;
   v.own[0] = c.rows_host[0] / c.Nqf;
   v.own[1] = c.rows_host[c.Nqf] / c.Nqf;
-  v.hs = c.pe_hs;
   v.elem_face = c.geo.elem_face;
   v.face_jf = c.geo.face_jf;
   v.fw = fw_dev;
