@@ -1033,6 +1033,8 @@ ehdg_status ehdg_create(const ehdg_mesh_desc* mesh, const ehdg_problem_desc* pro
   CKC(cudaMemcpyAsync(c.it_host, c.it, sizeof(IterState), cudaMemcpyDeviceToHost, c.stream));
   CKC(cudaStreamSynchronize(c.stream));
   if (c.it_host->status != 0) return cleanup(fail(EHDG_ERR_INVALID, "singular local operator"));
+  if (c.shared_op)
+    CKC(cudaMemcpy(c.fx_col, c.fx_col_d, sizeof(c.fx_col), cudaMemcpyDeviceToHost));
   if (c.pde == EHDG_TRANSPORT) {
     // face points with beta.n = 0 (average of both sides), finished after the sweep
     std::vector<int8_t> sg((size_t)trace);

@@ -1267,13 +1267,13 @@ cudaError_t BatchLoop::build(const std::vector<Ctx*>& ctxs, unsigned long long* 
     I.KE = c.KE;
     I.cn = (c.scheme == EHDG_CN) ? 1 : 0;
     I.ucoef = (c.scheme == EHDG_STEADY) ? 0.0 : 1.0 / c.dt_eff;
-    I.Px = FxOp{static_cast<const int2*>(c.fx_P), c.fx_Ps};
+    I.Px = fx_P(c);
     I.u = c.u;
     I.ey_idx = c.ey_idx;
     I.ey_val = c.ey_val;
     I.G = c.G;
-    I.Hx2 = FxOp{static_cast<const int2*>(c.fx_H), c.fx_Hs};
-    I.Eyx = FxOp{static_cast<const int2*>(c.fx_E), c.fx_Es};
+    I.Hx2 = fx_H(c);
+    I.Eyx = fx_Ey(c);
     I.uhat_n = c.uhat_n;
     I.gb = c.gb;
     I.gb_old = c.gb_old;

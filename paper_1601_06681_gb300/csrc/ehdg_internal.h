@@ -169,6 +169,8 @@ struct Ctx {
   // and, for shallow water, Hy as limbs with their scales
   void *fx_P = nullptr, *fx_H = nullptr, *fx_E = nullptr, *fx_Hy = nullptr;
   int *fx_Ps = nullptr, *fx_Hs = nullptr, *fx_Es = nullptr, *fx_Hys = nullptr;
+  int* fx_col_d = nullptr;
+  int fx_col[12] = {};           // scales of their groups of columns, three each
   bool use_pe = false;           // 2D shared-operator FP64 sweep, one thread per element
   double* pe_fw = nullptr;       // its face Gauss weights [Nqf]
   void* pe_hx = nullptr;         // its rows of Hy as fixed-point limbs, with their scales (pe_tile.cuh)

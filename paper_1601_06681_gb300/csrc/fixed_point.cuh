@@ -138,15 +138,19 @@ FX_INLINE long long fx_shift(long long v, int s) {
 }
 
 // A shared operator's rows as limbs in blocks of four rows, [rows / 4][cols][4]
-// (the last block zero-padded). The columns are in nf groups (the fields of the
-// state, which may differ in size by orders), and each row has a scale for each
-// group, scale[row * nf + f]: entry = 2^(scale - 56) (h 2^28 + l), the limbs'
-// value below 2 and its sum over the group below 32, so that a group's products
-// with 56-bit values sum below 2^62.
+// (the last block zero-padded), with scales of either sign: 2^col[a] for the
+// columns of group a (a field), and for each row one for each of
+// its ng groups of cols / ng columns whose values have units of their own (the
+// fields of the state), scale[row * ng + f]. entry = 2^(col + scale - 56) (h 2^28 +
+// l); with col divided out the limbs' value is below 2 and its sum over the group
+// below 32, so that a group's products with 56-bit values sum below 2^62.
 struct FxOp {
   const int2* x;
   const int* scale;
+  int col[3];
 };
+// a value that is not finite in the exponent of a set of values
+constexpr int kNotFinite = 1 << 16;
 // the scale of a group of columns that are zero, so low that its values do not
 // raise the others' unit
 constexpr int kZeroGroup = -4096;

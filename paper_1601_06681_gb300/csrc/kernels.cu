@@ -432,18 +432,36 @@ cudaError_t launch_face_signs(Ctx& c) {
 // Per-step right-hand side: G = P w, Gy = Ey G, Y0 = Ey u^n
 //   w = u^n / dt_eff + f (time-dependent) or w = f (steady)
 // ===========================================================================
-// A shared operator's matrix M [rows][cols] times coef as limbs (FxOp), one
-// block: the scales are the least with the group's largest entry below 2 and
-// its sum of magnitudes below 32. blocked: the layout of FxOp, else row-major.
-__global__ void k_fx_limbs(int rows, int cols, int nf, double coef, const double* M, int blocked,
-                           int2* x, int* scale) {
-  const int np = cols / nf, rows4 = blocked ? (rows + 3) / 4 * 4 : rows;
-  for (int i = threadIdx.x; i < rows4 * nf; i += blockDim.x) {
-    const int r = i / nf, f = i - r * nf;
+// A shared operator's matrix M [rows][cols] times coef as limbs (FxOp), one block.
+// Columns: nc groups with a scale each, the group of column c of row r being
+// idx[r * cols + c] / (n / nc) (idx null: c / (n / nc)), the scale its largest
+// entry's exponent. Rows: ng groups of columns; the scales are the least with the
+// group's largest entry below 2 and its sum of magnitudes below 32. blocked: the
+// layout of FxOp, else row-major.
+__global__ void k_fx_limbs(int rows, int cols, int ng, int nc, int n, const int* idx, double coef,
+                           const double* M, int blocked, int2* x, int* scale, int* col) {
+  __shared__ int s_col[3];
+  __shared__ double s_f[3];                     // coef over the group's scale
+  const int np = cols / ng, nf = n / nc, rows4 = blocked ? (rows + 3) / 4 * 4 : rows;
+  auto group = [&](int i) { return nc == 1 ? 0 : (idx ? idx[i] : i % cols) / nf; };
+  if (threadIdx.x < 3) s_col[threadIdx.x] = nc > 1 ? kZeroGroup : 0;
+  __syncthreads();
+  for (int i = threadIdx.x; i < (nc > 1 ? rows * cols : 0); i += blockDim.x)
+    if (M[i] != 0.0)
+      atomicMax(&s_col[group(i)], min(1000, max(-1000, ilogb(coef * M[i]))));
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    const int e = s_col[threadIdx.x];
+    col[threadIdx.x] = e;
+    s_f[threadIdx.x] = e == kZeroGroup ? 0.0 : coef * fx_pow2(-e);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < rows4 * ng; i += blockDim.x) {
+    const int r = i / ng, f = i - r * ng;
     double mx = 0.0, sum = 0.0;
     if (r < rows)
       for (int c = f * np; c < (f + 1) * np; ++c) {
-        const double v = fabs(coef * M[r * cols + c]);
+        const double v = fabs(s_f[group(r * cols + c)] * M[r * cols + c]);
         mx = fmax(mx, v);
         sum += v;
       }
@@ -452,31 +470,49 @@ __global__ void k_fx_limbs(int rows, int cols, int nf, double coef, const double
   __syncthreads();
   for (int i = threadIdx.x; i < rows4 * cols; i += blockDim.x) {
     const int r = i / cols, c = i - r * cols;
-    const double v = r < rows ? coef * M[r * cols + c] : 0.0;
-    const Limb l = fx_split(__double2ll_rn(scalbn(v, 56 - scale[r * nf + c / np])));
+    const double v = r < rows ? s_f[group(i)] * M[i] : 0.0;
+    const Limb l = fx_split(__double2ll_rn(scalbn(v, 56 - scale[r * ng + c / np])));
     x[blocked ? ((r / 4) * (int64_t)cols + c) * 4 + r % 4 : i] = make_int2(l.h, l.l);
   }
 }
 
+// Groups of P: the fields of the state, whose products are summed apart. Of Ey's
+// columns: the fields (a row is (phi + sqrt(Phi) vel.n) / 2, with phi about
+// sqrt(Phi) times vel).
 cudaError_t build_fx_operators(Ctx& c) {
-  auto make = [&](int rows, int cols, int nf, double coef, const double* M, bool blocked,
-                  void** x, int** scale) {
+  cudaError_t e = dalloc_raw(c, (void**)&c.fx_col_d, sizeof(c.fx_col));
+  if (e == cudaSuccess) e = cudaMemsetAsync(c.fx_col_d, 0, sizeof(c.fx_col), c.stream);
+  int at = 0;
+  auto make = [&](int rows, int cols, int ng, int nc, int n, const int* idx, double coef,
+                  const double* M, bool blocked, void** x, int** scale) {
     const int r4 = blocked ? (rows + 3) / 4 * 4 : rows;
-    cudaError_t e = dalloc_raw(c, x, sizeof(int2) * r4 * cols);
-    if (e == cudaSuccess) e = dalloc_raw(c, (void**)scale, sizeof(int) * r4 * nf);
-    if (e != cudaSuccess) return e;
-    k_fx_limbs<<<1, 512, 0, c.stream>>>(rows, cols, nf, coef, M, blocked ? 1 : 0,
-                                        static_cast<int2*>(*x), *scale);
-    return cudaGetLastError();
+    if (e == cudaSuccess) e = dalloc_raw(c, x, sizeof(int2) * r4 * cols);
+    if (e == cudaSuccess) e = dalloc_raw(c, (void**)scale, sizeof(int) * r4 * ng);
+    if (e != cudaSuccess) return;
+    k_fx_limbs<<<1, 512, 0, c.stream>>>(rows, cols, ng, nc, n, idx, coef, M, blocked ? 1 : 0,
+                                        static_cast<int2*>(*x), *scale, c.fx_col_d + 3 * at++);
+    e = cudaGetLastError();
   };
   const double uc = c.scheme == EHDG_STEADY ? 1.0 : 1.0 / c.dt_eff;
-  cudaError_t e = make(c.n, c.n, c.nf, uc, c.P, true, &c.fx_P, &c.fx_Ps);
-  if (e == cudaSuccess) e = make(c.n, c.NQFS, 1, 1.0, c.H, true, &c.fx_H, &c.fx_Hs);
-  if (e == cudaSuccess) e = make(c.NQFS, c.KE, 1, 1.0, c.ey_val, false, &c.fx_E, &c.fx_Es);
-  if (e == cudaSuccess && c.pde == EHDG_SW_LINEAR)
-    e = make(c.NQFS, c.NQFS, 1, 1.0, c.Hy, false, &c.fx_Hy, &c.fx_Hys);
+  const int nq = c.NQFS;
+  make(c.n, c.n, c.nf, 1, c.n, nullptr, uc, c.P, true, &c.fx_P, &c.fx_Ps);
+  make(c.n, nq, 1, 1, nq, nullptr, 1.0, c.H, true, &c.fx_H, &c.fx_Hs);
+  make(nq, c.KE, 1, c.nf, c.n, c.ey_idx, 1.0, c.ey_val, false, &c.fx_E, &c.fx_Es);
+  if (c.pde == EHDG_SW_LINEAR)
+    make(nq, nq, 1, 1, nq, nullptr, 1.0, c.Hy, false, &c.fx_Hy, &c.fx_Hys);
   return e;
 }
+
+// the operators as kernel arguments
+static FxOp fx_op(const Ctx& c, const void* x, const int* scale, int i) {
+  FxOp o = {static_cast<const int2*>(x), scale, {}};
+  std::copy(c.fx_col + 3 * i, c.fx_col + 3 * i + 3, o.col);
+  return o;
+}
+FxOp fx_P(const Ctx& c) { return fx_op(c, c.fx_P, c.fx_Ps, 0); }
+FxOp fx_H(const Ctx& c) { return fx_op(c, c.fx_H, c.fx_Hs, 1); }
+FxOp fx_Ey(const Ctx& c) { return fx_op(c, c.fx_E, c.fx_Es, 2); }
+FxOp fx_Hy(const Ctx& c) { return fx_op(c, c.fx_Hy, c.fx_Hys, 3); }
 
 // Tile of 32 consecutive elements (threadIdx.x) x kStepT row groups
 // (threadIdx.y); persistent over tiles. w and G of the tile live in shared
@@ -540,8 +576,8 @@ cudaError_t launch_step(Ctx& c) {
   s.KE = c.KE;
   s.shared = c.shared_op ? 1 : 0;
   s.fcoef = (c.scheme == EHDG_STEADY) ? 1.0 : c.dt_eff;
-  s.Px = FxOp{static_cast<const int2*>(c.fx_P), c.fx_Ps};
-  s.Eyx = FxOp{static_cast<const int2*>(c.fx_E), c.fx_Es};
+  s.Px = fx_P(c);
+  s.Eyx = fx_Ey(c);
   s.ucoef = (c.scheme == EHDG_STEADY) ? 0.0 : 1.0 / c.dt_eff;
   s.have_force = c.have_force ? 1 : 0;
   s.force_avg = (c.scheme == EHDG_CN) ? 1 : 0;
@@ -666,6 +702,7 @@ __global__ void __launch_bounds__(128) k_elem_fx(const __grid_constant__ ElemPar
   for (int i = threadIdx.x; i < NQ * NQ; i += 128) Hsh[i] = p.Hx.x[i];
   for (int i = threadIdx.x; i < NQ; i += 128) s_scale[i] = p.Hx.scale[i];
   __syncthreads();
+  const int t0 = p.Hx.col[0], t1 = p.Hx.col[1];        // scales of the axes' columns
   const int64_t ne = p.nel;
   const double* src = p.uhat + (int64_t)(p.it->k & 1) * NQF * p.nface;
   for (int64_t e = blockIdx.x * 128LL + threadIdx.x; e < ne; e += gridDim.x * 128LL) {
@@ -675,17 +712,19 @@ __global__ void __launch_bounds__(128) k_elem_fx(const __grid_constant__ ElemPar
     for (int f = 0; f < 4; ++f) face[f] = p.elem_face[f * ne + e];
 #pragma unroll
     for (int j = 0; j < NQ; ++j) gy[j] = p.Gy[j * ne + e];
-    int em = 1;
+    int ea[2] = {1, 1};
 #pragma unroll
     for (int f = 0; f < 4; ++f)
 #pragma unroll
       for (int g = 0; g < NQF; ++g) {
         u[f * NQF + g] = src[g * p.nface + face[f]];
-        em = max(em, fx_exponent(u[f * NQF + g]));
+        ea[f / 2] = max(ea[f / 2], fx_exponent(u[f * NQF + g]));
       }
+    const int em = max(ea[0] + t0, ea[1] + t1);
     Limb x[NQ];
 #pragma unroll
-    for (int c = 0; c < NQ; ++c) x[c] = fx_split(fx_from_double(u[c], em));
+    for (int c = 0; c < NQ; ++c)
+      x[c] = fx_split(fx_from_double(u[c], em - (c < NQ / 2 ? t0 : t1)));
 #pragma unroll
     for (int j = 0; j < NQ; ++j) {
       const int4* Hr = reinterpret_cast<const int4*>(Hsh + j * NQ);
@@ -696,8 +735,8 @@ __global__ void __launch_bounds__(128) k_elem_fx(const __grid_constant__ ElemPar
         t.mac(Cfx{h.x, h.y}, x[c]);
         t.mac(Cfx{h.z, h.w}, x[c + 1]);
       }
-      const double y = em == 0x7ff ? __hiloint2double(0x7ff80000, 0)
-                                   : fx_value(t.get(), em - 1078 + s_scale[j]);
+      const double y = max(ea[0], ea[1]) == 0x7ff ? __hiloint2double(0x7ff80000, 0)
+                                                  : fx_value(t.get(), em - 1078 + s_scale[j]);
       p.Y[(int64_t)j * ne + e] = gy[j] + y;
     }
   }
@@ -737,7 +776,7 @@ cudaError_t launch_elem(Ctx& c) {
   p.Gy = c.Gy;
   p.Hy = c.Hy;
   p.Y = c.Y;
-  p.Hx = FxOp{static_cast<const int2*>(c.fx_Hy), c.fx_Hys};
+  p.Hx = fx_Hy(c);
   if (c.fx_Hy) {   // every shallow-water shape (p <= 5)
     switch (c.NQFS) {
       case 8: return launch_elem_fx<8>(p, c.stream);
@@ -1120,7 +1159,7 @@ cudaError_t launch_final(Ctx& c) {
   p.it = c.it;
   p.G = c.G;
   p.H = c.H;
-  p.Hx = FxOp{static_cast<const int2*>(c.fx_H), c.fx_Hs};
+  p.Hx = fx_H(c);
   p.u = c.u;
   cudaError_t err;
   if (c.use_ozaki && c.oz_final.img) {

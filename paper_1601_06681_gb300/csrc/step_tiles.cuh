@@ -55,28 +55,43 @@ struct StepParams {
   const int* warm;
 };
 
-// the largest biased exponent over a tile's warps of each lane's values, >= 1
+// the operators of a context as kernel arguments (kernels.cu)
+FxOp fx_P(const Ctx& c);
+FxOp fx_H(const Ctx& c);
+FxOp fx_Ey(const Ctx& c);
+FxOp fx_Hy(const Ctx& c);
+
+// the largest over a tile's warps of each lane's values
 __device__ __forceinline__ int tile_max(int v) {
   __shared__ int s_max[kStepT][32];
   s_max[threadIdx.y][threadIdx.x] = v;
   __syncthreads();
-  int m = 1;
+  int m = v;
 #pragma unroll
   for (int t = 0; t < kStepT; ++t) m = max(m, s_max[t][threadIdx.x]);
   __syncthreads();
   return m;
 }
 
-// values v[c * 32] (c0 <= c < c1) of a lane to packed limbs in place, in units
-// of 2^(emax - 1078); returns emax (0x7ff: a value is not finite)
-__device__ __forceinline__ int tile_limbs(double* v, int c0, int c1) {
+// n values v[c * 32] of a lane (COL: in up to three groups of np, times 2^col of
+// their group) to packed limbs in place, in units of 2^(emax - 1078); returns emax
+// (kNotFinite: a value is not finite)
+template <bool COL>
+__device__ __forceinline__ int tile_limbs(double* v, int n, int np, const int (&col)[3]) {
   const int lane = threadIdx.x, t = threadIdx.y;
-  int em = 1;
-  for (int c = c0 + t; c < c1; c += kStepT) em = max(em, fx_exponent(v[c * 32 + lane]));
+  auto scale = [&](int c) {
+    return !COL ? 0 : (c < np ? col[0] : (c < 2 * np ? col[1] : col[2]));
+  };
+  int em = -kNotFinite;
+  for (int c = t; c < n; c += kStepT) {
+    const int e = fx_exponent(v[c * 32 + lane]);
+    em = max(em, e == 0x7ff ? kNotFinite : max(e, 1) + scale(c));
+  }
   em = tile_max(em);
-  long long* x = reinterpret_cast<long long*>(v);
-  for (int c = c0 + t; c < c1; c += kStepT)
-    x[c * 32 + lane] = fx_pack(fx_split(fx_from_double(v[c * 32 + lane], em)));
+  for (int c = t; c < n; c += kStepT) {
+    double& x = v[c * 32 + lane];
+    x = __longlong_as_double(fx_pack(fx_split(fx_from_double(x, em - scale(c)))));
+  }
   __syncthreads();
   return em;
 }
@@ -97,7 +112,7 @@ __device__ __forceinline__ void tile_rows4(const FxOp& op, const int2* osh, cons
     if (f >= nf) break;
     long long y[4];
     fx_rows4(osh + ((int64_t)b * cols + f * np) * 4, x + f * np * 32, np, y);
-    nan |= em[f] == 0x7ff;
+    nan |= em[f] == kNotFinite;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int Lf = em[f] - 1078 + sc[i * nf + f];
@@ -150,7 +165,7 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
       int em[3] = {1, 1, 1};
 #pragma unroll
       for (int f = 0; f < 3; ++f)
-        if (f < s.nf) em[f] = tile_limbs(w, f * np, (f + 1) * np);
+        if (f < s.nf) em[f] = tile_limbs<false>(w + f * np * 32, np, np, s.Px.col);
       for (int b = t; b * 4 < n; b += kStepT) {
         double v[4];
         tile_rows4(s.Px, Psh, w, b, n, s.nf, em, v);
@@ -231,7 +246,7 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
     return;
   }
   const bool limbs = SHARED && !s.g_ready;
-  const int ge = limbs ? tile_limbs(g, 0, n) : 0;
+  const int ge = limbs ? tile_limbs<true>(g, n, n / s.nf, s.Eyx.col) : 0;
   if (!live) return;
   // the rows the sweep computes (upwind and tangential points; every point
   // for shallow water): Gy in the sweep's slot order, and the element
@@ -248,7 +263,7 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
         const int2 c = s.Eyx.x[r * s.KE + k2];
         a.mac(Cfx{c.x, c.y}, fx_limb(gx[s.ey_idx[r * s.KE + k2] * 32]));
       }
-      s.Gy[j * ne + e] = ge == 0x7ff ? __hiloint2double(0x7ff80000, 0)
+      s.Gy[j * ne + e] = ge == kNotFinite ? __hiloint2double(0x7ff80000, 0)
                                      : fx_value(a.get(), ge - 1078 + s.Eyx.scale[r]);
       if (want_y0) {
         for (int k2 = 0; k2 < s.KE; ++k2)
@@ -301,7 +316,7 @@ __device__ __forceinline__ void final_tile(const FinalParams& p, const int2* Hsh
   }
   __syncthreads();
   if (p.shared) {
-    const int em[3] = {tile_limbs(uh, 0, p.NQFS), 1, 1};
+    const int em[3] = {tile_limbs<true>(uh, p.NQFS, 2 * p.Nqf, p.Hx.col), 1, 1};
     for (int b = t; b * 4 < p.n; b += kStepT) {
       double g[4];
 #pragma unroll

@@ -70,3 +70,28 @@ def test_quadrilateral_traces_keep_their_own_digits(p, beta, dt, axis):
     uh, _, uh_ref, _ = two_sweeps((6, 5), p, beta, dt, axis)
     assert 0 < np.abs(uh_ref[uh_ref != 0]).min() < 1e-7
     assert worst(uh, uh_ref) < TOL
+
+
+@pytest.mark.parametrize("p", [1, 3, 5])
+@pytest.mark.parametrize("k", [0, 23])
+def test_shallow_water_fields_of_different_size(p, k):
+    """With Phi = 4^k the wave speed is 2^k and phi is 2^k times the velocities: the
+    problem with Phi = 1 in other units, so its fields and traces are the oracle's
+    there times powers of two. 2^23 is far beyond a geopotential of 1e5 m^2/s^2, and
+    a sum that holds the velocities in units of phi's last place shows there.
+    Tolerance 1e-12, the FP64 parity bound, per field."""
+    from oracle.ehdg import Problem
+    mesh = W.structured_mesh((6, 5), boundary_tag=W.TAG_WALL)
+    dt, c = 2.0 ** -9, 2.0 ** k
+    prob = Problem(mesh, p, pde="sw", scheme="be", dt=dt, Phi=1.0)
+    u0 = np.random.default_rng(2).standard_normal((prob.nel, 3, prob.Np))
+    u_ref, uh_ref, _ = prob.solve_step(u0, prob.trace(u0), fixed_iters=3)
+    scale = np.array([c, 1.0, 1.0])[None, :, None]
+    with E.Solver(mesh, p, pde="sw", scheme="be", dt=dt / c, Phi=c * c) as s:
+        s.set_state(u0 * scale)
+        s.step_fixed(3)
+        u, uh = s.get_state()
+    u, uh = u / scale, uh / c
+    assert np.linalg.norm(uh - uh_ref) < TOL * np.linalg.norm(uh_ref)
+    for f in range(3):
+        assert np.linalg.norm(u[:, f] - u_ref[:, f]) < TOL * np.linalg.norm(u_ref[:, f])
