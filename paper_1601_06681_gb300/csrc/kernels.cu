@@ -478,7 +478,8 @@ __global__ void k_fx_limbs(int rows, int cols, int ng, int nc, int n, const int*
 
 // Groups of P: the fields of the state, whose products are summed apart. Of Ey's
 // columns: the fields (a row is (phi + sqrt(Phi) vel.n) / 2, with phi about
-// sqrt(Phi) times vel).
+// sqrt(Phi) times vel). Of H's and Hy's columns: the axes, whose faces' traces enter
+// with |beta_a| / h_a.
 cudaError_t build_fx_operators(Ctx& c) {
   cudaError_t e = dalloc_raw(c, (void**)&c.fx_col_d, sizeof(c.fx_col));
   if (e == cudaSuccess) e = cudaMemsetAsync(c.fx_col_d, 0, sizeof(c.fx_col), c.stream);
@@ -496,10 +497,10 @@ cudaError_t build_fx_operators(Ctx& c) {
   const double uc = c.scheme == EHDG_STEADY ? 1.0 : 1.0 / c.dt_eff;
   const int nq = c.NQFS;
   make(c.n, c.n, c.nf, 1, c.n, nullptr, uc, c.P, true, &c.fx_P, &c.fx_Ps);
-  make(c.n, nq, 1, 1, nq, nullptr, 1.0, c.H, true, &c.fx_H, &c.fx_Hs);
+  make(c.n, nq, 1, c.dim, nq, nullptr, 1.0, c.H, true, &c.fx_H, &c.fx_Hs);
   make(nq, c.KE, 1, c.nf, c.n, c.ey_idx, 1.0, c.ey_val, false, &c.fx_E, &c.fx_Es);
   if (c.pde == EHDG_SW_LINEAR)
-    make(nq, nq, 1, 1, nq, nullptr, 1.0, c.Hy, false, &c.fx_Hy, &c.fx_Hys);
+    make(nq, nq, 1, c.dim, nq, nullptr, 1.0, c.Hy, false, &c.fx_Hy, &c.fx_Hys);
   return e;
 }
 

@@ -72,6 +72,17 @@ def test_quadrilateral_traces_keep_their_own_digits(p, beta, dt, axis):
     assert worst(uh, uh_ref) < TOL
 
 
+@pytest.mark.parametrize("p,beta,dt,axis", [
+    (1, (0.8, 0.35), 1e-8, None),
+    (6, (-0.8, -0.35), 1e-8, None),
+    (4, (0.8, 1e-7), 1e-2, 1),
+    (3, (-1e-7, 0.6), 1e-2, 0),
+])
+def test_quadrilateral_values_keep_their_own_digits(p, beta, dt, axis):
+    _, u, _, u_ref = two_sweeps((6, 5), p, beta, dt, axis)
+    assert worst(u, u_ref) < TOL
+
+
 @pytest.mark.parametrize("p", [1, 3, 5])
 @pytest.mark.parametrize("k", [0, 23])
 def test_shallow_water_fields_of_different_size(p, k):
