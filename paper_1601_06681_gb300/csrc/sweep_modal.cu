@@ -25,12 +25,16 @@
 // The sweep forms them in fixed point on the integer pipe. The FP64 pipe
 // issues 1.6 operations per clock and SM, the integer pipe 57 multiply-adds
 // 32 x 32 + 64 (both measured); three of these make one product of 56-bit
-// numbers held as two limbs. Per element all traces and Gy are aligned to one
-// power of two, chosen from their largest magnitude, with IB = 55 or 56 bits
-// (one or two more than a double's rounding leaves of the largest value), and
-// the coefficients are rounded to 2^-56. Rounding errors of the element's
-// values are then at most a few 2^-56 of its largest trace, where a double
-// accumulation leaves 2^-53 of the partial sums. Traces live in HBM between
+// numbers held as two limbs. The equation is divided by sigma = tau + sum c. Of a
+// lift's coefficient c_a / sigma l, far below one where dt is small or the velocity
+// runs nearly along the axis's faces, the power of two goes to the traces (md_fill),
+// and the element's values are aligned to one power of two, in which the largest
+// scaled trace has IB = 54 to 56 bits and Gy and the outflow traces 57; the
+// coefficients are rounded to 2^-56. Rounding errors of the unknowns are then at most
+// a few 2^-IB of the element's largest lift, or 2^-57 of its largest outflow, where a
+// double accumulation leaves 2^-53 of the partial sums. (Without the scales t_a,
+// which cost 1% to 2% of a step, an element fed from rest at dt = 1e-8 lost 1e-10 of
+// its values.) Traces live in HBM between
 // sweeps as 62-bit integers with one exponent per block of 2 x 2 coefficients.
 // The sums of squares of the residual are exact integers.
 //
@@ -43,6 +47,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <vector>
 
@@ -121,7 +126,8 @@ struct FxParams {
   int64_t nel;
   const int32_t* elem_face;
   int fin[3], fout[3];
-  int ib;                        // bits of the element's largest input
+  int ib;                        // bits of the element's largest scaled trace
+  int t[3];                      // scales of the axes' lifts (md_fill)
   double fw[3];                  // J_f of each axis's faces
   Cfx clx[P1], crx[P1], rx[P1];  // first axis
   Cfx cl[2][4], cr[2][4], r[4];  // second and third axes, padded index
@@ -339,12 +345,26 @@ __device__ __forceinline__ void md_transform(double (&x)[P1 * P1 * P1],
     }
 }
 
-// an element's faces, its exponents and the unit of its values
+// an element's faces, its exponents and the unit 2^L of its values: the finest in
+// which the largest trace times its axis's 2^t has p.ib bits, and Gy and the outflow
+// traces, which are not scaled, have 57
 struct FxElem {
   unsigned e8, fi[3], fo[3];                   // byte offsets of the first coefficients
   unsigned long long ei[3], eo[3], eg[3];
-  int top, L;                                  // values in units of 2^L: the largest has p.ib bits
+  int L;
+  bool nan;                                    // an input is not finite
 };
+
+// the larger exponent fields of two words
+__device__ __forceinline__ unsigned long long fx_max(unsigned long long a, unsigned long long b) {
+  return (unsigned long long)__vmaxs2((unsigned)(a >> 32), (unsigned)(b >> 32)) << 32 |
+         __vmaxs2((unsigned)a, (unsigned)b);
+}
+// the largest field of a word
+__device__ __forceinline__ int fx_top(unsigned long long a) {
+  const unsigned m = __vmaxs2((unsigned)a, (unsigned)(a >> 32));
+  return max((int)(short)m, (int)(short)(m >> 16));
+}
 
 template <int P1, bool CG>
 __device__ __forceinline__ FxElem fx_element(const FxParams<P1>& p, int64_t e,
@@ -357,19 +377,19 @@ __device__ __forceinline__ FxElem fx_element(const FxParams<P1>& p, int64_t e,
     x.fi[a] = 8u * (unsigned)p.elem_face[p.fin[a] * ne + e];
     x.fo[a] = 8u * (unsigned)p.elem_face[p.fout[a] * ne + e];
   }
-  unsigned m0 = 0x80008000u, m1 = 0x80008000u;
+  int top = INT_MIN;
+  unsigned long long out = kExpAllZero;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     x.ei[a] = fx_ld<CG>(esrc, x.fi[a]);
     x.eo[a] = fx_ld<CG>(esrc, x.fo[a]);
     x.eg[a] = fx_at(p.tr.Ge + a * ne, x.e8);
-    m0 = __vmaxs2(__vmaxs2(m0, (unsigned)x.ei[a]), __vmaxs2((unsigned)x.eo[a], (unsigned)x.eg[a]));
-    m1 = __vmaxs2(__vmaxs2(m1, (unsigned)(x.ei[a] >> 32)),
-                  __vmaxs2((unsigned)(x.eo[a] >> 32), (unsigned)(x.eg[a] >> 32)));
+    top = max(top, fx_top(fx_max(x.ei[a], x.eo[a])) + p.t[a]);
+    out = fx_max(out, fx_max(x.eo[a], x.eg[a]));
   }
-  m0 = __vmaxs2(m0, m1);
-  x.top = max((int)(short)m0, (int)(short)(m0 >> 16));
-  x.L = x.top + 62 - p.ib;
+  const int eo = fx_top(out);
+  x.L = max(top + 62 - p.ib, eo + 5);
+  x.nan = max(top, eo) > kExpHigh;
   return x;
 }
 
@@ -382,7 +402,9 @@ __device__ __forceinline__ void fx_solve(const FxParams<P1>& p, const FxElem& el
   using B = MdBlocks<P1>;
   using S = FxShape<P1>;
   constexpr int NG = S::NG, OFF = S::OFF;
-  const int J = role % NG, K = role / NG, L = el.L;
+  const int J = role % NG, K = role / NG;
+  // units of the axes' traces, which enter times 2^t
+  const int L0 = el.L - p.t[0], L1 = el.L - p.t[1], L2 = el.L - p.t[2];
   const int64_t nface = p.tr.nface;
   const unsigned(&fi)[3] = el.fi, (&fo)[3] = el.fo;
   const unsigned long long(&ei)[3] = el.ei, (&eo)[3] = el.eo;
@@ -391,7 +413,7 @@ __device__ __forceinline__ void fx_solve(const FxParams<P1>& p, const FxElem& el
   {
     Limb xi[4], xo[4];
     const int b0 = J + 2 * K;
-    const Align ai(L, fx_field(ei[0], b0)), ao(L, fx_field(eo[0], b0));
+    const Align ai(L0, fx_field(ei[0], b0)), ao(L0, fx_field(eo[0], b0));
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int j = 2 * J + (u & 1) - OFF, k = 2 * K + (u >> 1) - OFF;
@@ -403,8 +425,8 @@ __device__ __forceinline__ void fx_solve(const FxParams<P1>& p, const FxElem& el
 #pragma unroll (SOLO || P1 == 4 ? 1 : P1)
     for (int i = 0; i < P1; ++i) {
       const int by = S::group(i) + 2 * K, bz = S::group(i) + 2 * J;
-      const Align yi(L, fx_field(ei[1], by)), yo(L, fx_field(eo[1], by));
-      const Align zi(L, fx_field(ei[2], bz)), zo(L, fx_field(eo[2], bz));
+      const Align yi(L1, fx_field(ei[1], by)), yo(L1, fx_field(eo[1], by));
+      const Align zi(L2, fx_field(ei[2], bz)), zo(L2, fx_field(eo[2], bz));
       Limb ty[2][2], tz[2][2];                  // [in, out][index in the group]
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
@@ -553,7 +575,7 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
     const unsigned e8 = el.e8;
     const unsigned(&fo)[3] = el.fo;
     const unsigned long long(&eo)[3] = el.eo, (&eg)[3] = el.eg;
-    const int top = el.top, L = el.L;
+    const int L = el.L;
 
     double r = 0.0;
 #pragma unroll 1
@@ -584,7 +606,7 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
       const int sh = __clzll((long long)any) - 2;
       int ex = L - sh;
       if (any == 0 || ex < kExpLow) ex = kExpZero;
-      if (ex > kExpHigh || top == kExpNan) ex = kExpNan;
+      if (ex > kExpHigh || el.nan) ex = kExpNan;
       if (live) {
 #pragma unroll
         for (int t = 0; t < 4; ++t)
@@ -657,7 +679,7 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
     }
     if (live) {
       const double sc = fx_pow2(max(-1022, min(1023, L)));
-      res = top == kExpNan ? __hiloint2double(0x7ff80000, 0) : fma(r * sc, sc, res);
+      res = el.nan ? __hiloint2double(0x7ff80000, 0) : fma(r * sc, sc, res);
     }
   }
   if (!PERSIST) {
@@ -780,7 +802,7 @@ __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 :
       long long& m = at(c % P1, (c / P1) % P1, c / N2);
       const Limb x = fx_limb(m);
       double v = fx_value(((long long)x.h << kW) + x.l, el.L);
-      if (el.top == kExpNan) v = __hiloint2double(0x7ff80000, 0);
+      if (el.nan) v = __hiloint2double(0x7ff80000, 0);
       m = __double_as_longlong(v + s.G[c * ne + e]);
     }
     sync();
@@ -1133,13 +1155,13 @@ bool md_block_inverse(int n, const Md1D& t, const ld (&ca)[3], ld tau, const int
   return invert(m, A, X);
 }
 
-// Bounds, for traces and Gy of magnitude at most one in every coefficient, of
+// Bounds, for scaled traces of magnitude at most one in every coefficient, of
 // what the fixed-point sweep forms: the right-hand side of each diagonal block
 // (A_bb v_b, split into limbs), the outflow coefficients without Gy, and the
 // largest sum of magnitudes in an accumulator of the lifts and couplings.
 // H = A^{-1} L exactly bounds v; A is upper block triangular.
-void md_bounds(int n, const Md1D& t, const ld (&ca)[3], ld tau, ld sigma, std::vector<double>* rhs,
-               double* out, double* sum) {
+void md_bounds(int n, const Md1D& t, const ld (&ca)[3], const ld (&lift)[3], ld tau, ld sigma,
+               std::vector<double>* rhs, double* out, double* sum) {
   const int n2 = n * n, N = n * n2, M = 6 * n2;
   std::vector<double> A((size_t)N * N, 0.0), H((size_t)N * M, 0.0), labs(N, 0.0);
   auto at = [&](int a, int i, int t1, int t2) {
@@ -1149,10 +1171,9 @@ void md_bounds(int n, const Md1D& t, const ld (&ca)[3], ld tau, ld sigma, std::v
     for (int g = 0; g < n2; ++g)
       for (int i = 0; i < n; ++i) {
         const int row = at(a, i, g % n, g / n);
-        H[(size_t)row * M + 2 * a * n2 + g] = (double)(ca[a] * t.l[i] / sigma);
-        H[(size_t)row * M + (2 * a + 1) * n2 + g] = (double)(ca[a] * t.r[i] / sigma);
-        labs[row] += std::fabs((double)(ca[a] * t.l[i] / sigma)) +
-                     std::fabs((double)(ca[a] * t.r[i] / sigma));
+        H[(size_t)row * M + 2 * a * n2 + g] = (double)(lift[a] * t.l[i]);
+        H[(size_t)row * M + (2 * a + 1) * n2 + g] = (double)(lift[a] * t.r[i]);
+        labs[row] += std::fabs((double)(lift[a] * t.l[i])) + std::fabs((double)(lift[a] * t.r[i]));
         for (int c = 0; c < n; ++c)
           A[(size_t)row * N + at(a, c, g % n, g / n)] += (double)(ca[a] * t.T[i * n + c] / sigma);
       }
@@ -1213,7 +1234,7 @@ void md_bounds(int n, const Md1D& t, const ld (&ca)[3], ld tau, ld sigma, std::v
       }
       for (int i = 0; i < n; ++i) m += std::fabs((double)t.r[i]) * v[at(a, i, g % n, g / n)];
       *out = std::max(*out, s);
-      *sum = std::max(*sum, m + 1.0);
+      *sum = std::max(*sum, m);
     }
 }
 
@@ -1284,7 +1305,15 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
   }
   // sigma makes the fixed-point coefficients and values of order one
   const ld sigma = tau + ca[0] + ca[1] + ca[2];
+  // The lifts of axis a go with c_a / sigma, far below one for a small time step or
+  // a velocity nearly along the axis's faces: 2^t_a goes to the traces, the
+  // coefficients lift_a l and lift_a r keep their bits (1/8 <= lift_a where t_a < 0).
   bool fits = sigma > 0.0L;
+  ld lift[3] = {0.0L, 0.0L, 0.0L};
+  for (int a = 0; a < 3 && fits; ++a) {
+    x->t[a] = std::max(-4096, std::min(0, std::ilogb(ca[a] / sigma) + 3));
+    lift[a] = std::ldexp(ca[a] / sigma, -x->t[a]);
+  }
   auto fix = [&](ld v) {
     if (!(std::fabs(v) < 7.9L)) {
       fits = false;
@@ -1300,8 +1329,8 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
     const bool ok = j >= 0 && j < P1;
     x->r[i] = ok ? fix(t.r[j]) : Cfx{0, 0};
     for (int a = 0; a < 2; ++a) {
-      x->cl[a][i] = ok ? fix(ca[1 + a] * t.l[j] / sigma) : Cfx{0, 0};
-      x->cr[a][i] = ok ? fix(ca[1 + a] * t.r[j] / sigma) : Cfx{0, 0};
+      x->cl[a][i] = ok ? fix(lift[1 + a] * t.l[j]) : Cfx{0, 0};
+      x->cr[a][i] = ok ? fix(lift[1 + a] * t.r[j]) : Cfx{0, 0};
       for (int c = 0; c < 2; ++c)
         if (i < 2)
           x->T[a][i][c] = ok && S::NG > 1 ? fix(-ca[1 + a] * t.T[j * P1 + 2 + c - S::OFF] / sigma)
@@ -1310,8 +1339,8 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
   }
   for (int i = 0; i < P1; ++i) {
     x->rx[i] = fix(t.r[i]);
-    x->clx[i] = fix(ca[0] * t.l[i] / sigma);
-    x->crx[i] = fix(ca[0] * t.r[i] / sigma);
+    x->clx[i] = fix(lift[0] * t.l[i]);
+    x->crx[i] = fix(lift[0] * t.r[i]);
     for (int j = 0; j < P1; ++j)
       x->Tx[i][j] = i < j ? fix(-ca[0] * t.T[i * P1 + j] / sigma) : Cfx{0, 0};
   }
@@ -1319,8 +1348,8 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
   const int N3 = P1 * P1 * P1;
   std::vector<double> rhs_bound(N3, 0.0);
   double out_bound = 0.0, sum_bound = 0.0;
-  md_bounds(P1, t, ca, tau, sigma, &rhs_bound, &out_bound, &sum_bound);
-  double split_bound = out_bound + 1.0;             // what must fit two limbs
+  md_bounds(P1, t, ca, lift, tau, sigma, &rhs_bound, &out_bound, &sum_bound);
+  double split_bound = out_bound;                   // what must fit two limbs
   for (int I = 0; I < B::NB; ++I)
     for (int J = 0; J < B::NB; ++J)
       for (int K = 0; K < B::NB; ++K) {

@@ -83,6 +83,19 @@ def test_quadrilateral_values_keep_their_own_digits(p, beta, dt, axis):
     assert worst(u, u_ref) < TOL
 
 
+@pytest.mark.parametrize("p,beta,dt,axis", [
+    (1, (0.8, 0.35, -0.5), 1e-8, None),
+    (2, (-0.8, 0.35, 0.5), 1e-8, None),
+    (3, (0.8, -0.35, 0.5), 1e-8, None),
+    (2, (0.8, 1e-7, -0.6), 1e-2, 1),
+    (3, (-0.8, 0.6, 1e-7), 1e-2, 2),
+])
+def test_hexahedral_traces_and_values_keep_their_own_digits(p, beta, dt, axis):
+    uh, u, uh_ref, u_ref = two_sweeps((3, 4, 2), p, beta, dt, axis)
+    assert worst(uh, uh_ref) < TOL
+    assert worst(u, u_ref) < TOL
+
+
 @pytest.mark.parametrize("p", [1, 3, 5])
 @pytest.mark.parametrize("k", [0, 23])
 def test_shallow_water_fields_of_different_size(p, k):
