@@ -269,6 +269,10 @@ ehdg_status ehdg_autotune_inner_sweeps(ehdg_ctx ctx, const int* candidates, int 
  * tensor-core path. The paper has no counterpart. */
 ehdg_status ehdg_autotune_fp64_path(ehdg_ctx ctx, int* tensor_cores, double* ms_dfma,
                                     double* ms_tensor);
+/* Chooses the FP64 path of such a context: nonzero, the tensor-core kernels;
+ * zero, those of EHDG_FP64. The state is left as it is. EHDG_ERR_INVALID for a
+ * context without the tensor-core path. The paper has no counterpart. */
+ehdg_status ehdg_set_fp64_path(ehdg_ctx ctx, int tensor_cores);
 /* Autotuner for the tile shape of the fused FP64 transport sweep (shared
  * operator, or a per-element operator without a tiled kernel; also the outer
  * sweeps of mixed precision): each 32-element tile is worked by 32 x FT

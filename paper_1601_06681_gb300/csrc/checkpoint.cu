@@ -174,6 +174,14 @@ extern "C" ehdg_status ehdg_load(ehdg_ctx h, const char* path) {
 
 namespace {
 
+// The captured step, which holds the launches of one variant
+void drop_graph(Ctx& c) {
+  if (c.gexec) cudaGraphExecDestroy(c.gexec);
+  if (c.graph) cudaGraphDestroy(c.graph);
+  c.gexec = nullptr;
+  c.graph = nullptr;
+}
+
 // Time one implicit step from the current state under each of n variants
 // (apply(k) configures variant k), restoring the state after every step;
 // ms[k] is the second of two steps (the first also captures the step graph),
@@ -202,14 +210,7 @@ ehdg_status time_step_variants(ehdg_ctx h, int n, Apply apply, double* ms) {
   for (int k = 0; k < n; ++k) {
     ms[k] = 1e300;
     if (st != EHDG_OK || !apply(k)) continue;
-    if (c.gexec) {
-      cudaGraphExecDestroy(c.gexec);
-      c.gexec = nullptr;
-    }
-    if (c.graph) {
-      cudaGraphDestroy(c.graph);
-      c.graph = nullptr;
-    }
+    drop_graph(c);
     int iters = 0;
     for (int rep = 0; rep < 2 && st == EHDG_OK; ++rep) {
       cudaEventRecord(e0, c.stream);
@@ -228,14 +229,7 @@ ehdg_status time_step_variants(ehdg_ctx h, int n, Apply apply, double* ms) {
   free_snap();
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  if (c.gexec) {
-    cudaGraphExecDestroy(c.gexec);
-    c.gexec = nullptr;
-  }
-  if (c.graph) {
-    cudaGraphDestroy(c.graph);
-    c.graph = nullptr;
-  }
+  drop_graph(c);
   return st;
 }
 
@@ -291,6 +285,20 @@ extern "C" ehdg_status ehdg_autotune_fp64_path(ehdg_ctx h, int* tensor_cores, do
   if (ms_dfma) *ms_dfma = ms[0];
   if (ms_tensor) *ms_tensor = ms[1];
   return st;
+}
+
+extern "C" ehdg_status ehdg_set_fp64_path(ehdg_ctx h, int tensor_cores) {
+  if (!h) return io_fail(EHDG_ERR_INVALID, "NULL context");
+  Ctx& c = h->c;
+  if (!c.oz_sweep.img)
+    return io_fail(EHDG_ERR_INVALID,
+                   "the context has no tensor-core FP64 path (FP64_EMULATED or emulated_outer)");
+  if (c.use_ozaki == (tensor_cores != 0)) return EHDG_OK;
+  cudaStreamSynchronize(c.stream);   // no launch of the step graph is in flight
+  drop_graph(c);
+  c.use_ozaki = tensor_cores != 0;
+  ++c.path_gen;                      // a batch recaptures its graph
+  return EHDG_OK;
 }
 
 extern "C" ehdg_status ehdg_autotune_sweep_tile(ehdg_ctx h, const int* cands, int n, int* best,

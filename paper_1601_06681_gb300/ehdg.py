@@ -89,6 +89,7 @@ _SIGS = [
     ("ehdg_load", C.c_int, [C.c_void_p, C.c_char_p]),
     ("ehdg_autotune_fp64_path", C.c_int, [C.c_void_p, C.POINTER(C.c_int),
                                           C.POINTER(C.c_double), C.POINTER(C.c_double)]),
+    ("ehdg_set_fp64_path", C.c_int, [C.c_void_p, C.c_int]),
     ("ehdg_autotune_inner_sweeps", C.c_int, [C.c_void_p, C.POINTER(C.c_int), C.c_int,
                                              C.POINTER(C.c_int), C.POINTER(C.c_double)]),
     ("ehdg_autotune_sweep_tile", C.c_int, [C.c_void_p, C.POINTER(C.c_int), C.c_int,
@@ -389,6 +390,10 @@ class Solver:
         tc, md, mt = C.c_int(), C.c_double(), C.c_double()
         _check(load().ehdg_autotune_fp64_path(self._h, C.byref(tc), C.byref(md), C.byref(mt)))
         return bool(tc.value), md.value, mt.value
+
+    def set_fp64_path(self, tensor_cores):
+        """ehdg_set_fp64_path: the tensor-core kernels, or those of "fp64"."""
+        _check(load().ehdg_set_fp64_path(self._h, int(bool(tensor_cores))))
 
     def autotune_sweep_tile(self, candidates=(2, 4, 8)):
         """Row groups per 32-element tile of the fused FP64 sweep, timed one
