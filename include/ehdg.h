@@ -281,9 +281,14 @@ ehdg_status ehdg_set_fp64_path(ehdg_ctx ctx, int tensor_cores);
  * (restoring the state after each), keeps the fastest, and reports it with
  * its time; the state is left as it was. Every row is one thread's FMA chain
  * for any FT, so the iterates do not change, only the summation order of the
- * residual. A batch recaptures its graph after the choice changed.
+ * residual. A batch recaptures its graph after the choice changed. A context
+ * whose FP64 sweep runs in Schur coefficients (FP64 on hexahedra with one
+ * shared operator and no beta.n = 0 point) has no such tile: one step is
+ * timed, and the choice stays as it is, or becomes the first valid candidate
+ * where it is not among them; it has no effect there.
  * EHDG_ERR_INVALID for a context whose FP64 sweep is another kernel (shallow
- * water, the tiled per-element sweep, the tensor-core FP64 path). */
+ * water, the tiled per-element sweep, the sweep of quadrilaterals with one
+ * shared operator, the tensor-core FP64 path). */
 ehdg_status ehdg_autotune_sweep_tile(ehdg_ctx ctx, const int* candidates, int n_candidates,
                                      int* best_ft, double* best_ms);
 /* Residual history r_0, r_1, ... of the last step (host buffer of cap entries). */

@@ -311,10 +311,23 @@ extern "C" ehdg_status ehdg_autotune_sweep_tile(ehdg_ctx h, const int* cands, in
                    "sweep)");
   const int saved = c.sweep_ft;
   std::vector<double> ms((size_t)n);
+  auto valid = [](int ft) { return ft == 2 || ft == 4 || ft == 8; };
+  if (md_active(c)) {
+    // the sweep in Schur coefficients has no tile of this kind, every candidate is
+    // the same step: one is timed, and the choice stays where it is a candidate
+    int keep = -1;
+    for (int k = 0; k < n; ++k)
+      if (valid(cands[k]) && (keep < 0 || cands[k] == saved)) keep = k;
+    const ehdg_status st = time_step_variants(h, n, [&](int k) { return k == keep; }, ms.data());
+    if (st == EHDG_OK && keep >= 0) c.sweep_ft = cands[keep];
+    if (best) *best = c.sweep_ft;
+    if (best_ms) *best_ms = keep >= 0 ? ms[keep] : 1e300;
+    return st;
+  }
   const ehdg_status st = time_step_variants(
       h, n,
       [&](int k) {
-        if (cands[k] != 2 && cands[k] != 4 && cands[k] != 8) return false;
+        if (!valid(cands[k])) return false;
         c.sweep_ft = cands[k];
         return true;
       },
