@@ -139,11 +139,11 @@ FX_INLINE long long fx_shift(long long v, int s) {
 
 // A shared operator's rows as limbs in blocks of four rows, [rows / 4][cols][4]
 // (the last block zero-padded), with scales of either sign: 2^col[a] for the
-// columns of group a (an axis's faces, a field), and for each row one for each of
-// its ng groups of cols / ng columns whose values have units of their own (the
-// fields of the state), scale[row * ng + f]. entry = 2^(col + scale - 56) (h 2^28 +
-// l); with col divided out the limbs' value is below 2 and its sum over the group
-// below 32, so that a group's products with 56-bit values sum below 2^62.
+// columns of group a (an axis's faces), and for each row one for each of its ng
+// parts, the columns whose values have units of their own (the fields of the state),
+// scale[row * ng + f]. entry = 2^(col + scale - 56) (h 2^28 + l); with col divided
+// out the limbs' value is below 2 and its sum over the part below 32, so that a
+// part's products with 56-bit values sum below 2^62.
 struct FxOp {
   const int2* x;
   const int* scale;

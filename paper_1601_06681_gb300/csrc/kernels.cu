@@ -433,22 +433,21 @@ cudaError_t launch_face_signs(Ctx& c) {
 //   w = u^n / dt_eff + f (time-dependent) or w = f (steady)
 // ===========================================================================
 // A shared operator's matrix M [rows][cols] times coef as limbs (FxOp), one block.
-// Columns: nc groups with a scale each, the group of column c of row r being
-// idx[r * cols + c] / (n / nc) (idx null: c / (n / nc)), the scale its largest
-// entry's exponent. Rows: ng groups of columns; the scales are the least with the
-// group's largest entry below 2 and its sum of magnitudes below 32. blocked: the
-// layout of FxOp, else row-major.
-__global__ void k_fx_limbs(int rows, int cols, int ng, int nc, int n, const int* idx, double coef,
-                           const double* M, int blocked, int2* x, int* scale, int* col) {
+// nc groups of cols / nc columns with a scale each, the exponent of the group's
+// largest entry; each row has a scale for each of its ng parts, the least with the
+// part's largest entry below 2 and its sum of magnitudes below 32. The parts are
+// cols / ng columns each, or (turns) every ng-th column. blocked: the layout of
+// FxOp, else row-major.
+__global__ void k_fx_limbs(int rows, int cols, int ng, bool turns, int nc, double coef,
+                           const double* M, bool blocked, int2* x, int* scale, int* col) {
   __shared__ int s_col[3];
   __shared__ double s_f[3];                     // coef over the group's scale
-  const int np = cols / ng, nf = n / nc, rows4 = blocked ? (rows + 3) / 4 * 4 : rows;
-  auto group = [&](int i) { return nc == 1 ? 0 : (idx ? idx[i] : i % cols) / nf; };
+  const int np = cols / ng, nq = cols / nc, rows4 = blocked ? (rows + 3) / 4 * 4 : rows;
   if (threadIdx.x < 3) s_col[threadIdx.x] = nc > 1 ? kZeroGroup : 0;
   __syncthreads();
   for (int i = threadIdx.x; i < (nc > 1 ? rows * cols : 0); i += blockDim.x)
     if (M[i] != 0.0)
-      atomicMax(&s_col[group(i)], min(1000, max(-1000, ilogb(coef * M[i]))));
+      atomicMax(&s_col[i % cols / nq], min(1000, max(-1000, ilogb(coef * M[i]))));
   __syncthreads();
   if (threadIdx.x < 3) {
     const int e = s_col[threadIdx.x];
@@ -459,48 +458,49 @@ __global__ void k_fx_limbs(int rows, int cols, int ng, int nc, int n, const int*
   for (int i = threadIdx.x; i < rows4 * ng; i += blockDim.x) {
     const int r = i / ng, f = i - r * ng;
     double mx = 0.0, sum = 0.0;
-    if (r < rows)
-      for (int c = f * np; c < (f + 1) * np; ++c) {
-        const double v = fabs(s_f[group(r * cols + c)] * M[r * cols + c]);
-        mx = fmax(mx, v);
-        sum += v;
-      }
+    for (int k = 0; k < (r < rows ? np : 0); ++k) {
+      const int c = turns ? k * ng + f : f * np + k;
+      const double v = fabs(s_f[c / nq] * M[r * cols + c]);
+      mx = fmax(mx, v);
+      sum += v;
+    }
     scale[i] = mx > 0.0 ? max(ilogb(mx), ilogb(sum) + 1 - 5) : 0;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < rows4 * cols; i += blockDim.x) {
     const int r = i / cols, c = i - r * cols;
-    const double v = r < rows ? s_f[group(i)] * M[i] : 0.0;
-    const Limb l = fx_split(__double2ll_rn(scalbn(v, 56 - scale[r * ng + c / np])));
+    const double v = r < rows ? s_f[c / nq] * M[i] : 0.0;
+    const int e = 56 - scale[r * ng + (turns ? c % ng : c / np)];
+    const Limb l = fx_split(__double2ll_rn(scalbn(v, e)));
     x[blocked ? ((r / 4) * (int64_t)cols + c) * 4 + r % 4 : i] = make_int2(l.h, l.l);
   }
 }
 
-// Groups of P: the fields of the state, whose products are summed apart. Of Ey's
-// columns: the fields (a row is (phi + sqrt(Phi) vel.n) / 2, with phi about
-// sqrt(Phi) times vel). Of H's and Hy's columns: the axes, whose faces' traces enter
+// The parts of P's rows are the fields of the state, those of Ey's phi and vel.n,
+// whose entries take turns: a field has a unit of its own and its products are summed
+// apart. The groups of H's and Hy's columns are the axes, whose faces' traces enter
 // with |beta_a| / h_a.
 cudaError_t build_fx_operators(Ctx& c) {
   cudaError_t e = dalloc_raw(c, (void**)&c.fx_col_d, sizeof(c.fx_col));
   if (e == cudaSuccess) e = cudaMemsetAsync(c.fx_col_d, 0, sizeof(c.fx_col), c.stream);
   int at = 0;
-  auto make = [&](int rows, int cols, int ng, int nc, int n, const int* idx, double coef,
-                  const double* M, bool blocked, void** x, int** scale) {
+  auto make = [&](int rows, int cols, int ng, bool turns, int nc, double coef, const double* M,
+                  bool blocked, void** x, int** scale) {
     const int r4 = blocked ? (rows + 3) / 4 * 4 : rows;
     if (e == cudaSuccess) e = dalloc_raw(c, x, sizeof(int2) * r4 * cols);
     if (e == cudaSuccess) e = dalloc_raw(c, (void**)scale, sizeof(int) * r4 * ng);
     if (e != cudaSuccess) return;
-    k_fx_limbs<<<1, 512, 0, c.stream>>>(rows, cols, ng, nc, n, idx, coef, M, blocked ? 1 : 0,
+    k_fx_limbs<<<1, 512, 0, c.stream>>>(rows, cols, ng, turns, nc, coef, M, blocked,
                                         static_cast<int2*>(*x), *scale, c.fx_col_d + 3 * at++);
     e = cudaGetLastError();
   };
   const double uc = c.scheme == EHDG_STEADY ? 1.0 : 1.0 / c.dt_eff;
   const int nq = c.NQFS;
-  make(c.n, c.n, c.nf, 1, c.n, nullptr, uc, c.P, true, &c.fx_P, &c.fx_Ps);
-  make(c.n, nq, 1, c.dim, nq, nullptr, 1.0, c.H, true, &c.fx_H, &c.fx_Hs);
-  make(nq, c.KE, 1, c.nf, c.n, c.ey_idx, 1.0, c.ey_val, false, &c.fx_E, &c.fx_Es);
+  make(c.n, c.n, c.nf, false, 1, uc, c.P, true, &c.fx_P, &c.fx_Ps);
+  make(c.n, nq, 1, false, c.dim, 1.0, c.H, true, &c.fx_H, &c.fx_Hs);
+  make(nq, c.KE, c.nf == 3 ? 2 : 1, true, 1, 1.0, c.ey_val, false, &c.fx_E, &c.fx_Es);
   if (c.pde == EHDG_SW_LINEAR)
-    make(nq, nq, 1, c.dim, nq, nullptr, 1.0, c.Hy, false, &c.fx_Hy, &c.fx_Hys);
+    make(nq, nq, 1, false, c.dim, 1.0, c.Hy, false, &c.fx_Hy, &c.fx_Hys);
   return e;
 }
 

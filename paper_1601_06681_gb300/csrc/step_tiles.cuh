@@ -73,25 +73,33 @@ __device__ __forceinline__ int tile_max(int v) {
   return m;
 }
 
-// n values v[c * 32] of a lane (COL: in up to three groups of np, times 2^col of
-// their group) to packed limbs in place, in units of 2^(emax - 1078); returns emax
-// (kNotFinite: a value is not finite)
-template <bool COL>
+// n values v[c * 32] of a lane (a field) to packed limbs in place, in units of
+// 2^(emax - 1078); returns emax (kNotFinite: a value is not finite)
+__device__ __forceinline__ int tile_limbs(double* v, int n) {
+  const int lane = threadIdx.x, t = threadIdx.y;
+  int em = 1;
+  for (int c = t; c < n; c += kStepT) em = max(em, fx_exponent(v[c * 32 + lane]));
+  em = tile_max(em);
+  long long* x = reinterpret_cast<long long*>(v);
+  for (int c = t; c < n; c += kStepT)
+    x[c * 32 + lane] = fx_pack(fx_split(fx_from_double(v[c * 32 + lane], em)));
+  __syncthreads();
+  return em == 0x7ff ? kNotFinite : em;
+}
+
+// the same for up to three groups of np values, each group times its 2^col
 __device__ __forceinline__ int tile_limbs(double* v, int n, int np, const int (&col)[3]) {
   const int lane = threadIdx.x, t = threadIdx.y;
-  auto scale = [&](int c) {
-    return !COL ? 0 : (c < np ? col[0] : (c < 2 * np ? col[1] : col[2]));
-  };
+  auto scale = [&](int c) { return c < np ? col[0] : (c < 2 * np ? col[1] : col[2]); };
   int em = -kNotFinite;
   for (int c = t; c < n; c += kStepT) {
     const int e = fx_exponent(v[c * 32 + lane]);
     em = max(em, e == 0x7ff ? kNotFinite : max(e, 1) + scale(c));
   }
   em = tile_max(em);
-  for (int c = t; c < n; c += kStepT) {
-    double& x = v[c * 32 + lane];
-    x = __longlong_as_double(fx_pack(fx_split(fx_from_double(x, em - scale(c)))));
-  }
+  long long* x = reinterpret_cast<long long*>(v);
+  for (int c = t; c < n; c += kStepT)
+    x[c * 32 + lane] = fx_pack(fx_split(fx_from_double(v[c * 32 + lane], em - scale(c))));
   __syncthreads();
   return em;
 }
@@ -165,7 +173,7 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
       int em[3] = {1, 1, 1};
 #pragma unroll
       for (int f = 0; f < 3; ++f)
-        if (f < s.nf) em[f] = tile_limbs<false>(w + f * np * 32, np, np, s.Px.col);
+        if (f < s.nf) em[f] = tile_limbs(w + f * np * 32, np);
       for (int b = t; b * 4 < n; b += kStepT) {
         double v[4];
         tile_rows4(s.Px, Psh, w, b, n, s.nf, em, v);
@@ -246,7 +254,10 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
     return;
   }
   const bool limbs = SHARED && !s.g_ready;
-  const int ge = limbs ? tile_limbs<true>(g, n, n / s.nf, s.Eyx.col) : 0;
+  int ge[3] = {1, 1, 1};
+#pragma unroll
+  for (int f = 0; f < 3; ++f)
+    if (limbs && f < s.nf) ge[f] = tile_limbs(g + f * (n / s.nf) * 32, n / s.nf);
   if (!live) return;
   // the rows the sweep computes (upwind and tangential points; every point
   // for shallow water): Gy in the sweep's slot order, and the element
@@ -258,13 +269,24 @@ __device__ __forceinline__ void step_tile(const StepParams& s, const int2* Psh, 
     double y0 = 0.0, gy = 0.0;
     if (limbs) {
       const long long* gx = reinterpret_cast<const long long*>(g) + lane;
-      Acc a(0);
-      for (int k2 = 0; k2 < s.KE; ++k2) {
-        const int2 c = s.Eyx.x[r * s.KE + k2];
-        a.mac(Cfx{c.x, c.y}, fx_limb(gx[s.ey_idx[r * s.KE + k2] * 32]));
+      Acc a(0), b(0);
+      const int2* E = s.Eyx.x + r * s.KE;
+      const int* idx = s.ey_idx + r * s.KE;
+      if (s.nf == 1) {
+        for (int k2 = 0; k2 < s.KE; ++k2)
+          a.mac(Cfx{E[k2].x, E[k2].y}, fx_limb(gx[idx[k2] * 32]));
+        gy = fx_value(a.get(), ge[0] - 1078 + s.Eyx.scale[r]);
+      } else {   // entries of phi and of vel.n in turn; the sum in the coarser of their units
+        for (int k2 = 0; k2 < s.KE; k2 += 2) {
+          a.mac(Cfx{E[k2].x, E[k2].y}, fx_limb(gx[idx[k2] * 32]));
+          b.mac(Cfx{E[k2 + 1].x, E[k2 + 1].y}, fx_limb(gx[idx[k2 + 1] * 32]));
+        }
+        const int La = ge[0] + s.Eyx.scale[2 * r];
+        const int Lb = (r < s.NQFS / 2 ? ge[1] : ge[2]) + s.Eyx.scale[2 * r + 1], L = max(La, Lb);
+        gy = fx_value(fx_shift(a.get(), L - La) + fx_shift(b.get(), L - Lb), L - 1078);
       }
-      s.Gy[j * ne + e] = ge == kNotFinite ? __hiloint2double(0x7ff80000, 0)
-                                     : fx_value(a.get(), ge - 1078 + s.Eyx.scale[r]);
+      const bool nan = max(max(ge[0], ge[1]), ge[2]) == kNotFinite;
+      s.Gy[j * ne + e] = nan ? __hiloint2double(0x7ff80000, 0) : gy;
       if (want_y0) {
         for (int k2 = 0; k2 < s.KE; ++k2)
           y0 = fma(s.ey_val[r * s.KE + k2], s.u[s.ey_idx[r * s.KE + k2] * ne + e], y0);
@@ -316,7 +338,7 @@ __device__ __forceinline__ void final_tile(const FinalParams& p, const int2* Hsh
   }
   __syncthreads();
   if (p.shared) {
-    const int em[3] = {tile_limbs<true>(uh, p.NQFS, 2 * p.Nqf, p.Hx.col), 1, 1};
+    const int em[3] = {tile_limbs(uh, p.NQFS, 2 * p.Nqf, p.Hx.col), 1, 1};
     for (int b = t; b * 4 < p.n; b += kStepT) {
       double g[4];
 #pragma unroll

@@ -72,6 +72,24 @@ def test_quadrilateral_traces_keep_their_own_digits(p, beta, dt, axis):
     assert worst(uh, uh_ref) < TOL
 
 
+@pytest.mark.parametrize("p", [1, 2, 4])
+def test_shallow_water_faces_do_not_take_the_other_velocity_s_unit(p):
+    """Each element's fields are of sizes 1e-12 to 1 of their own; a face's trace holds phi
+    and the normal velocity, and the other velocity, however large, only by dt squared."""
+    from oracle.ehdg import Problem
+    mesh = W.structured_mesh((6, 5), boundary_tag=W.TAG_WALL)
+    prob = Problem(mesh, p, pde="sw", scheme="be", dt=1e-8, Phi=1.0)
+    rng = np.random.default_rng(1)
+    u0 = rng.standard_normal((prob.nel, 3, prob.Np)) * 10.0 ** rng.integers(-12, 1, (prob.nel, 3, 1))
+    u_ref, uh_ref, _ = prob.solve_step(u0, prob.trace(u0), fixed_iters=2)
+    with E.Solver(mesh, p, pde="sw", scheme="be", dt=1e-8, Phi=1.0) as s:
+        s.set_state(u0)
+        s.step_fixed(2)
+        u, uh = s.get_state()
+    assert worst(uh, uh_ref) < TOL
+    assert worst(u, u_ref) < TOL
+
+
 @pytest.mark.parametrize("p,beta,dt,axis", [
     (1, (0.8, 0.35), 1e-8, None),
     (6, (-0.8, -0.35), 1e-8, None),
