@@ -76,6 +76,20 @@ typedef enum { EHDG_BE = 0, EHDG_CN = 1, EHDG_STEADY = 2 } ehdg_scheme;
  * equation delta = R + S H delta and the FP64 update uhat += delta; the fixed
  * point and the stopping rule are those of the FP64 iteration. MIXED_FP32 uses
  * float32 operands and accumulation on the CUDA cores.
+ * FP64: states, traces and residuals are doubles. The sums of products of an
+ * operator shared by all elements (transport on quadrilaterals and on hexahedra
+ * without a beta.n = 0 point, shallow water without a beta-plane) and of the
+ * per-element transport sweep on its tiles run in fixed point on the integer pipe:
+ * an element's values (of shallow water: a field's) are held in 54 to 56 bits of the
+ * largest of them, a row's coefficients in 56 bits of its largest, and a sum is
+ * rounded once. It is as accurate as the same sum in double or more where the
+ * largest values meet the row's larger coefficients, and off by at most
+ * (2 n + 1) 2^-54 times the largest value times the row's largest coefficient for n
+ * products (on hexahedra, where the unknowns of a triangular solve are held so,
+ * likewise up to the size of the solve). Values below 2^-3 of their element's
+ * largest keep fewer than a double's bits. The operator's rows and the columns of
+ * each axis have scales of their own, which keep a small time step, a velocity
+ * nearly along a face and the size of Phi out of this.
  * FP64_EMULATED: every sweep FP64-accurate without the FP64 pipe's products:
  * in fixed point on the integer pipe where that form exists (as EHDG_FP64
  * there: transport on quadrilaterals and hexahedra without a beta.n = 0 point,
@@ -162,10 +176,13 @@ typedef struct {
   int64_t device_bytes;        /* device memory held by the context */
   int64_t sweep_rows;          /* face-point rows the element sweep computes, summed over
                                   elements (upwind/tangential points only for transport) */
-  int sum_factorised;          /* 1 if the FP64 sweep and reconstruction apply the face term
-                                  by 1D passes per face (hexahedra, one shared transport
-                                  operator): per element 2 NQFS q + NQFS + rows NB FMAs per
-                                  sweep, NB = (p+1)^3 - (p-1)^3 boundary nodes */
+  int sum_factorised;          /* 1 on hexahedra with one shared transport operator: the outer
+                                  FP64 sweeps of MIXED_* precision, and all FP64 sweeps where
+                                  a component of the velocity is zero, apply the face term by
+                                  1D passes per face (per element 2 NQFS q + NQFS + rows NB
+                                  FMAs, NB = (p+1)^3 - (p-1)^3 boundary nodes). The other FP64
+                                  contexts solve in Schur coefficients in fixed point, 936
+                                  products per element and sweep at p = 3 */
   int warm_start;              /* 1 if, after a step with at least one sweep, the next step
                                   starts from that step's final trace instead of forming the
                                   trace formula of u^n (Algorithm 1's initial trace): the last

@@ -34,9 +34,10 @@ struct ehdg_batch_s {
   // looped instances allow it (FP64 or FP32 corrections)
   bool use_persist = false;
   // no form chosen by the caller or a tuner: the persistent one where every
-  // looped instance is FP64 (48 instances, 124,000 elements, 4 steps: 11.3 ms
-  // against 15.7 for the loop of launches, whose every iteration waits for its
-  // slowest instance; with FP32 corrections the two are equal within 1%)
+  // looped instance is FP64 (a mix of 48 instances, 4 steps: 14.5 ms against 20.0
+  // for the loop of launches, whose every iteration waits for its slowest instance).
+  // With FP32 corrections the loop is the faster one, 10.2 against 11.5 ms: its short
+  // items do not pay for a claim and a count each.
   bool auto_form = true;
   int last_run_steps = 0;               // steps of the last run: what the autotuners time
   // kernel accounting of the batched loop (ehdg_batch_set_profiling)
@@ -1080,9 +1081,9 @@ ehdg_status ehdg_create(const ehdg_mesh_desc* mesh, const ehdg_problem_desc* pro
   }
   // The tensor-core products stay where no fixed-point form exists (mixed
   // precision on hexahedra, beta.n = 0 points). Elsewhere fixed point is at least
-  // as accurate (2^-56 of the largest value against 2^-49) and faster: 37 x 29 x
-  // 31 hexahedra, p = 3: 51 against 65 us per iteration, 64^3: 243 against 297 a
-  // sweep; shallow water, 512 x 512, p = 3: 46 against 66 us of element values.
+  // as accurate (56 bits of the largest value against 49) and faster: 37 x 29 x
+  // 31 hexahedra, p = 3: 51 against 65 us per iteration, 64^3: 250 against 297 a
+  // sweep; shallow water, 512 x 512, p = 3: 42 against 66 us of element values.
   // ehdg_autotune_fp64_path still compares the two.
   if (c.use_pe || c.md || c.pde == EHDG_SW_LINEAR) c.use_ozaki = false;
   // their persistent forms launch resident blocks only

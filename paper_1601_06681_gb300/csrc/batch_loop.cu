@@ -219,8 +219,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // One FP64 sweep of every instance that still iterates: items = (instance,
 // 128-element tile) from the lists; the instance's own single-problem tile
 // body, reduction and stopping test.
-// (five blocks per SM, 102 registers: 15.7 ms for the 48-instance mix, two at
-// the 250 registers of the unconstrained p = 6 body 18.0)
+// Five blocks per SM, although the 96 registers spill 1.8 KB of the p = 6 body: an
+// iteration's many small tiles are bound by latency. A mix of 48 FP64 instances,
+// four steps: 20.0 ms; 20.8, 22.1 and 22.8 at four, three and two blocks.
 __global__ void __launch_bounds__(kPeTile, 5) k_batch_sweep(const BInst* inst, const int4* counts,
                                                           int* lists, int n_inst,
                                                           unsigned int* ticket, int graph_mode,

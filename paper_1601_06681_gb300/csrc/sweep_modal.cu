@@ -94,17 +94,12 @@ template <int P1>
 struct MdParams {
   int64_t nel, nface;
   const int32_t* elem_face;      // [6][nel]
-  int fin[3], fout[3];           // local inflow and outflow face of each axis
-  double cl[3][P1], cr[3][P1];   // c_a l_i, c_a r_i
+  int fout[3];                   // local outflow face of each axis
   double r[P1];
   double T[3][P1][P1];           // c_a T (entries right of the diagonal blocks)
   double inv[MdBlocks<P1>::NINV];
   FxTraces tr;
-  IterState* it;
 };
-
-// The same tables in fixed point for the sweep, the equation divided by sigma
-// (Cfx, fixed_point.cuh).
 
 // The fixed-point sweep splits an element over warps: along the second and
 // third axes the coefficients go in pairs (groups; at P1 = 3 the first group
@@ -121,6 +116,8 @@ struct FxShape {
   __host__ __device__ static constexpr int group(int t) { return (t + OFF) >> 1; }
 };
 
+// The tables in fixed point for the sweep and the reconstruction, the equation
+// divided by sigma (Cfx, fixed_point.cuh).
 template <int P1>
 struct FxParams {
   int64_t nel;
@@ -175,7 +172,6 @@ __device__ __forceinline__ const T& fx_at(const T* base, unsigned off) {
   return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
 }
 
-// named barriers 1 and 2 of a 128-thread block
 // the same for data that a persistent launch rewrites: through L2 only
 template <bool CG, class T>
 __device__ __forceinline__ T fx_ld(const T* base, unsigned off) {
@@ -183,6 +179,7 @@ __device__ __forceinline__ T fx_ld(const T* base, unsigned off) {
   else return fx_at(base, off);
 }
 
+// named barriers 1 and 2 of a 128-thread block
 template <int ID>
 __device__ __forceinline__ void bar_sync() {
   asm volatile("bar.sync %0, 128;" ::"n"(ID) : "memory");
@@ -422,6 +419,8 @@ __device__ __forceinline__ void fx_solve(const FxParams<P1>& p, const FxElem& el
       xi[u] = fx_split(ok ? ai(fx_ld<CG>(src + g * nface, fi[0])) : 0);
       xo[u] = fx_split(ok ? ao(fx_ld<CG>(src + g * nface, fo[0])) : 0);
     }
+    // unrolled for the team at P1 = 3 (17 x 12 x 9, four Crank-Nicolson steps: 1.73 ->
+    // 1.57 ms), rolled at P1 = 4 (p = 3 on the same mesh: 1.85, unrolled 1.89)
 #pragma unroll (SOLO || P1 == 4 ? 1 : P1)
     for (int i = 0; i < P1; ++i) {
       const int by = S::group(i) + 2 * K, bz = S::group(i) + 2 * J;
@@ -538,13 +537,13 @@ __device__ __forceinline__ void fx_solve(const FxParams<P1>& p, const FxElem& el
 // in turn; otherwise a team of NW warps, one role each.
 //
 // Why roles and rolled loops: one thread per element, straight-line, is 936
-// products instead of 1,140 but 17,200 instructions, more than the instruction
-// caches hold; it took 768 us per sweep at 64^3, p = 3, its warps waiting for
-// instructions. This form runs 15,500 instructions per tile from about 1,000
-// distinct ones: 243 us (1,721 with the sum-factorised FP64 sweep, 567 with
-// this algorithm on the FP64 pipe). 224 MB are read and 79 MB written to DRAM,
-// 1.2 TB/s: the ALU (a mad.wide is a multiply and a 64-bit add) and the latency
-// of the sums at 12 warps per SM bound it.
+// products instead of 1,140 but more code than the instruction caches hold; it took
+// 768 us per sweep at 64^3, p = 3, its warps waiting for instructions. This form
+// takes 250 us (1,721 with the sum-factorised FP64 sweep, 567 with this algorithm on
+// the FP64 pipe), 15,300 warp instructions per tile. Neither a pipe nor memory
+// binds it: the multiply pipe is 50% busy, the ALU 45%, issue slots 46%, DRAM 15%;
+// the latency of the sums and of the trace loads is left, at 11 warps per SM (166
+// registers and 16.6 KB of shared memory a warp).
 template <int P1, bool SOLO, bool PERSIST>
 __global__ void __launch_bounds__(32 * (SOLO ? 1 : FxShape<P1>::NW), SOLO ? 12 : 4)
     k_sweep_fx(const __grid_constant__ FxParams<P1> p, const __grid_constant__ MdResid q) {
@@ -1275,17 +1274,14 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
   for (int a = 0; a < 3; ++a) {
     const bool rev = c.beta_const[a] < 0.0;
     ca[a] = 2.0L * std::fabs((ld)c.beta_const[a]) / (ld)c.elem_h[a];
-    p->fin[a] = 2 * a + (rev ? 1 : 0);
     p->fout[a] = 2 * a + (rev ? 0 : 1);
     ld jf = 1.0L;
     for (int d = 0; d < 3; ++d)
       if (d != a) jf *= 0.5L * (ld)c.elem_h[d];
-    x->fin[a] = p->fin[a];
+    x->fin[a] = 2 * a + (rev ? 1 : 0);
     x->fout[a] = p->fout[a];
     x->fw[a] = (double)jf;
     for (int i = 0; i < P1; ++i) {
-      p->cl[a][i] = (double)(ca[a] * t.l[i]);
-      p->cr[a][i] = (double)(ca[a] * t.r[i]);
       p->r[i] = (double)t.r[i];
       for (int j = 0; j < P1; ++j) {
         p->T[a][i][j] = (double)(ca[a] * t.T[i * P1 + j]);
@@ -1353,7 +1349,7 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
   for (int I = 0; I < B::NB; ++I)
     for (int J = 0; J < B::NB; ++J)
       for (int K = 0; K < B::NB; ++K) {
-        // the blocks of the FP64 kernels (the step and the reconstruction)
+        // the blocks of the FP64 kernel (the step)
         const int s3[3] = {B::size(I), B::size(J), B::size(K)}, o3[3] = {I, J, K};
         std::vector<ld> X;
         if (!md_block_inverse(P1, t, ca, tau, s3, o3, &X)) return false;
@@ -1399,7 +1395,7 @@ bool md_fill(const Ctx& c, const Md1D& t, MdKernelArgs<P1>* args) {
   p->nface = c.nface;
   p->elem_face = x->elem_face = c.geo.elem_face;
   p->tr = x->tr = f->tr = md_traces(c);
-  p->it = x->it = c.it;
+  x->it = c.it;
   s->ucoef = c.scheme == EHDG_STEADY ? 0.0 : 1.0 / c.dt_eff;
   s->have_force = 0;
   s->force_avg = s->cn = f->cn = c.scheme == EHDG_CN ? 1 : 0;
@@ -1451,9 +1447,9 @@ cudaError_t step_t(Ctx& c) {
 }
 
 // One warp does all groups of its elements where there are tiles enough to
-// keep 12 warps per SM on full runs: 243 against 265 us at 8,192 tiles (64^3,
-// p = 3). With fewer the team's shorter tile wins: 93 against 109 us per
-// iteration at 2,000 tiles, 31 against 45 at 16.
+// keep 12 warps per SM on full runs: two steps of 70 iterations at 64^3, p = 3 (8,192
+// tiles) 22.1 ms, by teams 23.7. With fewer the team's shorter tile wins: 64
+// iterations at 2,000 tiles 6.4 against 7.9 ms, 36 at 16 tiles 1.08 against 1.66.
 bool fx_solo(int64_t nel) { return (nel + 31) / 32 >= 32 * device_sms(); }
 
 template <int P1, bool SOLO>

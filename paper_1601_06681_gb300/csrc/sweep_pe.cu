@@ -16,9 +16,11 @@ namespace ehdg {
 
 namespace {
 
-// three blocks per SM from p = 4 on, four below: 253 x 187, p = 4 (370 tiles)
-// then runs in one wave (6.75 ms for ten Crank-Nicolson steps; 7.74 at two
-// blocks, 6.95 at four, which spill)
+// Blocks per SM: three from p = 4 on, four below. The spills that takes (32 to 304
+// bytes from p = 3 up) cost less than another wave of blocks. Six Crank-Nicolson steps, ms at 2 / 3 / 4 / 5 blocks:
+//   94 tiles:  p = 2 1.28 1.29 1.34 1.40  p = 4 1.88 2.02 2.24 2.30  p = 6 2.94 3.07 3.38 3.67
+//   370 tiles: p = 2 2.70 2.40 2.45 2.51  p = 4 4.18 3.59 3.79 3.85  p = 6 6.98 5.70 5.95 6.49
+//   938 tiles: p = 2 5.56 5.58 5.21 6.10  p = 4 8.70 9.27 8.65 10.7  p = 6 14.9 16.9 16.7 22.4
 template <int NQ>
 __global__ void __launch_bounds__(kPeTile, NQ >= 20 ? 3 : 4) k_sweep_pe(const __grid_constant__ PeView v,
                                                       const int2* Hx, int graph_mode,
@@ -104,8 +106,9 @@ __device__ __forceinline__ void pe_cluster_store(double* p, int rank, double x) 
 // CL: the grid is one cluster (up to kPeCluster tiles). Its hardware barrier
 // ends a pass, every block holds all partial sums in shared memory and decides
 // for itself: such a mesh is all latency, and the counter and the polled word
-// in L2 cost more than the pass. 16 x 16, p = 2, 10 steps: 2.62 -> 1.42 ms with
-// the cluster; 253 x 187, p = 4 with a block per tile 6.96 -> 6.38. The sums are those of pe_total, so iterates,
+// in L2 cost more than the pass. 16 x 16, p = 2, 10 steps: 2.62 -> 1.35 ms with
+// the cluster; 253 x 187, p = 4 with a block per tile 6.96 -> 5.70 (of both, 0.05 and
+// 0.6 since Gy is aligned apart). The sums are those of pe_total, so iterates,
 // residuals and decisions are bit for bit the same in every form.
 constexpr int kPeCluster = 16;
 

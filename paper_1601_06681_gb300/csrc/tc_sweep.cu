@@ -538,7 +538,7 @@ cudaError_t launch_lp_sweep_tc(Ctx& c, const float* in, float* out, bool fuse_ap
     int64_t grid = (int64_t)bpsm * device_sms();
     if (grid > ntiles) grid = ntiles;
     // a dependent launch on hexahedra, where two sweeps overlap by the staging
-    // (64^3, p = 3: four steps 17.1 -> 16.8 ms). Not on quadrilaterals: 301 x 170
+    // (64^3, p = 3: four steps 16.90 -> 16.68 ms). Not on quadrilaterals: 301 x 170
     // shallow water gained nothing, and a batch's branches lost 1%, since the
     // waiting blocks take room from other instances' kernels.
     if (c.dim == 3)
