@@ -675,7 +675,8 @@ def run_2d(args, ws, dev, stream, standalone=False):
 def fp64_sweep(info):
     """(kernel, FP64 flops one sweep executes, flops of the dense form
     2 rows NQFS) of a transport context's DFMA sweep. The sum-factorised
-    sweep (hexahedra, shared operator) executes per element two 1D passes per
+    sweep (the outer sweeps of mixed precision on hexahedra with a shared
+    operator; the FP64 ones are schur_roofline's) executes per element two 1D passes per
     face (2 NQFS q FMAs), the face scaling (NQFS) and the dense rows x NB
     product over the NB = (p+1)^3 - (p-1)^3 boundary nodes."""
     nel, nq, rows = info["n_elem"], 2 * info["dim"] * info["Nqf"], info["sweep_rows"]
@@ -710,6 +711,10 @@ def schur_roofline(info, sweeps, ms, sms, mhz):
 
 # the dominant kernel of each kind the profiling run times, per path
 def _kernel_name(kind, precision, emulated_outer, info=None):
+    if info and info.get("sum_factorised") and precision in ("fp64", "fp64_emulated"):
+        # FP64 on hexahedra: the step in Schur coefficients
+        return {"elem": "k_sweep_fx", "step": "k_step_md + k_bnd_md",
+                "final": "k_final_fx + k_trace_end_md", "aux": "transposes, resets"}.get(kind, kind)
     emulated = precision == "fp64_emulated" or emulated_outer
     fp64_name = fp64_sweep(info)[0] if info else "k_sweep_fused"
     return {"elem": "k_ozaki (sweep mode)" if emulated else fp64_name,
