@@ -1081,10 +1081,14 @@ ehdg_status ehdg_create(const ehdg_mesh_desc* mesh, const ehdg_problem_desc* pro
   }
   // The tensor-core products stay where no fixed-point form exists (mixed
   // precision on hexahedra, beta.n = 0 points). Elsewhere fixed point is at least
-  // as accurate (56 bits of the largest value against 49) and faster: 37 x 29 x
-  // 31 hexahedra, p = 3: 51 against 65 us per iteration, 64^3: 250 against 297 a
-  // sweep; shallow water, 512 x 512, p = 3: 42 against 66 us of element values.
-  // ehdg_autotune_fp64_path still compares the two.
+  // more accurate (56 bits of the largest value against 49: 40^3, p = 2, u 2.1e-15
+  // off a 64-bit solution against 1.1e-14) and mostly faster: 37 x 29 x 31 hexahedra,
+  // p = 3: 51 against 65 us per iteration, 64^3: 250 against 297 a sweep; 56^3, p = 1:
+  // 2.2 against 5.4 ms for two steps; shallow water, 512 x 512, p = 3: 42 against 66 us
+  // of element values. Large hexahedral meshes at p = 2 pay for the accuracy (two
+  // steps of 28 x 30 x 26: 2.51 against 2.42 ms, 40^3: 5.2 against 4.3, 56^3: 13.0
+  // against 10.5; 20^3 1.29 against 1.53): ehdg_set_fp64_path and
+  // ehdg_autotune_fp64_path choose the other path there.
   if (c.use_pe || c.md || c.pde == EHDG_SW_LINEAR) c.use_ozaki = false;
   // their persistent forms launch resident blocks only
   if (c.use_pe || c.md) c.persist_fits = true;
