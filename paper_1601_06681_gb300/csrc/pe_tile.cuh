@@ -5,19 +5,20 @@
 // of the two faces it is upwind of (NQ / 2 rows; no point has beta.n = 0),
 // writes the new trace there and adds w (uhat^{k+1} - uhat^k)^2 to the residual.
 //
-// The products run in fixed point on the integer pipe (fixed_point.cuh). The
-// operator is equilibrated: Hy[j][c] = 2^(s_j + t_a) Hx[j][c], t_a for the columns
+// The products run in fixed point on the integer pipe (fixed_point.cuh): the FP64
+// pipe, 1.6 operations per clock and SM, bounded the double form (NQ^2 / 2 products
+// per element, 200 at p = 4). What is left there is four operations per row: the
+// conversion of the result, the increment, its square, the sum. Every load of a tile
+// is issued before the first product, so that a small problem waits for memory twice
+// (face ids, then all values).
+//
+// The operator is equilibrated: Hy[j][c] = 2^(s_j + t_a) Hx[j][c], t_a for the columns
 // of axis a's faces, s_j for row j, both of either sign, since the columns go with
 // |beta_a| / h_a and all entries with dt where that is small. The element's traces
-// times 2^t_a are aligned to the largest of them with 56 bits, a row's sum and its
-// Gy to the larger of the two. (One scale for the whole operator, not below one,
+// times 2^t_a are aligned to the largest of them with 56 bits, a row's sum and its Gy
+// to the coarser of their units. (One scale for the whole operator, not below one,
 // lost 2.6e-13 of a trace at 16 x 16, p = 2, dt = 1e-6, in an element fed from rest;
-// the present form 5e-17, an FMA chain 8e-17.) The FP64
-// pipe, 1.6 operations per clock and SM, bounded the double form (NQ^2 / 2
-// products per element, 200 at p = 4). What is left there is four operations
-// per row: the conversion of the result, the increment, its square, the sum.
-// Every load of a tile is issued before the first product, so that a small
-// problem waits for memory twice (face ids, then all values).
+// the present form 5e-17, an FMA chain 8e-17.)
 //
 // The residual is reduced per tile (warp sums, then the warps in order) into
 // partials[tile]; the tile that takes the last ticket of the sweep adds the
